@@ -181,8 +181,11 @@ typedef struct qcd_gauge qcd_gauge;
 /* Load a gauge field (Sec. II A: links U_mu(x) in SU(3)).
  * U: canonical complex128 (4, V, 3, 3), device or host.  The library keeps
  * even-odd reordered copies in FP64 (18 reals), in FP32 and FP16 (geom->recon
- * reals) and in double-float (18 hi/lo FP32 pairs); the caller's buffer is not
- * referenced after the call returns.
+ * reals), in double-float (18 hi/lo FP32 pairs) and, where every link row and
+ * column has a 2-norm in [1/2, 5/4], in fixed point for both ends of each link
+ * (used by the FP64 operators; given back when device memory runs out, the FP64
+ * operators then use the FP64 copy); the caller's buffer is not referenced after
+ * the call returns.
  * Errors: QCD_ERR_ARG for a NULL pointer, odd or non-positive extents, bc not
  * +-1, recon not 12/18, or V >= 2^31; QCD_ERR_OOM if the copies do not fit. */
 qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd_gauge** out);

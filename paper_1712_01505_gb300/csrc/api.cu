@@ -90,10 +90,31 @@ void* Workspace::get(const std::string& name, size_t bytes) {
   if (getenv("QCD_FAULT") && strcmp(getenv("QCD_FAULT"), "alloc") == 0)
     raise(QCD_ERR_OOM, "workspace allocation of %zu bytes refused (QCD_FAULT=alloc)", bytes);
   void* p = nullptr;
-  QCD_CK(cudaMalloc(&p, bytes));
+  cudaError_t e = cudaMalloc(&p, bytes);
+  if (e == cudaErrorMemoryAllocation && drop_optional()) {
+    cudaGetLastError();
+    e = cudaMalloc(&p, bytes);
+  }
+  QCD_CK(e);
   bufs[name] = {p, bytes};
   ++generation;
   return p;
+}
+
+bool Workspace::drop_optional() {
+  bool any = false;
+  for (auto it = bufs.begin(); it != bufs.end();) {
+    if (it->first.compare(0, 4, "opt.") == 0) {
+      cudaFree(it->second.p);  // waits for the device
+      it = bufs.erase(it);
+      any = true;
+    } else {
+      ++it;
+    }
+  }
+  if (any) ++generation;
+  if (opt_in_use) *opt_in_use = false;
+  return any;
 }
 
 void Workspace::release() {
@@ -276,6 +297,7 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
     QCD_CK(cudaStreamCreateWithFlags(&g->work, cudaStreamNonBlocking));
     QCD_CK(cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming));
     QCD_CK(cudaEventCreateWithFlags(&g->ev_out, cudaEventDisableTiming));
+    QCD_CK(cudaEventCreateWithFlags(&g->fx_ev, cudaEventDisableTiming));
     size_t links = 4 * (size_t)lat.V;
     g->U64 = g->ws.get("gauge.U64", links * 18 * sizeof(double));
     g->U32 = g->ws.get("gauge.U32", links * lat.recon * sizeof(float));
@@ -285,7 +307,20 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
     Staged su = stage_in(g, "io.gauge", U, bytes, st, true);
     gauge_reorder(g, su.dev, st);
     links_to_df(g, st);
+    int fx_bad = 1;
+    int* fx_flag = (int*)g->ws.get("gauge.fx", sizeof(int));
+    g->ws.opt_in_use = &g->fx_ok;
+    try {  // optional: without it the FP64 stencil runs on U64
+      g->Ufx = g->ws.get("opt.Ufx", fx_link_bytes(lat));
+      links_to_fx(g, fx_flag, st);
+      QCD_CK(cudaMemcpyAsync(&fx_bad, fx_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+    } catch (const Error& e) {
+      if (e.status != QCD_ERR_OOM) throw;
+      cudaGetLastError();
+    }
     QCD_CK(cudaStreamSynchronize(st));
+    g->fx_ok = fx_bad == 0;
+    if (!g->fx_ok) g->ws.drop_optional();  // links that are not of unit size
   });
   if (s != QCD_OK) {
     if (g) {
@@ -296,6 +331,7 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
       if (g->work) cudaStreamDestroy(g->work);
       if (g->ev_in) cudaEventDestroy(g->ev_in);
       if (g->ev_out) cudaEventDestroy(g->ev_out);
+      if (g->fx_ev) cudaEventDestroy(g->fx_ev);
       delete g;
     }
     if (out) *out = nullptr;
@@ -315,6 +351,7 @@ qcd_status qcd_gauge_free(qcd_gauge* g) {
     cudaStreamDestroy(g->work);
     cudaEventDestroy(g->ev_in);
     cudaEventDestroy(g->ev_out);
+    cudaEventDestroy(g->fx_ev);
     delete g;
   });
 }

@@ -830,6 +830,7 @@ void dd_create(const qcd_dd_geom* geom, int nlocal, const int32_t* ids, const vo
       lg.recon = d->recon;
       const qcd_status stt = qcd_gauge_load(&lg, U[k], st, &s.g);
       if (stt != QCD_OK) raise(stt, "subdomain %d: %s", s.id, qcd_last_error());
+      s.g->ws.drop_optional();  // the subdomains' stencils run on the plain link copies
       d->subs.push_back(s);  // owned from here on (freed with the handle)
       Sub& sb = d->subs.back();
       sb.halo = sb.g->ws.get("dd.halo", halo_bytes(d, QCD_F64));

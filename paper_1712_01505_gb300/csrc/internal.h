@@ -99,7 +99,11 @@ struct Workspace {
   };
   std::map<std::string, Buf> bufs;
   long generation = 0;  // bumped whenever a buffer is (re)allocated or freed
+  // Buffers named "opt.*" speed things up but are not needed: when the device is out of memory they are
+  // given back (and *opt_in_use cleared) before an allocation fails.
+  bool* opt_in_use = nullptr;
   void* get(const std::string& name, size_t bytes);
+  bool drop_optional();
   void release();
 };
 
@@ -121,9 +125,13 @@ struct qcd_gauge {
   void* U32 = nullptr;  // FP32, lat.recon reals
   void* U16 = nullptr;  // FP16, lat.recon reals
   void* Udf = nullptr;  // double-float, 18 reals as hi/lo FP32 pairs
+  void* Ufx = nullptr;  // the FP64 links of the eight hops of every site in fixed point (fixed.cuh)
+  bool fx_ok = false;   // Ufx is there and every link has the size the fixed-point stencil takes
+  bool fx_used = false;             // the fixed-point scratch has been used, last on fx_stream
+  cudaStream_t fx_stream = nullptr;
   qcd::Workspace ws;
   cudaStream_t work = nullptr;  // private stream (capturable) for the solver
-  cudaEvent_t ev_in = nullptr, ev_out = nullptr;
+  cudaEvent_t ev_in = nullptr, ev_out = nullptr, fx_ev = nullptr;
   int device = 0;
 };
 
@@ -168,6 +176,18 @@ struct RedSpec {
 void hop(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int dagger, double a,
          const Field* x, cudaStream_t st, const int* stop = nullptr, bool allow_tuning = true,
          const RedSpec* red = nullptr);
+
+// ----------------------------------------------------------------------------- fixed point (wilson_fx.cu)
+// hop() on FP64 fields with the link products in fixed point; false (nothing done) where that path is not
+// available: links of other than unit size, a caller's stream capture, no memory for its scratch
+bool hop_fx(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int dagger, double a, const Field* x,
+            cudaStream_t st, const int* stop, const RedSpec* red);
+// the same for the Wilson Schur operator out = in - k2 H_eo H_oe in, the intermediate kept in fixed point
+bool mhat_fx(const qcd_gauge* g, const Field& in, Field& out, int dagger, double k2, cudaStream_t st, const int* stop,
+             const RedSpec* red);
+// Ufx from U64; *flag (device) becomes nonzero if a link's size is outside the fixed-point range
+size_t fx_link_bytes(const Lattice& lat);
+void links_to_fx(qcd_gauge* g, int* flag, cudaStream_t st);
 
 // ----------------------------------------------------------------------------- double float (wilson_df.cu)
 // out = [x1 + c2 x2 +] a * H_{p,1-p} in on double-float fields (x2 only with x1)

@@ -20,8 +20,9 @@ void apply_mhat(const OpCtx& c, const Field& in, Field& out, int dagger, cudaStr
                 const char* tag, const int* stop, const RedSpec* red) {
   std::string t = tag;
   if (c.f.type == QCD_WILSON) {
-    Field tmp = ws_field(c.g, t + ".mhat.t", c.prec, in.ls, in.nrhs);
     const double k2 = c.f.kappa * c.f.kappa;
+    if (c.prec == QCD_F64 && mhat_fx(c.g, in, out, dagger, k2, st, stop, red)) return;
+    Field tmp = ws_field(c.g, t + ".mhat.t", c.prec, in.ls, in.nrhs);
     hop(c.g, in, tmp, 1, dagger, 1.0, nullptr, st, stop);
     hop(c.g, tmp, out, 0, dagger, -k2, &in, st, stop, true, red);
     return;

@@ -1,0 +1,707 @@
+// The FP64 Wilson hopping stencil with its link products in fixed point
+// (fixed.cuh): the same operation and storage as the FP64 kernels of wilson.cu,
+//
+//   out(x) = [x(x) +] a * sum_mu [ (1 - gamma_mu) U_mu(x) in(x+mu)
+//                                + (1 + gamma_mu) U_mu(x-mu)^dag in(x-mu) ]
+//
+// The input is first rewritten as fixed-point parts with one exponent per site (k_to_fx), the links
+// are kept that way from the loading of the gauge field, and only the final sum goes through the
+// FP64 pipe: 24 conversions and 24 multiply-adds per site instead of 864.  Measured at 32^3 x 64:
+// FP64 kernel 1.57 ms (FP64 pipe), here 0.315 ms, 5.8 TB/s = 85% of the copy rate (HBM: links 1152 B, input
+// 196 B, x and output 192 B each per site), and 0.063 ms for k_to_fx (HBM); 16^3 x 32 x 16 slices
+// 1.56 -> 0.28 + 0.07 ms (issue slots).  Forms that were slower: the conversion inside the stencil (8 times per
+// site: 0.555 ms), three integer products per real one instead of one and two FP32 ones (0.355 ms, the
+// integer multiply pipe), one thread per site (0.333 ms at 168 registers, 12 warps per SM).
+#include <cstdio>
+#include <vector>
+
+#include "common.cuh"
+#include "fixed.cuh"
+#include "internal.h"
+#include "stencil.cuh"
+
+namespace qcd {
+
+namespace {
+
+using namespace stencil;
+using namespace fx;
+
+using HA = HopArgs<P64, 18>;
+
+// Layouts.  Links: the matrices of all eight hops of a site, W[2 mu] = U_mu(x) and
+// W[2 mu + 1] = U_mu(x - mu)^dag, as [parity][block of 32 sites][hop][element][32] (each link is stored
+// for both of its ends: a half-dslash reads as many bytes as from one copy, contiguously and with
+// no transposition).  Spinors: [slice][block of 32 sites][component][32] and one exponent field per
+// site.  A unit is int4 (re.h, re.l, im.h, im.l).  A site of exponent field kBad holds its FP64 values.
+constexpr int kSB = 16;  // sites per block of the layouts
+constexpr int kHopUnits = 9 * kSB, kSiteUnits = 12 * kSB;
+
+struct FxField {
+  int4* __restrict__ p;
+  int* __restrict__ e;
+  long nsb;  // blocks of kSB sites per slice
+};
+
+// FP64 -> fixed point: one thread per site, blockIdx.y: (right-hand side, slice)
+__global__ void __launch_bounds__(128) k_to_fx(const int4* __restrict__ in, long stride, FxField out, int Vh, int ls,
+                                               const int* stop) {
+  pdl_enter();
+  if (stop && *stop) return;
+  const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cb >= Vh) return;
+  const int s = blockIdx.y % ls, r = blockIdx.y / ls;
+  in += (long)r * 12 * stride + (long)s * Vh + cb;
+  int4 w[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) w[k] = __ldg(in + k * stride);
+  unsigned mx = 0;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) mx = max(mx, max((unsigned)w[k].y & 0x7fffffffu, (unsigned)w[k].w & 0x7fffffffu));
+  int e = (int)(mx >> 20);
+  if (mx == 0) {  // all zero, or subnormals below 2^-1042
+    unsigned low = 0;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) low |= (unsigned)(w[k].x | w[k].z);
+    e = low ? 0 : kEmin;
+  }
+  const long blk = (long)blockIdx.y * out.nsb + cb / kSB;
+  int4* o = out.p + blk * kSiteUnits + cb % kSB;
+  if (e < kEmin || e > kEmax) {
+    e = kBad;
+#pragma unroll
+    for (int k = 0; k < 12; ++k) o[k * kSB] = w[k];
+  } else {
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const Part re = spinor_part(w[k].y, w[k].x, e), im = spinor_part(w[k].w, w[k].z, e);
+      o[k * kSB] = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
+    }
+  }
+  out.e[blk * kSB + cb % kSB] = e;
+}
+
+// A warp owns 16 sites, lane = 16 sp + site: the lane computes the link products of spin sp of the half
+// spinors (three colours instead of six: half the registers per thread, twice the warps), sums the upper spin
+// sp and, of the lower spins, the one that spin sp of the half spinor feeds: 1 - sp in the x and y hops, sp in the z and
+// t hops, so the sums of the lower spins change lanes once, between them.
+//
+// Shared memory of a block: the links of a warp's sites, one hop per buffer, brought by bulk copies
+// (a hop's 9 elements x 16 sites are 2304 contiguous bytes) kBuf hops ahead; and each
+// site's eight neighbour indices (the sign bit: the hop carries the antiperiodic factor).
+constexpr int kWarps = 4;  // warps per block
+constexpr int kBuf = 2;
+struct FxShared {
+  int4 w[kWarps][kBuf][kHopUnits];
+  int nb[8][kWarps * kSB];
+  unsigned long long bar[kWarps][kBuf];
+};
+
+struct FxWarp {
+  FxShared* sm;
+  const int4* links;  // of this warp's sites
+  int warp, lane;
+  bool failed;
+  __device__ __forceinline__ void issue(int hop, int buf) {
+    if (lane == 0) {
+      unsigned long long* bar = &sm->bar[warp][buf];
+      fence_proxy_async();  // the lanes' reads of the buffer (ordered by the last __syncwarp) before the copy
+      mbar_expect_tx(bar, kHopUnits * 16u);
+      bulk_g2s(&sm->w[warp][buf][0], links + hop * kHopUnits, kHopUnits * 16u, bar);
+    }
+  }
+};
+
+// the order of the hops: y, x, z, t (forward, backward)
+__device__ __forceinline__ constexpr int fx_order(int i) { return i < 2 ? 2 + i : (i < 4 ? i - 2 : i); }
+
+// barriers and the first copies (the links are constant: before the predecessor kernel is waited for)
+__device__ __forceinline__ FxWarp fx_begin(FxShared& sm, const int4* links, long block) {
+  FxWarp W{&sm, links + block * (8 * kHopUnits), (int)(threadIdx.x >> 5), (int)(threadIdx.x & 31), false};
+  if (W.lane < kBuf) mbar_init(&sm.bar[W.warp][W.lane], 1);
+  if (W.lane < kBuf) mbar_init_fence();
+  __syncwarp();
+#pragma unroll
+  for (int b = 0; b < kBuf; ++b) W.issue(fx_order(b), b);
+  return W;
+}
+__device__ __forceinline__ void fx_abandon(FxWarp& W) {  // wait for the copies in flight
+#pragma unroll
+  for (int b = 0; b < kBuf; ++b) mbar_wait(&W.sm->bar[W.warp][b], 0u);
+}
+
+// Hop number I (of fx_order) added to up (upper spin sp) and lo (a lower spin; up to the sign that the caller
+// applies).  m: the sign of the lower input spin.  Packed FP32 lanes: (re, im).
+template <int I>
+__device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int sp, int m, int64_t (&up)[6],
+                                       int64_t (&lo)[6]) {
+  constexpr int HOP = fx_order(I), MU = HOP >> 1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
+  const int nbw = W.sm->nb[HOP][W.warp * kSB + W.lane % kSB], ncb = nbw & 0x7fffffff;
+  const int4* q = f.p + (long)(ncb / kSB) * kSiteUnits + ncb % kSB;
+  const int4* qu = q + sp * (3 * kSB);
+  const int4* ql = q + 6 * kSB + (MU < 2 ? 1 - sp : sp) * (3 * kSB);  // the lower spin that meets upper spin sp
+  const int d3 = min(E - __ldg(f.e + ncb), 100) + 3;
+  m *= SG;
+  const float mf = (float)m;
+  int hr[3], hi[3];
+  float2 y[3];  // the FP32 parts
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    const int4 a = __ldg(qu + c * kSB), b = __ldg(ql + c * kSB);
+    const float ar = __int_as_float(a.y), ai = __int_as_float(a.w);
+    const float br = __int_as_float(b.y), bi = __int_as_float(b.w);
+    if (MU == 0 || MU == 2) {  // -+ i l
+      hr[c] = a.x + m * b.z;
+      hi[c] = a.z - m * b.x;
+      y[c] = make_float2(fmaf(mf, bi, ar), fmaf(-mf, br, ai));
+    } else {
+      hr[c] = a.x + m * b.x;
+      hi[c] = a.z + m * b.z;
+      y[c] = make_float2(fmaf(mf, br, ar), fmaf(mf, bi, ai));
+    }
+  }
+  if (nbw < 0) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      hr[c] = -hr[c];
+      hi[c] = -hi[c];
+      y[c] = make_float2(-y[c].x, -y[c].y);
+    }
+  }
+  int hn[3];
+  float2 g[3], ys[3], gs[3];  // the integer parts as FP32; both with the lanes exchanged
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    g[c] = make_float2((float)hr[c], (float)hi[c]);
+    ys[c] = swp(y[c]);
+    gs[c] = swp(g[c]);
+    hn[c] = -hi[c];
+  }
+  const float sc = __int_as_float((127 - d3) << 23);
+  if (!mbar_wait(&W.sm->bar[W.warp][I % kBuf], (unsigned)(I / kBuf) & 1u)) W.failed = true;
+  const int4* w = &W.sm->w[W.warp][I % kBuf][W.lane % kSB];
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int64_t Hr = 0, Hi = 0;
+    float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 u = w[(a * 3 + b) * kSB];
+      Hr += (int64_t)u.x * hr[b];
+      Hr += (int64_t)u.z * hn[b];
+      Hi += (int64_t)u.x * hi[b];
+      Hi += (int64_t)u.z * hr[b];
+      C = fma2(bc2((float)u.x), y[b], C);
+      C = fma2(bc2(__int_as_float(u.y)), g[b], C);
+      D = fma2(bc2((float)u.z), ys[b], D);
+      D = fma2(bc2(__int_as_float(u.w)), gs[b], D);
+    }
+    const int64_t wr = (Hr >> d3) + (int64_t)__float2int_rn((C.x - D.x) * sc);
+    const int64_t wi = (Hi >> d3) + (int64_t)__float2int_rn((C.y + D.y) * sc);
+    up[2 * a] += wr;
+    up[2 * a + 1] += wi;
+    if (MU == 0 || MU == 2) {  // SG i w
+      lo[2 * a] -= SG * wi;
+      lo[2 * a + 1] += SG * wr;
+    } else {
+      lo[2 * a] += SG * wr;
+      lo[2 * a + 1] += SG * wi;
+    }
+  }
+  __syncwarp();  // every lane has read the buffer
+  if (I + kBuf < 8) W.issue(fx_order(I + kBuf < 8 ? I + kBuf : 0), I % kBuf);
+}
+
+// The hop sum of one site in FP64 from the fixed-point field (neighbours whose values are kept in
+// FP64), added to acc.
+__device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int cb, Cx<double>* out) {
+  const SiteCoords c = cb_to_site(A.g, cb, A.out_parity);
+  const double sg = A.dagger ? 1.0 : -1.0;
+  Cx<double> acc[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
+  auto hop = [&](auto mu, bool back) {
+    constexpr int MU = decltype(mu)::value;
+    int wrap;
+    const int n = neighbour_index(A.g, c, MU, back ? -1 : +1, &wrap) >> 1;
+    const double sf = (wrap && A.g.apbc[MU]) ? -1.0 : 1.0, sgn = back ? -sg : sg;
+    const int e = f.e[n];
+    Cx<double> U[9], psi[12], h[6], gg[6];
+    A.U.load(back ? 1 - A.out_parity : A.out_parity, MU, back ? n : cb, U);
+    for (int k = 0; k < 12; ++k) {
+      const int4 u = f.p[(long)(n / kSB) * kSiteUnits + k * kSB + n % kSB];
+      if (e == kBad)
+        psi[k] = {__hiloint2double(u.y, u.x), __hiloint2double(u.w, u.z)};
+      else
+        psi[k] = {part_value({u.x, __int_as_float(u.y)}, e), part_value({u.z, __int_as_float(u.w)}, e)};
+    }
+    project<MU>(psi, sgn, h);
+    if (back)
+      link_mul<true>(U, h, gg);
+    else
+      link_mul<false>(U, h, gg);
+    reconstruct_add<MU>(gg, sgn, sf, acc);
+  };
+  for (int back = 0; back < 2; ++back) {
+    hop(std::integral_constant<int, 0>{}, back);
+    hop(std::integral_constant<int, 1>{}, back);
+    hop(std::integral_constant<int, 2>{}, back);
+    hop(std::integral_constant<int, 3>{}, back);
+  }
+  for (int k = 0; k < 12; ++k) out[k] = acc[k];
+}
+
+// [x +] a H in of one site in FP64, stored
+__device__ __noinline__ void fp64_site_store(const HA& A, const FxField& f, int cb, int r, long site) {
+  Cx<double> acc[12], o[12];
+  fp64_site(A, f, cb, acc);
+  if (A.xpay) {
+    A.x.offset_rhs(r).load(site, o);
+    for (int k = 0; k < 12; ++k) o[k] = fmac(A.a, acc[k], o[k]);
+  } else {
+    for (int k = 0; k < 12; ++k) o[k] = A.a * acc[k];
+  }
+  A.out.offset_rhs(r).store(site, o);
+}
+
+// H in of one site in FP64, stored in the fixed-point field o as a kBad site
+__device__ __noinline__ void fp64_site_store_fx(const HA& A, const FxField& f, const FxField& o, int cb) {
+  Cx<double> acc[12];
+  fp64_site(A, f, cb, acc);
+  int4* p = o.p + (long)(cb / kSB) * kSiteUnits + cb % kSB;
+  for (int k = 0; k < 12; ++k)
+    p[k * kSB] = make_int4(__double2loint(acc[k].re), __double2hiint(acc[k].re), __double2loint(acc[k].im),
+                           __double2hiint(acc[k].im));
+  o.e[cb] = kBad;
+}
+
+// The exponent field of the site's largest neighbour (its neighbour indices go to shared memory).
+__device__ __forceinline__ int fx_neighbours(const HA& A, FxWarp& W, const FxField& f, int cb) {
+  const SiteCoords c = cb_to_site(A.g, cb, A.out_parity);
+  int E = kEmin;
+  const bool back = W.lane >= kSB;  // the site's other lane does the forward hops
+#pragma unroll
+  for (int mu = 0; mu < 4; ++mu) {
+    int wrap;
+    const int n = neighbour_index(A.g, c, mu, back ? -1 : +1, &wrap) >> 1;
+    W.sm->nb[2 * mu + back][W.warp * kSB + W.lane % kSB] = n | ((wrap && A.g.apbc[mu]) ? 0x80000000 : 0);
+    E = max(E, __ldg(f.e + n));
+  }
+  E = max(E, __shfl_xor_sync(0xffffffffu, E, kSB));
+  __syncwarp();
+  return E;
+}
+
+__device__ __forceinline__ void flip(int64_t (&v)[6], bool minus) {
+  const int64_t n = minus ? -1 : 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v[k] = (v[k] ^ n) - n;
+}
+
+// up, lo = the sum of the eight hops for spins sp and 2 + sp, in units of the returned value
+// (lo: times -1 for H^dag = g5 H g5); the whole warp calls it
+__device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, int64_t (&up)[6],
+                                         int64_t (&lo)[6]) {
+  const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) up[k] = lo[k] = 0;
+  fx_hop<0>(W, f, E, sp, -gs, up, lo);  // y: B = (-l1, l0)
+  fx_hop<1>(W, f, E, sp, -gs, up, lo);
+  flip(lo, sp == 0);                    // B^dag = (g1, -g0)
+  fx_hop<2>(W, f, E, sp, g5, up, lo);   // x: B = -i (l1, l0)
+  fx_hop<3>(W, f, E, sp, g5, up, lo);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) lo[k] = __shfl_xor_sync(0xffffffffu, lo[k], kSB);
+  flip(lo, sp != 0);
+  fx_hop<4>(W, f, E, sp, gs, up, lo);   // z: B = (-i l0, i l1)
+  fx_hop<5>(W, f, E, sp, gs, up, lo);
+  flip(lo, sp != 0);
+  fx_hop<6>(W, f, E, sp, g5, up, lo);   // t: B = 1
+  fx_hop<7>(W, f, E, sp, g5, up, lo);
+  if (W.failed) return __longlong_as_double(0x7ff8000000000000ll);  // a copy that never arrived: NaN output
+  return __hiloint2double((E - 56) << 20, 0);  // 2^(E - 1079)
+}
+
+// The sums as a fixed-point field of their own (a = 1, no x term: the first half-dslash of Mhat, whose
+// result only the second one reads): both lanes of a site find its largest sum.
+__device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, bool valid, int E, bool minus_lo, bool nan,
+                                         int64_t (&up)[6], int64_t (&lo)[6]) {
+  flip(lo, minus_lo);
+  uint64_t mx = 0;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    mx |= (uint64_t)(up[k] ^ (up[k] >> 63));
+    mx |= (uint64_t)(lo[k] ^ (lo[k] >> 63));
+  }
+  mx |= __shfl_xor_sync(0xffffffffu, mx, kSB);
+  if (!valid || E == kBad) return;  // kBad: fp64_site_store_fx
+  const int b = 64 - __clzll((long long)mx);  // -2^b <= every sum < 2^b
+  const int e = mx ? b + E - 57 : kEmin, shift = b - 30;
+  int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
+  const bool wide = nan || e < kEmin || e > kEmax;
+  const double unit = nan ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double((E - 56) << 20, 0);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int c = k % 3;
+    const int64_t re = k < 3 ? up[2 * c] : lo[2 * c], im = k < 3 ? up[2 * c + 1] : lo[2 * c + 1];
+    int4 w;
+    if (wide) {
+      const double x = (double)re * unit, y = (double)im * unit;
+      w = make_int4(__double2loint(x), __double2hiint(x), __double2loint(y), __double2hiint(y));
+    } else {
+      const Part pr = sum_part(re, shift), pi = sum_part(im, shift);
+      w = make_int4(pr.h, __float_as_int(pr.l), pi.h, __float_as_int(pi.l));
+    }
+    o[(k < 3 ? c : 6 + c) * kSB] = w;
+  }
+  if (sp == 0) out.e[cb] = wide ? kBad : e;
+}
+
+// OUT = 0: [x +] a H in as FP64; OUT = 1: H in as the fixed-point field O
+template <int MINB, int OUT>
+__global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_constant__ HA A,
+                                                              const int4* __restrict__ links,
+                                                              const __grid_constant__ FxField F,
+                                                              const __grid_constant__ FxField O) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
+  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
+  const int q = blockIdx.x - sblock * A.ntiles;
+  const int cb0 = (sblock * kWarps + (threadIdx.x >> 5)) * kSB;  // the warp's first site
+  if (cb0 >= A.g.Vh) return;                                   // a whole warp
+  const int cb = cb0 + threadIdx.x % kSB, sp = (threadIdx.x & 31) / kSB;
+  const bool valid = cb < A.g.Vh;
+  FxWarp W = fx_begin(sm, links, (long)A.out_parity * F.nsb + cb0 / kSB);
+  pdl_enter();
+  if (A.stop && *A.stop) {
+    fx_abandon(W);
+    return;
+  }
+  const int r = fdiv(q, A.d_ls), s = q - r * A.ls;
+  const long site = (long)s * A.g.Vh + cb;
+  const FxField f{F.p + (long)q * F.nsb * kSiteUnits, F.e + (long)q * F.nsb * kSB, F.nsb};
+  const int E = fx_neighbours(A, W, f, valid ? cb : 0);
+  int64_t up[6], lo[6];
+  const double unit = fx_sum(A, W, f, E, sp, up, lo);
+  if constexpr (OUT == 1) {
+    const FxField o{O.p + (long)q * O.nsb * kSiteUnits, O.e + (long)q * O.nsb * kSB, O.nsb};
+    fx_store(o, cb, sp, valid, E, A.dagger != 0, W.failed, up, lo);
+    if (E == kBad && valid && sp == 0) fp64_site_store_fx(A, f, o, cb);
+    return;
+  }
+  if (!valid) return;
+  if (E == kBad) {
+    if (sp == 0) fp64_site_store(A, f, cb, r, site);
+    return;
+  }
+  const double au = A.a * unit, al = A.dagger ? -au : au;
+  const long xstr = A.x.stride, ostr = A.out.stride;
+  const double2* x = A.x.offset_rhs(r).p + 3 * sp * xstr + site;
+  double2* o = A.out.offset_rhs(r).p + 3 * sp * ostr + site;
+  if (A.xpay) {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      const double2 xu = __ldg(x + c * xstr), xl = __ldg(x + (6 + c) * xstr);
+      o[c * ostr] = make_double2(fma(au, (double)up[2 * c], xu.x), fma(au, (double)up[2 * c + 1], xu.y));
+      o[(6 + c) * ostr] = make_double2(fma(al, (double)lo[2 * c], xl.x), fma(al, (double)lo[2 * c + 1], xl.y));
+    }
+  } else {
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      o[c * ostr] = make_double2(au * (double)up[2 * c], au * (double)up[2 * c + 1]);
+      o[(6 + c) * ostr] = make_double2(al * (double)lo[2 * c], al * (double)lo[2 * c + 1]);
+    }
+  }
+}
+
+// one right-hand side, the BiCGStab inner products of k_hop_red (wilson.cu) in the epilogue
+template <int MINB, int RED>
+__global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx_red(const __grid_constant__ HA A,
+                                                                  const int4* __restrict__ links,
+                                                                  const __grid_constant__ FxField F) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
+  const int cb0 = (blockIdx.x * kWarps + (threadIdx.x >> 5)) * kSB;
+  const int cb = cb0 + threadIdx.x % kSB, sp = (threadIdx.x & 31) / kSB;
+  const bool valid = cb < A.g.Vh, warp_valid = cb0 < A.g.Vh;
+  FxWarp W;
+  if (warp_valid) W = fx_begin(sm, links, (long)A.out_parity * F.nsb + cb0 / kSB);
+  pdl_enter();
+  if (A.stop && *A.stop) {
+    if (warp_valid) fx_abandon(W);
+    return;
+  }
+  double red[3] = {0.0, 0.0, 0.0};
+  if (warp_valid) {
+    const int E = fx_neighbours(A, W, F, valid ? cb : 0);
+    const bool bad = E == kBad;
+    if (bad && valid && sp == 0) fp64_site_store(A, F, cb, 0, cb);
+    __syncwarp();
+    int64_t up[6], lo[6];
+    const double unit = fx_sum(A, W, F, E, sp, up, lo);
+    const double au = A.a * unit, al = A.dagger ? -au : au;
+    if (valid) {
+      const double2* x = A.x.p + 3 * sp * A.x.stride + cb;
+      const double2* rt = A.rt.p + 3 * sp * A.rt.stride + cb;
+      double2* out = A.out.p + 3 * sp * A.out.stride + cb;
+      Cx<double> d = {0.0, 0.0};
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {  // colour k of spin sp, colour k - 3 of spin 2 + sp
+        const int c = k % 3, n = k < 3 ? c : 6 + c;
+        const double a = k < 3 ? au : al;
+        const double vr = (double)(k < 3 ? up[2 * c] : lo[2 * c]), vi = (double)(k < 3 ? up[2 * c + 1] : lo[2 * c + 1]);
+        const double2 xs = __ldg(x + n * A.x.stride);
+        Cx<double> o = {fma(a, vr, xs.x), fma(a, vi, xs.y)};
+        if (bad) {  // as stored above
+          const volatile double2* w = out + n * A.out.stride;
+          o = {w->x, w->y};
+        } else {
+          out[n * A.out.stride] = make_double2(o.re, o.im);
+        }
+        if (RED == 1) {  // (rt, out)
+          const double2 w = __ldg(rt + n * A.rt.stride);
+          d = cjmadd(Cx<double>{w.x, w.y}, o, d);
+        } else {  // (out, x), |out|^2
+          d = cjmadd(o, Cx<double>{xs.x, xs.y}, d);
+          red[2] = fma(o.re, o.re, fma(o.im, o.im, red[2]));
+        }
+      }
+      red[0] = d.re;
+      red[1] = d.im;
+    }
+  }
+  red_epilogue<double>(A, red);
+}
+
+// ----------------------------------------------------------------------------- links
+// The links of the eight hops as parts, and whether every link has the size the fixed point takes:
+// *flag becomes nonzero if a row or column 2-norm lies outside [kNormMin, kNormMax] (or is NaN).
+// One thread per (parity, mu, site): both ends of its link.
+__global__ void __launch_bounds__(128) k_links_fx(Geom g, const double2* __restrict__ U64, int4* __restrict__ W, long nsb,
+                                                  int* flag) {
+  const long i = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  const long Vh = g.Vh;
+  if (i >= 8 * Vh) return;
+  const int pm = (int)(i / Vh), cb = (int)(i % Vh), par = pm >> 2, mu = pm & 3;
+  const double2* u64 = U64 + (long)pm * 9 * Vh + cb;
+  const SiteCoords c = cb_to_site(g, cb, par);
+  int wrap, j = 0;
+#pragma unroll
+  for (int m = 0; m < 4; ++m)
+    if (m == mu) j = neighbour_index(g, c, m, +1, &wrap) >> 1;
+  int4* wf = W + (((long)par * nsb + cb / kSB) * 8 + 2 * mu) * kHopUnits + cb % kSB;
+  int4* wb = W + (((long)(1 - par) * nsb + j / kSB) * 8 + 2 * mu + 1) * kHopUnits + j % kSB;
+  float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+#pragma unroll
+  for (int k = 0; k < 9; ++k) {
+    const double2 u = u64[k * Vh];
+    const float x = (float)u.x, y = (float)u.y, n = fmaf(x, x, y * y);
+    row[k / 3] += n;
+    col[k % 3] += n;
+    const Part re = link_part(u.x), im = link_part(u.y);
+    wf[k * kSB] = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
+    wb[((k % 3) * 3 + k / 3) * kSB] = make_int4(re.h, __float_as_int(re.l), -im.h, __float_as_int(-im.l));
+  }
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) {
+    constexpr float lo = (float)(kNormMin * kNormMin), hi = (float)(kNormMax * kNormMax);
+    ok = ok && row[k] >= lo && row[k] <= hi && col[k] >= lo && col[k] <= hi;
+  }
+  if (!ok) *flag = 1;
+}
+
+struct FxLaunch {
+  HA args;
+  const int4* links;
+  FxField F, O;
+  bool fx_out;
+  cudaStream_t st;
+};
+
+template <int MINB>
+void launch_fx(FxLaunch* L) {
+  const HA& A = L->args;
+  constexpr int block = 32 * kWarps;
+  constexpr size_t smem = sizeof(FxShared);
+  const unsigned sblocks = (unsigned)((A.g.Vh + kWarps * kSB - 1) / (kWarps * kSB));
+  if (A.red == 1)
+    launch_k(k_hop_fx_red<MINB, 1>, sblocks, block, smem, L->st, A, L->links, L->F);
+  else if (A.red == 2)
+    launch_k(k_hop_fx_red<MINB, 2>, sblocks, block, smem, L->st, A, L->links, L->F);
+  else if (L->fx_out)
+    launch_k(k_hop_fx<MINB, 1>, sblocks * (unsigned)A.ntiles, block, smem, L->st, A, L->links, L->F, L->O);
+  else
+    launch_k(k_hop_fx<MINB, 0>, sblocks * (unsigned)A.ntiles, block, smem, L->st, A, L->links, L->F, L->O);
+}
+
+// cfg.tile: blocks per SM that the registers are bounded for (5: 96 registers, 20 warps; 4: 128, 16 warps;
+// within 2% of each other where HBM bounds them, 4 is 10% faster on a few hundred sites.  6 and 7 spill: 0.345
+// and 0.376 ms against 0.315 at 32^3 x 64)
+void run_fx(void* ctx, const LaunchCfg& cfg) {
+  auto* L = (FxLaunch*)ctx;
+  if (cfg.tile == 4)
+    launch_fx<4>(L);
+  else
+    launch_fx<5>(L);
+}
+
+SpinorView<P64> fx_view(const Field& f) {
+  SpinorView<P64> v;
+  v.p = (double2*)f.data;
+  v.norm = nullptr;
+  v.stride = f.nsites();
+  return v;
+}
+
+// A scratch field of the handle.
+FxField fx_scratch(qcd_gauge* g, const char* name, const Field& like) {
+  const long nsb = (like.Vh + kSB - 1) / kSB, nq = (long)like.ls * like.nrhs;
+  const size_t data = (size_t)nq * nsb * kSiteUnits * sizeof(int4), exps = (size_t)nq * nsb * kSB * sizeof(int);
+  char* p = (char*)g->ws.get(name, data + exps);
+  return {(int4*)p, (int*)(p + data), nsb};
+}
+
+void fx_pack(const Field& in, const FxField& out, cudaStream_t st, const int* stop) {
+  launch_k(k_to_fx, dim3((unsigned)((in.Vh + 127) / 128), (unsigned)(in.ls * in.nrhs)), 128, 0, st,
+           (const int4*)in.data, in.nsites(), out, (int)in.Vh, in.ls, stop);
+  QCD_LAUNCH_CK();
+}
+
+// out = [x +] a H in (out FP64), or the fixed-point field fout = H in (a = 1, x null)
+void fx_launch(const qcd_gauge* gh, const FxField& in, const Field& shape, Field* out, const FxField* fout,
+               int out_parity, int dagger, double a, const Field* x, cudaStream_t st, const int* stop,
+               const RedSpec* red) {
+  FxLaunch L;
+  HA& A = L.args;
+  A.red = 0;
+  A.partial = A.gpartial = nullptr;
+  A.counters = A.npartial = nullptr;
+  if (red && red->mode) {
+    if (!x || (red->mode == 1 && !red->rt) || shape.nrhs * shape.ls > 1)
+      raise(QCD_ERR_ARG, "fused reductions in FP64 need one slice and an x term");
+    A.red = red->mode;
+    A.partial = red->partial;
+    A.gpartial = red->gpartial;
+    A.counters = red->counters;
+    A.npartial = red->npartial;
+  }
+  A.g = make_geom(gh->lat.L, gh->lat.bc, gh->lat.V, gh->lat.Vh);
+  A.out_parity = out_parity;
+  A.ls = shape.ls;
+  A.d_ls = make_fastdiv((unsigned)shape.ls);
+  A.nslices = A.ntiles = shape.ls * shape.nrhs;
+  A.d_ntiles = make_fastdiv((unsigned)A.ntiles);
+  A.dagger = dagger;
+  A.xpay = x != nullptr;
+  A.a = a;
+  A.U.p = (const double2*)gh->U64;
+  A.U.Vh = gh->lat.Vh;
+  A.out = out ? fx_view(*out) : fx_view(shape);
+  A.in = A.out;  // not read: the input is L.F
+  A.x = x ? fx_view(*x) : A.out;
+  A.rt = red && red->rt ? fx_view(*red->rt) : A.out;
+  A.stop = stop;
+  L.links = (const int4*)gh->Ufx;
+  L.F = in;
+  L.O = fout ? *fout : in;
+  L.fx_out = fout != nullptr;
+  L.st = st;
+  static std::atomic<unsigned long long> attr_mask{0};
+  if (first_use_on_device(attr_mask))
+    for (const void* k : {(const void*)k_hop_fx<4, 0>, (const void*)k_hop_fx<4, 1>, (const void*)k_hop_fx<5, 0>,
+                          (const void*)k_hop_fx<5, 1>, (const void*)k_hop_fx_red<4, 1>, (const void*)k_hop_fx_red<4, 2>,
+                          (const void*)k_hop_fx_red<5, 1>, (const void*)k_hop_fx_red<5, 2>})
+      QCD_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared)));
+  const std::vector<LaunchCfg> cands = {{32 * kWarps, 5}, {32 * kWarps, 4}};
+  char key[160];
+  snprintf(key, sizeof key, "hopfx L%dx%dx%dx%d ns%d xp%d red%d out%d", gh->lat.L[0], gh->lat.L[1], gh->lat.L[2],
+           gh->lat.L[3], A.nslices, A.xpay, A.red, (int)L.fx_out);
+  LaunchCfg cfg = tune(key, cands, &run_fx, &L, st, true, stop);
+  run_fx(&L, cfg);
+  QCD_LAUNCH_CK();
+}
+
+// The scratch fields belong to the handle, and calls on device buffers are asynchronous on the caller's
+// stream: work on another stream than the last user's waits for that user's event.  (The solver's own
+// stream is recorded only when another stream follows it: the handle owns it.)
+struct FxOrder {
+  qcd_gauge* g;
+  cudaStream_t st;
+  FxOrder(qcd_gauge* g_, cudaStream_t st_) : g(g_), st(st_) {
+    if (!g->fx_used || g->fx_stream == st) return;
+    if (g->fx_stream == g->work) QCD_CK(cudaEventRecord(g->fx_ev, g->work));
+    QCD_CK(cudaStreamWaitEvent(st, g->fx_ev, 0));
+  }
+  void done() {
+    g->fx_used = true;
+    g->fx_stream = st;
+    if (st != g->work) QCD_CK(cudaEventRecord(g->fx_ev, st));
+  }
+};
+
+// Whether the fixed-point path may run on `st`: never under a caller's stream capture (a graph that
+// outlives the call must not hold the handle's scratch).
+bool fx_usable(const qcd_gauge* g, cudaStream_t st) {
+  if (!g->fx_ok) return false;
+  if (st == g->work) return true;
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  QCD_CK(cudaStreamIsCapturing(st, &cs));
+  return cs == cudaStreamCaptureStatusNone;
+}
+
+}  // namespace
+
+size_t fx_link_bytes(const Lattice& lat) { return (size_t)2 * ((lat.Vh + kSB - 1) / kSB) * 8 * kHopUnits * sizeof(int4); }
+
+void links_to_fx(qcd_gauge* g, int* flag, cudaStream_t st) {
+  const long n = 8 * g->lat.Vh;
+  QCD_CK(cudaMemsetAsync(flag, 0, sizeof(int), st));
+  k_links_fx<<<(unsigned)((n + 127) / 128), 128, 0, st>>>(make_geom(g->lat.L, g->lat.bc, g->lat.V, g->lat.Vh),
+                                                         (const double2*)g->U64, (int4*)g->Ufx, (g->lat.Vh + kSB - 1) / kSB, flag);
+  QCD_LAUNCH_CK();
+}
+
+bool hop_fx(const qcd_gauge* gh, const Field& in, Field& out, int out_parity, int dagger, double a, const Field* x,
+            cudaStream_t st, const int* stop, const RedSpec* red) {
+  if (!fx_usable(gh, st)) return false;
+  qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  FxField f;
+  try {
+    f = fx_scratch(g, "opt.fx.a", in);
+  } catch (const Error& e) {
+    if (e.status != QCD_ERR_OOM) throw;
+    return false;
+  }
+  if (!g->fx_ok) return false;  // the links gave way to another allocation
+  FxOrder order(g, st);
+  fx_pack(in, f, st, stop);
+  fx_launch(g, f, in, &out, nullptr, out_parity, dagger, a, x, st, stop, red);
+  order.done();
+  return true;
+}
+
+bool mhat_fx(const qcd_gauge* gh, const Field& in, Field& out, int dagger, double k2, cudaStream_t st, const int* stop,
+             const RedSpec* red) {
+  if (!fx_usable(gh, st)) return false;
+  qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  FxField f, t;
+  try {
+    fx_scratch(g, "opt.fx.a", in);
+    t = fx_scratch(g, "opt.fx.b", in);
+    if (g->fx_ok) f = fx_scratch(g, "opt.fx.a", in);
+  } catch (const Error& e) {
+    if (e.status != QCD_ERR_OOM) throw;
+    return false;
+  }
+  if (!g->fx_ok) return false;
+  FxOrder order(g, st);
+  fx_pack(in, f, st, stop);
+  fx_launch(g, f, in, nullptr, &t, 1, dagger, 1.0, nullptr, st, stop, nullptr);
+  fx_launch(g, t, in, &out, nullptr, 0, dagger, -k2, &in, st, stop, red);
+  order.done();
+  return true;
+}
+
+}  // namespace qcd
