@@ -180,6 +180,36 @@ void blas_axpby(double a, const Field& x, double b, Field& y, cudaStream_t st) {
   QCD_LAUNCH_CK();
 }
 
+namespace {
+// out[r * stride] = the sum of right-hand side r's nb partials, in a fixed order
+__global__ void k_norm2_fold(const double* partial, int nb, double* out, int stride) {
+  double v[1] = {0.0};
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) v[0] += partial[(long)blockIdx.x * nb + b];
+  block_sum<1>(v);
+  if (threadIdx.x == 0) out[(long)blockIdx.x * stride] = v[0];
+}
+}  // namespace
+
+double* blas_norm2_workspace(const Field& x, qcd_gauge* g) {
+  return (double*)g->ws.get("blas.norm2.partial", sizeof(double) * grid_for(x.nsites()) * x.nrhs);
+}
+
+void blas_norm2_device(const Field& x, double* out, int stride, cudaStream_t st, qcd_gauge* g) {
+  const long n = x.nsites();
+  const unsigned nb = grid_for(n);
+  double* partial = blas_norm2_workspace(x, g);
+  const dim3 grid(nb, x.nrhs);
+  if (x.prec == QCD_F64)
+    k_norm2<double, P64><<<grid, kThreads, 0, st>>>(any_view(x), n, partial);
+  else if (x.prec == QCD_F32)
+    k_norm2<float, P32><<<grid, kThreads, 0, st>>>(any_view(x), n, partial);
+  else
+    k_norm2<float, P16><<<grid, kThreads, 0, st>>>(any_view(x), n, partial);
+  QCD_LAUNCH_CK();
+  k_norm2_fold<<<x.nrhs, kThreads, 0, st>>>(partial, (int)nb, out, stride);
+  QCD_LAUNCH_CK();
+}
+
 void blas_norm2(const Field& x, double* out_host, cudaStream_t st, qcd_gauge* g) {
   long n = x.nsites();
   if (n == 0) {

@@ -185,6 +185,22 @@ bool hop_fx(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int
 // the same for the Wilson Schur operator out = in - k2 H_eo H_oe in, the intermediate kept in fixed point
 bool mhat_fx(const qcd_gauge* g, const Field& in, Field& out, int dagger, double k2, cudaStream_t st, const int* stop,
              const RedSpec* red);
+// One outer step of the Wilson solve with FP64 outer precision, in fixed point (all on one handle's scratch):
+//   x += xin, xin = 0 (xin null: x as it is);  x_o = b_o + kappa H_oe x;  r = b_e - x + kappa H_eo x_o
+// or, with x_zero, r = b_e + kappa H_eo b_o.  r in its own precision.  Per right-hand side r, on the device:
+// sums[r * stride] = |r|^2 before its rounding to that precision, sums[r * stride + 1] = |b_o - x_o + kappa H_oe x|^2.
+// outer_fx_ready: the path is available on this stream and its workspace allocated for `shape`
+struct OuterStep {
+  Field x, b_e, b_o, x_o, r;
+  const Field* xin = nullptr;
+  double kappa = 0.0;
+  int dagger = 0;
+  bool x_zero = false;
+  double* sums = nullptr;
+  int sums_stride = 0;
+};
+bool outer_fx_ready(const qcd_gauge* g, const Field& shape, cudaStream_t st);
+void outer_fx(const qcd_gauge* g, const OuterStep& o, cudaStream_t st);
 // Ufx from U64; *flag (device) becomes nonzero if a link's size is outside the fixed-point range
 size_t fx_link_bytes(const Lattice& lat);
 void links_to_fx(qcd_gauge* g, int* flag, cudaStream_t st);
@@ -246,6 +262,9 @@ void blas_copy(const Field& src, Field& dst, cudaStream_t st);  // any precision
 void blas_axpby(double a, const Field& x, double b, Field& y, cudaStream_t st);
 // per right-hand side |x|^2 into host array (synchronises st)
 void blas_norm2(const Field& x, double* out_host, cudaStream_t st, qcd_gauge* g);
+// the same into out[r * stride] on the device (F64 / F32 / F16), asynchronous
+double* blas_norm2_workspace(const Field& x, qcd_gauge* g);  // its partial sums, allocated on first use
+void blas_norm2_device(const Field& x, double* out, int stride, cudaStream_t st, qcd_gauge* g);
 // per right-hand side sum |z|^2 of a canonical complex128 device array (synchronises st)
 void canon_norm2(const double* z, long n_per_rhs, int nrhs, double* out_host, cudaStream_t st,
                  qcd_gauge* g);

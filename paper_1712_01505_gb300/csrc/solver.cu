@@ -505,6 +505,21 @@ __global__ void k_rdot(AnyView a_, AnyView b_, long n, double* partial, const Sc
 
 __global__ void k_reset(int* ctl) { *ctl = 0; }
 
+// per right-hand side: out[r * stride + k] = sum over the nblk blocks of partial[(r * nblk + b) * kMaxPartial + k]
+template <int NR>
+__global__ void __launch_bounds__(kThreads) k_fold(const double* partial, int nblk, double* out, int stride) {
+  pdl_enter();
+  double v[NR];
+  sum_partials<NR>(partial, nblk, blockIdx.x, v);
+  if (threadIdx.x == 0)
+#pragma unroll
+    for (int k = 0; k < NR; ++k) out[(long)blockIdx.x * stride + k] = v[k];
+}
+
+// The sums that an outer step in fixed point leaves on the device for each right-hand side: |r|^2, the odd
+// half of the full residual, (rt, r) re and im, |b_e|^2, |b_o|^2; read by the host once per step.
+enum { SUM_RE = 0, SUM_RO = 1, SUM_RT = 2, SUM_BE = 4, SUM_BO = 5, kSums = 6 };
+
 // Blocks of a grid-stride iteration kernel: one full wave (its resident blocks per SM
 // times the SMs; fewer for short vectors), so that no partly filled last wave leaves
 // SMs idle (the FP32 x / r update holds 3 blocks per SM; launched as 4 per SM, its
@@ -720,6 +735,23 @@ struct Solver {
     QCD_CK(cudaStreamSynchronize(st));
   }
 
+  // the same into out[r * stride + 0, 1] on the device
+  void cdot_device(const Field& a, const Field& b, double* out, int stride) {
+    auto run = [&](auto kernel) {
+      const dim3 grid(wave_blocks((const void*)kernel, a.nsites()), a.nrhs);
+      launch_k(kernel, grid, kThreads, 0, st, any_view(a), any_view(b), a.nsites(), partial, nullptr, nullptr);
+      QCD_LAUNCH_CK();
+      launch_k(k_fold<2>, a.nrhs, kThreads, 0, st, partial, (int)grid.x, out, stride);
+      QCD_LAUNCH_CK();
+    };
+    if (a.prec == QCD_F64)
+      run(k_cdot<double, P64>);
+    else if (a.prec == QCD_F32)
+      run(k_cdot<float, P32>);
+    else
+      run(k_cdot<float, P16>);
+  }
+
   // host-side complex dot products (rt, r) per rhs (synchronises)
   void cdot_host(const Field& a, const Field& b, std::vector<double>& re, std::vector<double>& im) {
     const int nrhs = a.nrhs;
@@ -772,18 +804,13 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
 
   S.b_e = ws_field(g, "s.b_e", QCD_F64, ls, nrhs);
   S.b_o = ws_field(g, "s.b_o", QCD_F64, ls, nrhs);
-  S.bh = ws_field(g, "s.bh", QCD_F64, ls, nrhs);
   S.x64 = ws_field(g, "s.x64", QCD_F64, ls, nrhs);
-  S.r64 = ws_field(g, "s.r64", QCD_F64, ls, nrhs);
-  S.t64 = ws_field(g, "s.t64", QCD_F64, ls, nrhs);
-  S.u64 = ws_field(g, "s.u64", QCD_F64, ls, nrhs);
   // IEEE-FP64 outer steps of the Wilson solve keep the reconstructed odd half of x
   const bool wil64 = !dwf && !(prm.outer == QCD_DF64 && S.inner != QCD_F64);
   if (wil64) S.xo64 = ws_field(g, "s.xo64", QCD_F64, ls, nrhs);
   // ... and the even half r_e of the full-system residual: the inner residual itself for
   // BiCGStab, the source of Mhat^dag r_e for CG on the normal equations
   if (wil64 && !S.bicg()) S.re64 = ws_field(g, "s.re64", QCD_F64, ls, nrhs);
-  Field& r_e64 = S.bicg() ? S.r64 : S.re64;
   S.r = ws_field(g, "s.r", S.inner, ls, nrhs);
   S.p = ws_field(g, "s.p", S.inner, ls, nrhs);
   if (S.bicg()) {
@@ -818,6 +845,26 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
     if (g->ws.generation != gen) QCD_CK(cudaMemsetAsync(S.counters, 0, sizeof(int) * ngroups, st));
   }
   S.hsc.assign(nrhs, Scal{});
+  // BiCGStab with IEEE-FP64 outer steps: the steps in fixed point (three fused kernels, wilson_fx.cu) where
+  // that path is available, else the separate operators below.  Everything the solve allocates on the
+  // device is allocated by here, so that no later allocation can take the links of that path back.
+  bool fxo = false;
+  double* dsum = nullptr;
+  std::vector<double> hsum;
+  if (wil64 && S.bicg()) {
+    if (S.inner != QCD_F64) ws_field(g, "in.mhat.t", S.inner, ls, nrhs);  // apply_mhat's intermediate
+    dsum = (double*)g->ws.get("s.sums", sizeof(double) * kSums * nrhs);
+    hsum.assign((size_t)kSums * nrhs, 0.0);
+    blas_norm2_workspace(S.b_e, g);
+    fxo = outer_fx_ready(g, S.x64, st);
+  }
+  if (!fxo) {
+    S.bh = ws_field(g, "s.bh", QCD_F64, ls, nrhs);
+    S.r64 = ws_field(g, "s.r64", QCD_F64, ls, nrhs);
+    S.t64 = ws_field(g, "s.t64", QCD_F64, ls, nrhs);
+    S.u64 = ws_field(g, "s.u64", QCD_F64, ls, nrhs);
+  }
+  Field& r_e64 = S.bicg() ? S.r64 : S.re64;
   // Double-float outer steps (mixed solves): the prepared source, the solution
   // and the outer residual live in FP32 pairs and the outer operator
   // applications use the double-float stencil (and A^-1 for domain-wall); the
@@ -846,9 +893,14 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   pack_field(lat, 0, b, S.b_e, st);
   pack_field(lat, 1, b, S.b_o, st);
   std::vector<double> bn_e(nrhs), bn_o(nrhs), bnorm(nrhs);
-  blas_norm2(S.b_e, bn_e.data(), st, g);
-  blas_norm2(S.b_o, bn_o.data(), st, g);
-  for (int r = 0; r < nrhs; ++r) bnorm[r] = std::sqrt(bn_e[r] + bn_o[r]);
+  if (fxo) {  // read with the first residual
+    blas_norm2_device(S.b_e, dsum + SUM_BE, kSums, st, g);
+    blas_norm2_device(S.b_o, dsum + SUM_BO, kSums, st, g);
+  } else {
+    blas_norm2(S.b_e, bn_e.data(), st, g);
+    blas_norm2(S.b_o, bn_o.data(), st, g);
+    for (int r = 0; r < nrhs; ++r) bnorm[r] = std::sqrt(bn_e[r] + bn_o[r]);
+  }
   const DwParams dp = dw_params(f);
   if (dfo) {
     blas_copy(S.b_e, be_d, st);
@@ -861,8 +913,8 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       dw_ainv(dp, u_d, bh_d, 0, 1.0, nullptr, st);
     }
   } else if (!dwf) {
-    // bhat = b_e + kappa H_eo b_o
-    hop(g, S.b_o, S.bh, 0, dag, f.kappa, &S.b_e, st);
+    // bhat = b_e + kappa H_eo b_o (formed by the first outer step in fixed point)
+    if (!fxo) hop(g, S.b_o, S.bh, 0, dag, f.kappa, &S.b_e, st);
   } else {
     // bhat = W (b_e + 1/2 H_eo W b_o), W = B A^-1 (A^-1 for Shamir)
     dw_ainv(dp, S.b_o, S.t64, 0, 1.0, nullptr, st);
@@ -983,7 +1035,55 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
     blas_norm2(r64, rn.data() + r0, st, g);
   };
 
-  true_residual(!prm.x0_given, 0, nrhs);
+  // The outer step in fixed point for the right-hand sides [r0, r0 + n): x += xin (add), the true residual into the
+  // inner vector r, its sums on the device, (rt, r) among them (first: rt = r, p = v = 0 before it).  The host
+  // reads the sums once for all of them (fetch_sums).
+  auto outer_step = [&](bool x_is_zero, bool add, bool first, int r0, int n) {
+    Field xin = sub(S.xin, r0, n), xo = sub(S.xo64, r0, n), r = sub(S.r, r0, n);
+    OuterStep o;
+    o.x = sub(S.x64, r0, n);
+    o.b_e = sub(S.b_e, r0, n);
+    o.b_o = sub(S.b_o, r0, n);
+    o.x_o = xo;
+    o.r = r;
+    if (add && S.inner != QCD_F64) o.xin = &xin;
+    o.kappa = f.kappa;
+    o.dagger = dag;
+    o.x_zero = x_is_zero;
+    o.sums = dsum + (size_t)r0 * kSums + SUM_RE;
+    o.sums_stride = kSums;
+    if (x_is_zero) blas_copy(o.b_o, xo, st);
+    outer_fx(g, o, st);
+    Field rt = sub(S.rt, r0, n);
+    if (first) {
+      Field p = sub(S.p, r0, n), v = sub(S.v, r0, n);
+      blas_copy(r, rt, st);
+      blas_zero(p, st);
+      blas_zero(v, st);
+      if (S.inner != QCD_F64) blas_zero(xin, st);
+    }
+    S.cdot_device(rt, r, dsum + (size_t)r0 * kSums + SUM_RT, kSums);
+  };
+  auto fetch_sums = [&] {
+    QCD_CK(cudaMemcpyAsync(hsum.data(), dsum, sizeof(double) * hsum.size(), cudaMemcpyDeviceToHost, st));
+    QCD_CK(cudaStreamSynchronize(st));
+    for (int r = 0; r < nrhs; ++r) {
+      rn[r] = hsum[(size_t)r * kSums + SUM_RE];
+      rfull[r] = std::sqrt(rn[r]);
+    }
+  };
+
+  if (fxo) {
+    outer_step(!prm.x0_given, false, true, 0, nrhs);
+    fetch_sums();
+    for (int r = 0; r < nrhs; ++r) {
+      bn_e[r] = hsum[(size_t)r * kSums + SUM_BE];
+      bn_o[r] = hsum[(size_t)r * kSums + SUM_BO];
+      bnorm[r] = std::sqrt(bn_e[r] + bn_o[r]);
+    }
+  } else {
+    true_residual(!prm.x0_given, 0, nrhs);
+  }
   std::vector<double> target(nrhs);
   std::vector<int> conv(nrhs, 0), status(nrhs, QCD_OK), updates(nrhs, 0), restarts(nrhs, 0);
   int nactive = 0;
@@ -999,16 +1099,24 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
     }
   }
 
-  auto restart_from_residual = [&](bool full, int r0, int n) {
-    // r (inner) = outer residual; the recursion continues from the true residual
+  auto restart_from_residual = [&](bool full, int r0, int n, bool ready = false) {
+    // r (inner) = outer residual; the recursion continues from the true residual.  ready: the outer step in
+    // fixed point has left r, xin = 0 and (rt, r)
     Field r = sub(S.r, r0, n), rt = sub(S.rt, r0, n), p = sub(S.p, r0, n), v = sub(S.v, r0, n);
-    if (!cg_inner_normal) blas_copy(sub(r_outer, r0, n), r, st);
-    if (S.inner != QCD_F64) {
+    if (!cg_inner_normal && !fxo) blas_copy(sub(r_outer, r0, n), r, st);
+    if (S.inner != QCD_F64 && !ready) {
       Field xin = sub(S.xin, r0, n);
       blas_zero(xin, st);
     }
     std::vector<double> re, im;
-    if (S.bicg()) {
+    if (ready) {
+      re.resize(n);
+      im.resize(n);
+      for (int k = 0; k < n; ++k) {
+        re[k] = hsum[(size_t)(r0 + k) * kSums + SUM_RT];
+        im[k] = hsum[(size_t)(r0 + k) * kSums + SUM_RT + 1];
+      }
+    } else if (S.bicg()) {
       if (full) {
         blas_copy(r, rt, st);
         blas_zero(p, st);
@@ -1054,7 +1162,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   };
 
   for (int r = 0; r < nrhs; ++r) S.hsc[r].iters = 0;
-  if (nactive > 0) restart_from_residual(true, 0, nrhs);
+  if (nactive > 0) restart_from_residual(true, 0, nrhs, fxo);
   S.upload();
 
   // host-side fault injection for tests (no device fault is ever provoked):
@@ -1145,7 +1253,14 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
         full[r] = 1;
       }
     }
-    for_runs(due, [&](int r0, int n) {
+    if (fxo) {
+      for_runs(due, [&](int r0, int n) {
+        outer_step(false, true, false, r0, n);
+        for (int r = r0; r < r0 + n; ++r) stale[r] = 0;
+      });
+      fetch_sums();
+    }
+    if (!fxo) for_runs(due, [&](int r0, int n) {
       if (S.inner != QCD_F64) {
         Field xin = sub(S.xin, r0, n), xo = sub(dfo ? x_d : S.x64, r0, n);
         blas_axpby(1.0, xin, 1.0, xo, st);
@@ -1174,7 +1289,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       }
     }
     if (nactive == 0) break;
-    for_runs(again, [&](int r0, int n) { restart_from_residual(false, r0, n); });
+    for_runs(again, [&](int r0, int n) { restart_from_residual(false, r0, n, fxo); });
     for_runs(again_full, [&](int r0, int n) { restart_from_residual(true, r0, n); });
     S.upload();
   }
@@ -1185,9 +1300,25 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   if (wil64) {
     // x_e = x64 and x_o, h and r_e of the last outer step (recomputed where a plain FP64
     // solve stopped at maxiter after iterating past it)
-    for_runs(stale, [&](int r0, int n) { true_residual(false, r0, n); });
+    if (fxo) {
+      bool any = false;
+      for_runs(stale, [&](int r0, int n) {
+        outer_step(false, false, false, r0, n);
+        any = true;
+      });
+      if (any) fetch_sums();
+    } else {
+      for_runs(stale, [&](int r0, int n) { true_residual(false, r0, n); });
+    }
     unpack_field(lat, 0, S.x64, x, st);
     unpack_field(lat, 1, S.xo64, x, st);
+  }
+  if (fxo) {  // both halves of the full residual from the last outer step
+    for (int r = 0; r < nrhs; ++r) {
+      re_[r] = hsum[(size_t)r * kSums + SUM_RE];
+      ro_[r] = hsum[(size_t)r * kSums + SUM_RO];
+    }
+  } else if (wil64) {
     blas_norm2(r_e64, re_.data(), st, g);
     // odd half of the full residual: b_o - x_o + kappa h (rounding of the reconstruction)
     blas_copy(S.b_o, S.bh, st);

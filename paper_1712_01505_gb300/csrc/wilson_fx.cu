@@ -43,6 +43,51 @@ struct FxField {
   long nsb;  // blocks of kSB sites per slice
 };
 
+// the exponent field of a site's 12 components (words of doubles); kBad out of range
+__device__ __forceinline__ int fx_field_of(unsigned mx, unsigned low) {
+  const int e = (int)(mx >> 20);
+  if (mx == 0) return low ? kBad : kEmin;  // subnormals below 2^-1042 / all zero
+  return e < kEmin || e > kEmax ? kBad : e;
+}
+template <int N>
+__device__ __forceinline__ unsigned max_word(const int4 (&w)[N]) {
+  unsigned mx = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) mx = max(mx, max((unsigned)w[k].y & 0x7fffffffu, (unsigned)w[k].w & 0x7fffffffu));
+  return mx;
+}
+template <int N>
+__device__ __forceinline__ unsigned low_words(const int4 (&w)[N]) {
+  unsigned low = 0;
+#pragma unroll
+  for (int k = 0; k < N; ++k) low |= (unsigned)(w[k].x | w[k].z);
+  return low;
+}
+__device__ __forceinline__ int fx_exponent(const int4 (&w)[12]) { return fx_field_of(max_word(w), low_words(w)); }
+// of a site whose components are in the lanes sp = 0, 1 (six each)
+__device__ __forceinline__ int fx_exponent_pair(const int4 (&w)[6]) {
+  unsigned mx = max_word(w), low = low_words(w);
+  mx = max(mx, __shfl_xor_sync(0xffffffffu, mx, kSB));
+  low |= __shfl_xor_sync(0xffffffffu, low, kSB);
+  return fx_field_of(mx, low);
+}
+
+// store a site's 12 components (words of doubles); blk0: the slice's first block
+__device__ __forceinline__ void fx_put(const int4 (&w)[12], int e, const FxField& out, long blk0, int cb) {
+  const long blk = blk0 + cb / kSB;
+  int4* o = out.p + blk * kSiteUnits + cb % kSB;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) {
+    int4 u = w[k];
+    if (e != kBad) {
+      const Part re = spinor_part(w[k].y, w[k].x, e), im = spinor_part(w[k].w, w[k].z, e);
+      u = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
+    }
+    o[k * kSB] = u;
+  }
+  out.e[blk * kSB + cb % kSB] = e;
+}
+
 // FP64 -> fixed point: one thread per site, blockIdx.y: (right-hand side, slice)
 __global__ void __launch_bounds__(128) k_to_fx(const int4* __restrict__ in, long stride, FxField out, int Vh, int ls,
                                                const int* stop) {
@@ -55,30 +100,7 @@ __global__ void __launch_bounds__(128) k_to_fx(const int4* __restrict__ in, long
   int4 w[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) w[k] = __ldg(in + k * stride);
-  unsigned mx = 0;
-#pragma unroll
-  for (int k = 0; k < 12; ++k) mx = max(mx, max((unsigned)w[k].y & 0x7fffffffu, (unsigned)w[k].w & 0x7fffffffu));
-  int e = (int)(mx >> 20);
-  if (mx == 0) {  // all zero, or subnormals below 2^-1042
-    unsigned low = 0;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) low |= (unsigned)(w[k].x | w[k].z);
-    e = low ? 0 : kEmin;
-  }
-  const long blk = (long)blockIdx.y * out.nsb + cb / kSB;
-  int4* o = out.p + blk * kSiteUnits + cb % kSB;
-  if (e < kEmin || e > kEmax) {
-    e = kBad;
-#pragma unroll
-    for (int k = 0; k < 12; ++k) o[k * kSB] = w[k];
-  } else {
-#pragma unroll
-    for (int k = 0; k < 12; ++k) {
-      const Part re = spinor_part(w[k].y, w[k].x, e), im = spinor_part(w[k].w, w[k].z, e);
-      o[k * kSB] = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
-    }
-  }
-  out.e[blk * kSB + cb % kSB] = e;
+  fx_put(w, fx_exponent(w), out, (long)blockIdx.y * out.nsb, cb);
 }
 
 // A warp owns 16 sites, lane = 16 sp + site: the lane computes the link products of spin sp of the half
@@ -474,6 +496,255 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx_red(const __grid_c
   red_epilogue<double>(A, red);
 }
 
+// ----------------------------------------------------------------------------- outer step
+// One outer step of the mixed-precision Wilson solve (true residual of the full system) is three kernels:
+// x += xin with the result also in fixed point (k_outer_x); x_o = b_o + kappa H_oe x, in FP64 and in fixed
+// point (k_outer_odd); r_e = b_e - x + kappa H_eo x_o, kept only as the inner residual and its norm
+// (k_outer_res).  As separate stencils, copies, axpys, norms and conversions the step moved 7.4 KB per site, here
+// 4.6, and 14 launches and 3 synchronisations became 6 and 1.  Measured: 24^3 x 48 with FP16 inner vectors (6
+// steps) 16.2 -> 14.6 ms, 8^3 x 16 2.77 -> 2.25 ms, 12 right-hand sides 156 -> 150 ms, 32^3 x 64 51.3 -> 49.5 ms.
+
+// two sums of the block (all its warps one slice) into partial[(q * nsb + block) * 4 + k0 ..]
+__device__ __forceinline__ void block_partial(double v0, double* partial, long row, int k) {
+  double v[1] = {v0};
+  block_sum<1>(v);
+  if (threadIdx.x == 0) partial[row * 4 + k] = v[0];
+}
+
+// x += xin, xin = 0 (xin may be null: x as it is), and x in fixed point; blockIdx.y: right-hand side
+__global__ void __launch_bounds__(128) k_outer_x(SpinorView<P64> x, SpinorView<P32> xin, int has_xin, FxField out,
+                                                 int Vh) {
+  pdl_enter();
+  const int cb = blockIdx.x * blockDim.x + threadIdx.x;
+  if (cb >= Vh) return;
+  x = x.offset_rhs(blockIdx.y);
+  Cx<double> v[12];
+  if (has_xin) {
+    xin = xin.offset_rhs(blockIdx.y);
+    float4 d[6];
+#pragma unroll
+    for (int k = 0; k < 12; ++k) {
+      const double2 w = x.p[k * x.stride + cb];
+      v[k] = {w.x, w.y};
+    }
+#pragma unroll
+    for (int q = 0; q < 6; ++q) d[q] = xin.p[q * xin.stride + cb];
+#pragma unroll
+    for (int q = 0; q < 6; ++q) {
+      const int k = q < 3 ? q : q + 3;  // spins a (component k) and b (k + 3) of the pair
+      v[k] = {v[k].re + (double)d[q].x, v[k].im + (double)d[q].z};
+      v[k + 3] = {v[k + 3].re + (double)d[q].y, v[k + 3].im + (double)d[q].w};
+    }
+    x.store(cb, v);
+#pragma unroll
+    for (int q = 0; q < 6; ++q) xin.p[q * xin.stride + cb] = make_float4(0.f, 0.f, 0.f, 0.f);
+  } else {
+    x.load(cb, v);
+  }
+  int4 w[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k)
+    w[k] = make_int4(__double2loint(v[k].re), __double2hiint(v[k].re), __double2loint(v[k].im), __double2hiint(v[k].im));
+  const int e = fx_exponent(w);
+  fx_put(w, e, out, (long)blockIdx.y * out.nsb, cb);
+}
+
+// acc = the sum of the eight hops in FP64 values with factor a (slow path: fp64_site); the lane's six components,
+// upper spin sp then lower spin 2 + sp.  false: the warp has no such site.
+struct FxLane {
+  int cb0, cb, sp, q, r;
+  bool valid, warp_valid;
+};
+__device__ __forceinline__ FxLane fx_lane(const HA& A) {
+  FxLane L;
+  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
+  L.q = blockIdx.x - sblock * A.ntiles;
+  L.r = L.q;  // Wilson: one slice per right-hand side
+  L.cb0 = (sblock * kWarps + (threadIdx.x >> 5)) * kSB;
+  L.cb = L.cb0 + threadIdx.x % kSB;
+  L.sp = (threadIdx.x & 31) / kSB;
+  L.valid = L.cb < A.g.Vh;
+  L.warp_valid = L.cb0 < A.g.Vh;
+  return L;
+}
+
+// a H in for the lane's six components (upper spin sp, lower spin 2 + sp) as a[k / 3] v[k]
+__device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField& f, const FxLane& L, Cx<double> v[6],
+                                          double a[2]) {
+  const int E = fx_neighbours(A, W, f, L.valid ? L.cb : 0);
+  Cx<double> slow[12];
+  const bool bad = E == kBad && L.valid;
+  if (bad) fp64_site(A, f, L.cb, slow);  // both lanes of the site
+  int64_t up[6], lo[6];
+  const double unit = fx_sum(A, W, f, E, L.sp, up, lo);
+  a[0] = A.a * unit;
+  a[1] = A.dagger ? -a[0] : a[0];
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    v[c] = {(double)up[2 * c], (double)up[2 * c + 1]};
+    v[3 + c] = {(double)lo[2 * c], (double)lo[2 * c + 1]};
+  }
+  if (bad) {
+    a[0] = a[1] = A.a;
+    const Cx<double>* w = slow + 3 * L.sp;
+#pragma unroll
+    for (int n = 0; n < 6; ++n) v[n] = w[n < 3 ? n : 3 + n];
+  }
+}
+
+// out = x + a H in, FP64 and as the fixed-point field O; partial k = 1: |x - out + a H in|^2, the rounding of out
+__global__ void __launch_bounds__(32 * kWarps, 4) k_outer_odd(const __grid_constant__ HA A,
+                                                              const int4* __restrict__ links,
+                                                              const __grid_constant__ FxField F,
+                                                              const __grid_constant__ FxField O) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
+  const FxLane L = fx_lane(A);
+  FxWarp W;
+  if (L.warp_valid) W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
+  pdl_enter();
+  double res = 0.0;
+  if (L.warp_valid) {
+    const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+    Cx<double> h[6];
+    double a[2];
+    fx_values(A, W, f, L, h, a);
+    int4 w[6];
+    if (L.valid) {
+      const double2* x = A.x.offset_rhs(L.r).p + 3 * L.sp * A.x.stride + L.cb;
+      double2* o = A.out.offset_rhs(L.r).p + 3 * L.sp * A.out.stride + L.cb;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        const int n = k < 3 ? k : 3 + k;
+        const double2 xs = __ldg(x + n * A.x.stride);
+        const double ak = a[k / 3];
+        const Cx<double> v = {fma(ak, h[k].re, xs.x), fma(ak, h[k].im, xs.y)};
+        o[n * A.out.stride] = make_double2(v.re, v.im);
+        const double dr = fma(ak, h[k].re, xs.x - v.re), di = fma(ak, h[k].im, xs.y - v.im);
+        res = fma(dr, dr, fma(di, di, res));
+        w[k] = make_int4(__double2loint(v.re), __double2hiint(v.re), __double2loint(v.im), __double2hiint(v.im));
+      }
+    } else {
+#pragma unroll
+      for (int k = 0; k < 6; ++k) w[k] = make_int4(0, 0, 0, 0);
+    }
+    const int e = fx_exponent_pair(w);
+    if (L.valid) {
+      int4* o = O.p + ((long)L.q * O.nsb + L.cb / kSB) * kSiteUnits + 3 * L.sp * kSB + L.cb % kSB;
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        int4 u = w[k];
+        if (e != kBad) {
+          const Part re = spinor_part(w[k].y, w[k].x, e), im = spinor_part(w[k].w, w[k].z, e);
+          u = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
+        }
+        o[(k < 3 ? k : 3 + k) * kSB] = u;
+      }
+      if (L.sp == 0) O.e[(long)L.q * O.nsb * kSB + L.cb] = e;
+    }
+  }
+  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
+  block_partial(res, A.partial, (long)L.q * (gridDim.x / A.ntiles) + sblock, 1);
+}
+
+// r = b - x + a H in (x only with A.xpay = 2), stored in the inner precision PR; partial k = 0: |b - x + a H in|^2
+template <int PR>
+__global__ void __launch_bounds__(32 * kWarps, 4) k_outer_res(const __grid_constant__ HA A,
+                                                              const int4* __restrict__ links,
+                                                              const __grid_constant__ FxField F,
+                                                              const __grid_constant__ SpinorView<PR> R) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
+  const FxLane L = fx_lane(A);
+  FxWarp W;
+  if (L.warp_valid) W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
+  pdl_enter();
+  double res = 0.0;
+  if (L.warp_valid) {
+    const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+    Cx<double> h[6];
+    double a[2];
+    fx_values(A, W, f, L, h, a);
+    const int cb = L.valid ? L.cb : 0;
+    const double2* b = A.rt.offset_rhs(L.r).p + 3 * L.sp * A.rt.stride + cb;
+    const double2* x = A.x.offset_rhs(L.r).p + 3 * L.sp * A.x.stride + cb;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) {
+      const int n = k < 3 ? k : 3 + k;
+      double2 t = __ldg(b + n * A.rt.stride);
+      if (A.xpay == 2) {
+        const double2 xs = __ldg(x + n * A.x.stride);
+        t = make_double2(t.x - xs.x, t.y - xs.y);
+      }
+      h[k] = {fma(a[k / 3], h[k].re, t.x), fma(a[k / 3], h[k].im, t.y)};
+      if (L.valid) res = fma(h[k].re, h[k].re, fma(h[k].im, h[k].im, res));
+    }
+    const SpinorView<PR> rv = R.offset_rhs(L.r);
+    if constexpr (PR == P64) {
+      if (L.valid)
+#pragma unroll
+        for (int k = 0; k < 6; ++k)
+          rv.p[(3 * L.sp + (k < 3 ? k : 3 + k)) * rv.stride + cb] = make_double2(h[k].re, h[k].im);
+    } else {
+      // FP32 / FP16 units hold a spin pair: the lanes of a site exchange halves, lane 0 stores the upper pairs, lane 1
+      // the lower ones
+      float mine[6], other[6], m = 0.f;
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        const Cx<double> keep = L.sp ? h[3 + c] : h[c], give = L.sp ? h[c] : h[3 + c];
+        mine[2 * c] = (float)keep.re;
+        mine[2 * c + 1] = (float)keep.im;
+        other[2 * c] = __shfl_xor_sync(0xffffffffu, (float)give.re, kSB);
+        other[2 * c + 1] = __shfl_xor_sync(0xffffffffu, (float)give.im, kSB);
+      }
+      float inv = 1.f;
+      if constexpr (PR == P16) {
+#pragma unroll
+        for (int k = 0; k < 6; ++k) m = fmaxf(m, fmaxf(fabsf(mine[k]), fabsf(other[k])));
+        m = fmaxf(m, __shfl_xor_sync(0xffffffffu, m, kSB));
+        inv = (m > 0.f) ? 1.0f / m : 0.f;
+      }
+      if (L.valid) {
+#pragma unroll
+        for (int c = 0; c < 3; ++c) {
+          const int q = 3 * L.sp + c;
+          // spins (a, b): lane 0 has spin a of the upper pair, lane 1 spin b of the lower one
+          const float ar = L.sp ? other[2 * c] : mine[2 * c], br = L.sp ? mine[2 * c] : other[2 * c];
+          const float ai = L.sp ? other[2 * c + 1] : mine[2 * c + 1], bi = L.sp ? mine[2 * c + 1] : other[2 * c + 1];
+          if constexpr (PR == P32) {
+            rv.p[q * rv.stride + cb] = make_float4(ar, br, ai, bi);
+          } else {
+            const __half2 re = __floats2half2_rn(ar * inv, br * inv), im = __floats2half2_rn(ai * inv, bi * inv);
+            uint2* u = reinterpret_cast<uint2*>(rv.p + (q >> 1) * rv.stride + cb) + (q & 1);
+            *u = make_uint2(*reinterpret_cast<const unsigned*>(&re), *reinterpret_cast<const unsigned*>(&im));
+          }
+        }
+        if constexpr (PR == P16)
+          if (L.sp == 0) rv.norm[cb] = m;
+      }
+    }
+  }
+  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
+  block_partial(res, A.partial, (long)L.q * (gridDim.x / A.ntiles) + sblock, 0);
+}
+
+// sums[q * stride + k] = sum over the blocks of partial[(q * nb + b) * 4 + k], k < 2 (k = 1 only with both)
+__global__ void __launch_bounds__(256) k_outer_sums(const double* __restrict__ partial, int nb, double* __restrict__ sums,
+                                                    int stride, int both) {
+  pdl_enter();
+  const int q = blockIdx.x;
+  double v[2] = {0.0, 0.0};
+  for (int b = threadIdx.x; b < nb; b += blockDim.x) {
+    v[0] += partial[((long)q * nb + b) * 4];
+    if (both) v[1] += partial[((long)q * nb + b) * 4 + 1];
+  }
+  block_sum<2>(v);
+  if (threadIdx.x == 0) {
+    sums[(long)q * stride] = v[0];
+    sums[(long)q * stride + 1] = v[1];
+  }
+}
+
 // ----------------------------------------------------------------------------- links
 // The links of the eight hops as parts, and whether every link has the size the fixed point takes:
 // *flag becomes nonzero if a row or column 2-norm lies outside [kNormMin, kNormMax] (or is NaN).
@@ -569,6 +840,19 @@ void fx_pack(const Field& in, const FxField& out, cudaStream_t st, const int* st
   QCD_LAUNCH_CK();
 }
 
+void fx_args(HA& A, const qcd_gauge* gh, const Field& shape, int out_parity, int dagger, double a) {
+  A.g = make_geom(gh->lat.L, gh->lat.bc, gh->lat.V, gh->lat.Vh);
+  A.out_parity = out_parity;
+  A.ls = shape.ls;
+  A.d_ls = make_fastdiv((unsigned)shape.ls);
+  A.nslices = A.ntiles = shape.ls * shape.nrhs;
+  A.d_ntiles = make_fastdiv((unsigned)A.ntiles);
+  A.dagger = dagger;
+  A.a = a;
+  A.U.p = (const double2*)gh->U64;
+  A.U.Vh = gh->lat.Vh;
+}
+
 // out = [x +] a H in (out FP64), or the fixed-point field fout = H in (a = 1, x null)
 void fx_launch(const qcd_gauge* gh, const FxField& in, const Field& shape, Field* out, const FxField* fout,
                int out_parity, int dagger, double a, const Field* x, cudaStream_t st, const int* stop,
@@ -587,17 +871,8 @@ void fx_launch(const qcd_gauge* gh, const FxField& in, const Field& shape, Field
     A.counters = red->counters;
     A.npartial = red->npartial;
   }
-  A.g = make_geom(gh->lat.L, gh->lat.bc, gh->lat.V, gh->lat.Vh);
-  A.out_parity = out_parity;
-  A.ls = shape.ls;
-  A.d_ls = make_fastdiv((unsigned)shape.ls);
-  A.nslices = A.ntiles = shape.ls * shape.nrhs;
-  A.d_ntiles = make_fastdiv((unsigned)A.ntiles);
-  A.dagger = dagger;
+  fx_args(A, gh, shape, out_parity, dagger, a);
   A.xpay = x != nullptr;
-  A.a = a;
-  A.U.p = (const double2*)gh->U64;
-  A.U.Vh = gh->lat.Vh;
   A.out = out ? fx_view(*out) : fx_view(shape);
   A.in = A.out;  // not read: the input is L.F
   A.x = x ? fx_view(*x) : A.out;
@@ -702,6 +977,73 @@ bool mhat_fx(const qcd_gauge* gh, const Field& in, Field& out, int dagger, doubl
   fx_launch(g, t, in, &out, nullptr, 0, dagger, -k2, &in, st, stop, red);
   order.done();
   return true;
+}
+
+bool outer_fx_ready(const qcd_gauge* gh, const Field& shape, cudaStream_t st) {
+  if (!fx_usable(gh, st)) return false;
+  qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  try {
+    fx_scratch(g, "opt.fx.a", shape);
+    fx_scratch(g, "opt.fx.b", shape);
+    const size_t nb = (size_t)(shape.Vh + kWarps * kSB - 1) / (kWarps * kSB);
+    g->ws.get("s.outer", sizeof(double) * 4 * nb * shape.nrhs);
+  } catch (const Error& e) {
+    if (e.status != QCD_ERR_OOM) throw;
+    return false;
+  }
+  return g->fx_ok;
+}
+
+void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
+  qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  const Field& shape = o.x;
+  const FxField fa = fx_scratch(g, "opt.fx.a", shape), fb = fx_scratch(g, "opt.fx.b", shape);
+  const unsigned nb = (unsigned)((shape.Vh + kWarps * kSB - 1) / (kWarps * kSB)), n = (unsigned)shape.nrhs;
+  double* partial = (double*)g->ws.get("s.outer", sizeof(double) * 4 * nb * n);
+  const int4* links = (const int4*)g->Ufx;
+  static std::atomic<unsigned long long> attr_mask{0};
+  if (first_use_on_device(attr_mask))
+    for (const void* k : {(const void*)k_outer_odd, (const void*)k_outer_res<P64>, (const void*)k_outer_res<P32>,
+                          (const void*)k_outer_res<P16>})
+      QCD_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared)));
+  FxOrder order(g, st);
+  const dim3 sites((unsigned)((shape.Vh + 127) / 128), n);
+  if (o.x_zero) {
+    fx_pack(o.b_o, fb, st, nullptr);  // x_o = b_o
+  } else {
+    SpinorView<P32> xin{};
+    if (o.xin) xin = {(float4*)o.xin->data, nullptr, o.xin->nsites()};
+    launch_k(k_outer_x, sites, 128, 0, st, fx_view(o.x), xin, (int)(o.xin != nullptr), fa, (int)shape.Vh);
+    QCD_LAUNCH_CK();
+    HA A;
+    fx_args(A, g, shape, 1, o.dagger, o.kappa);
+    A.stop = nullptr;
+    A.partial = partial;
+    A.x = fx_view(o.b_o);
+    A.out = fx_view(o.x_o);
+    launch_k(k_outer_odd, nb * n, 32 * kWarps, sizeof(FxShared), st, A, links, fa, fb);
+    QCD_LAUNCH_CK();
+  }
+  HA A;
+  fx_args(A, g, shape, 0, o.dagger, o.kappa);
+  A.stop = nullptr;
+  A.partial = partial;
+  A.xpay = o.x_zero ? 1 : 2;
+  A.rt = fx_view(o.b_e);
+  A.x = fx_view(o.x);
+  if (o.r.prec == QCD_F64) {
+    launch_k(k_outer_res<P64>, nb * n, 32 * kWarps, sizeof(FxShared), st, A, links, fb, fx_view(o.r));
+  } else if (o.r.prec == QCD_F32) {
+    const SpinorView<P32> r{(float4*)o.r.data, nullptr, o.r.nsites()};
+    launch_k(k_outer_res<P32>, nb * n, 32 * kWarps, sizeof(FxShared), st, A, links, fb, r);
+  } else {
+    const SpinorView<P16> r{(uint4*)o.r.data, o.r.norm, o.r.nsites()};
+    launch_k(k_outer_res<P16>, nb * n, 32 * kWarps, sizeof(FxShared), st, A, links, fb, r);
+  }
+  QCD_LAUNCH_CK();
+  launch_k(k_outer_sums, n, 256, 0, st, partial, (int)nb, o.sums, o.sums_stride, (int)!o.x_zero);
+  QCD_LAUNCH_CK();
+  order.done();
 }
 
 }  // namespace qcd

@@ -158,3 +158,33 @@ def test_capture_and_streams():
     for k in range(4):
         assert torch.equal(bufs[4 + k].view(torch.float64), want[k])
     g.free()
+
+
+@pytest.mark.parametrize("inner", ["f64", "f32", "f16"])
+@pytest.mark.parametrize("dagger", [False, True])
+@pytest.mark.parametrize("L,nrhs", [((2, 2, 2, 4), 1), ((6, 4, 6, 10), 1), ((4, 6, 4, 6), 3)])
+def test_outer_steps_of_a_solve(inner, dagger, L, nrhs):
+    """The solve whose outer steps run in fixed point: ragged site blocks, one and several right-hand sides, an initial
+    guess, sources that are zero or 1e-250 away from one site.  Tolerance: the requested residual, by the oracle."""
+    device()
+    V = int(np.prod(L))
+    U = inputs.gauge_field(L, 0.3, 15)
+    b = inputs.z2_source((nrhs, V, 4, 3), 16)
+    b[0] *= 1e-250
+    b[0, V // 3, 1, 2] = 1.0
+    if nrhs > 1:
+        b[1] = 0
+        b[1, 5, 3, 0] = 1.0
+    g = qcd.Gauge.load(to_dev(U), L, BC, recon=12)
+    f = qcd.wilson(KAPPA)
+    x = torch.zeros((nrhs, V, 4, 3), dtype=torch.complex128, device=device())
+    for guess in (False, True):
+        if guess:
+            x = x * 1.25
+        info, _ = qcd.solve(g, f, to_dev(b), x, nrhs=nrhs, tol=1e-12, inner=inner, dagger=dagger, use_graph=True,
+                            graph_chunk=8, x0_given=guess)
+        xr = x.cpu().numpy()
+        for r in range(nrhs):
+            res = np.linalg.norm(b[r] - ora.wilson(L, BC, KAPPA, U, xr[r], dagger=dagger)) / np.linalg.norm(b[r])
+            assert res <= 1.01e-12 and abs(res - info[r]["true_resid"]) <= 1e-2 * res + 2e-15, (res, info[r])
+    g.free()
