@@ -281,8 +281,9 @@ qcd_status qcd_force_project(const qcd_gauge* g, const void* dSdU, void* F, void
 /* Molecular-dynamics updates on canonical arrays of nlinks 3x3 complex128
  * matrices (device; e.g. (4, V, 3, 3) gauge links and su(3) momenta):
  *   qcd_link_update: U <- exp(eps P) U for every link (P traceless
- *     anti-Hermitian; exp by scaling and squaring of a degree-13 Taylor
- *     polynomial, accurate to rounding);
+ *     anti-Hermitian; exp by its Taylor series of degree 11 or 16 modulo the
+ *     characteristic polynomial, after scaling for large |eps P|, accurate to
+ *     rounding);
  *   qcd_mom_update:  P <- P + c F;
  *   qcd_mom_energy:  *out = sum over all entries of |P_ab|^2 (= sum tr(P^dag P)),
  *     summed in FP64 in a fixed order; synchronises the stream.  Its partial
