@@ -297,7 +297,6 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
     QCD_CK(cudaStreamCreateWithFlags(&g->work, cudaStreamNonBlocking));
     QCD_CK(cudaEventCreateWithFlags(&g->ev_in, cudaEventDisableTiming));
     QCD_CK(cudaEventCreateWithFlags(&g->ev_out, cudaEventDisableTiming));
-    QCD_CK(cudaEventCreateWithFlags(&g->fx_ev, cudaEventDisableTiming));
     size_t links = 4 * (size_t)lat.V;
     g->U64 = g->ws.get("gauge.U64", links * 18 * sizeof(double));
     g->U32 = g->ws.get("gauge.U32", links * lat.recon * sizeof(float));
@@ -308,10 +307,10 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
     gauge_reorder(g, su.dev, st);
     links_to_df(g, st);
     int fx_bad = 1;
-    int* fx_flag = (int*)g->ws.get("gauge.fx", sizeof(int));
     g->ws.opt_in_use = &g->fx_ok;
     try {  // optional: without it the FP64 stencil runs on U64
-      g->Ufx = g->ws.get("opt.Ufx", fx_link_bytes(lat));
+      g->Ufx = g->ws.get("opt.Ufx", fx_link_bytes(lat) + sizeof(int));
+      int* fx_flag = (int*)((char*)g->Ufx + fx_link_bytes(lat));
       links_to_fx(g, fx_flag, st);
       QCD_CK(cudaMemcpyAsync(&fx_bad, fx_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     } catch (const Error& e) {
@@ -351,7 +350,7 @@ qcd_status qcd_gauge_free(qcd_gauge* g) {
     cudaStreamDestroy(g->work);
     cudaEventDestroy(g->ev_in);
     cudaEventDestroy(g->ev_out);
-    cudaEventDestroy(g->fx_ev);
+    if (g->fx_ev) cudaEventDestroy(g->fx_ev);
     delete g;
   });
 }

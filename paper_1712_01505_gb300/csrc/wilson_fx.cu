@@ -905,6 +905,7 @@ struct FxOrder {
   qcd_gauge* g;
   cudaStream_t st;
   FxOrder(qcd_gauge* g_, cudaStream_t st_) : g(g_), st(st_) {
+    if (!g->fx_ev) QCD_CK(cudaEventCreateWithFlags(&g->fx_ev, cudaEventDisableTiming));
     if (!g->fx_used || g->fx_stream == st) return;
     if (g->fx_stream == g->work) QCD_CK(cudaEventRecord(g->fx_ev, g->work));
     QCD_CK(cudaStreamWaitEvent(st, g->fx_ev, 0));
