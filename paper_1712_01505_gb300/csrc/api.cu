@@ -446,6 +446,10 @@ qcd_status qcd_dslash(const qcd_gauge* gc, const qcd_fermion* fermion, qcd_prec 
     check_disjoint(in, out, cb);
     Staged si = stage_in(g, "io.in", in, cb, st, true);
     Staged so = stage_in(g, "io.out", out, cb, st, false);
+    if (!dwf && prec == QCD_F64 && canon_fx(g, *fermion, op, si.dev, so.dev, nrhs, st)) {
+      stage_out(so, out, cb, st);
+      return;
+    }
     Field a = ws_field(g, "d.a", prec, ls, nrhs);
     Field b = ws_field(g, "d.b", prec, ls, nrhs);
     const int nvec = nrhs * ls;

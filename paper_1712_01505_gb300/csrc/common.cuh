@@ -159,6 +159,13 @@ __device__ __forceinline__ SiteCoords cb_to_site(const Geom& g, int cb, int pari
   return c;
 }
 
+// canonical index of checkerboard site cb of `parity`
+__device__ __forceinline__ int canon_index(const Geom& g, int cb, int parity) {
+  const int r = fdiv(2 * cb, g.dL[0]), r2 = fdiv(r, g.dL[1]), t = fdiv(r2, g.dL[2]);
+  const int y = r - r2 * g.L[1], z = r2 - t * g.L[2];
+  return 2 * cb + ((parity + y + z + t) & 1);  // an x row starts at an even index (Lx even)
+}
+
 // canonical index of the neighbour x +- mu_hat; *wrap = 1 if the step crosses
 // the lattice boundary.
 __device__ __forceinline__ int neighbour_index(const Geom& g, const SiteCoords& c, int mu, int dir,
@@ -529,6 +536,44 @@ __device__ __forceinline__ void any_store(const AnyView& v, int r, long site, co
     any_store_p<R, P32>(v, r, site, in);
   else
     any_store_p<R, P16>(v, r, site, in);
+}
+
+// ----------------------------------------------------------------------------- canonical fields
+// A canonical site is 12 complex128 in a row (192 bytes).  A warp turns 32 of them around in shared memory, so
+// that the memory side moves runs of 16-byte units (a thread that walks its own site touches 32 lines per
+// access: unpacking a parity of 24^3 x 48 took 49 us, 20 this way) and each lane has its own site.
+constexpr int kCanonPitch = 13;  // units between sites (12 and one of padding against bank conflicts)
+struct CanonWarp {
+  double2 u[32 * kCanonPitch];
+  long base[32];  // first unit of the lane's site, -1: none
+};
+// lanes' sites -> v (12 units); the whole warp calls it
+__device__ __forceinline__ void canon_load(CanonWarp& w, const double2* __restrict__ canon, long base, double2 (&v)[12]) {
+  const int lane = threadIdx.x & 31;
+  w.base[lane] = base;
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 12; ++j) {
+    const int u = j * 32 + lane, site = u / 12, k = u - 12 * site;
+    const long b = w.base[site];
+    if (b >= 0) w.u[site * kCanonPitch + k] = __ldg(canon + b + k);
+  }
+  __syncwarp();
+#pragma unroll
+  for (int k = 0; k < 12; ++k) v[k] = w.u[lane * kCanonPitch + k];
+}
+__device__ __forceinline__ void canon_store(CanonWarp& w, double2* canon, long base, const double2 (&v)[12]) {
+  const int lane = threadIdx.x & 31;
+  w.base[lane] = base;
+#pragma unroll
+  for (int k = 0; k < 12; ++k) w.u[lane * kCanonPitch + k] = v[k];
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < 12; ++j) {
+    const int u = j * 32 + lane, site = u / 12, k = u - 12 * site;
+    const long b = w.base[site];
+    if (b >= 0) canon[b + k] = w.u[site * kCanonPitch + k];
+  }
 }
 
 // ----------------------------------------------------------------------------- block reduction

@@ -185,6 +185,9 @@ bool hop_fx(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int
 // the same for the Wilson Schur operator out = in - k2 H_eo H_oe in, the intermediate kept in fixed point
 bool mhat_fx(const qcd_gauge* g, const Field& in, Field& out, int dagger, double k2, cudaStream_t st, const int* stop,
              const RedSpec* red);
+// an operator of qcd_dslash on canonical FP64 Wilson fields on the device; false as hop_fx
+bool canon_fx(const qcd_gauge* g, const qcd_fermion& f, int op, const double* in, double* out, int nrhs,
+              cudaStream_t st);
 // One outer step of the Wilson solve with FP64 outer precision, in fixed point (all on one handle's scratch):
 //   x += xin, xin = 0 (xin null: x as it is);  x_o = b_o + kappa H_oe x;  r = b_e - x + kappa H_eo x_o
 // or, with x_zero, r = b_e + kappa H_eo b_o.  r in its own precision.  Per right-hand side r, on the device:

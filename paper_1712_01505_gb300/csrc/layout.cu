@@ -65,57 +65,59 @@ __global__ void k_gauge_reorder(Geom g, const double2* __restrict__ U, double2* 
   }
 }
 
+constexpr int kPackThreads = 128;
+
+// the site of thread n: its right-hand side, its place in the field and its first unit in the canonical array
+struct PackSite {
+  int r;
+  long q, base;
+};
+__device__ __forceinline__ PackSite pack_site(const Geom& g, int parity, int ls, long n) {
+  const long nsites = (long)ls * g.Vh;
+  PackSite p;
+  p.r = (int)(n / nsites);
+  p.q = n - p.r * nsites;
+  const int s = (int)(p.q / g.Vh), cb = (int)(p.q - (long)s * g.Vh);
+  p.base = (((long)p.r * ls + s) * g.V + canon_index(g, cb, parity)) * 12;
+  return p;
+}
+
 // one thread per (rhs, slice, cb) of the requested parity
 template <int P>
-__global__ void k_pack(Geom g, int parity, const double2* __restrict__ canon, SpinorView<P> out,
-                       int ls, int nrhs) {
-  long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  long nsites = (long)ls * g.Vh;
-  if (n >= nsites * nrhs) return;
-  int r = (int)(n / nsites);
-  long q = n % nsites;
-  int s = (int)(q / g.Vh);
-  long cb = q % g.Vh;
-  // canonical index of this cb on `parity`
-  long i2 = 2 * cb;
-  int x0 = (int)(i2 % g.L[0]);
-  long rr = i2 / g.L[0];
-  int y = (int)(rr % g.L[1]);
-  rr /= g.L[1];
-  int z = (int)(rr % g.L[2]);
-  int t = (int)(rr / g.L[2]);
-  long i = i2 + ((parity + y + z + t) & 1);
-  (void)x0;
-  const double2* src = canon + (((long)r * ls + s) * g.V + i) * 12;
+__global__ void __launch_bounds__(kPackThreads) k_pack(Geom g, int parity, const double2* __restrict__ canon,
+                                                       SpinorView<P> out, int ls, long total) {
+  __shared__ CanonWarp sm[kPackThreads / 32];
+  const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  PackSite p{0, 0, -1};
+  if (n < total) p = pack_site(g, parity, ls, n);
+  double2 src[12];
+  canon_load(sm[threadIdx.x >> 5], canon, p.base, src);
+  if (n >= total) return;
   using R = typename SpinorView<P>::R;
   Cx<R> v[12];
 #pragma unroll
   for (int k = 0; k < 12; ++k) v[k] = {(R)src[k].x, (R)src[k].y};
-  out.offset_rhs(r).store(q, v);
+  out.offset_rhs(p.r).store(p.q, v);
 }
 
 template <int P>
-__global__ void k_unpack(Geom g, int parity, SpinorView<P> in, double2* canon, int ls, int nrhs) {
-  long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
-  long nsites = (long)ls * g.Vh;
-  if (n >= nsites * nrhs) return;
-  int r = (int)(n / nsites);
-  long q = n % nsites;
-  int s = (int)(q / g.Vh);
-  long cb = q % g.Vh;
-  long i2 = 2 * cb;
-  long rr = i2 / g.L[0];
-  int y = (int)(rr % g.L[1]);
-  rr /= g.L[1];
-  int z = (int)(rr % g.L[2]);
-  int t = (int)(rr / g.L[2]);
-  long i = i2 + ((parity + y + z + t) & 1);
+__global__ void __launch_bounds__(kPackThreads) k_unpack(Geom g, int parity, SpinorView<P> in, double2* canon, int ls,
+                                                         long total) {
+  __shared__ CanonWarp sm[kPackThreads / 32];
+  const long n = blockIdx.x * (long)blockDim.x + threadIdx.x;
+  PackSite p{0, 0, -1};
   using R = typename SpinorView<P>::R;
-  Cx<R> v[12];
-  in.offset_rhs(r).load(q, v);
-  double2* dst = canon + (((long)r * ls + s) * g.V + i) * 12;
+  double2 dst[12];
 #pragma unroll
-  for (int k = 0; k < 12; ++k) dst[k] = make_double2((double)v[k].re, (double)v[k].im);
+  for (int k = 0; k < 12; ++k) dst[k] = make_double2(0.0, 0.0);
+  if (n < total) {
+    p = pack_site(g, parity, ls, n);
+    Cx<R> v[12];
+    in.offset_rhs(p.r).load(p.q, v);
+#pragma unroll
+    for (int k = 0; k < 12; ++k) dst[k] = make_double2((double)v[k].re, (double)v[k].im);
+  }
+  canon_store(sm[threadIdx.x >> 5], canon, p.base, dst);
 }
 
 __global__ void k_zero_parity(Geom g, int parity, double2* canon, long nvec) {
@@ -165,16 +167,16 @@ void pack_field(const Lattice& lat, int parity, const double* canon, Field& f, c
   const double2* c = (const double2*)canon;
   switch (f.prec) {
     case QCD_F64:
-      k_pack<P64><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, c, view_of<P64>(f), f.ls, f.nrhs);
+      k_pack<P64><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, c, view_of<P64>(f), f.ls, n);
       break;
     case QCD_F32:
-      k_pack<P32><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, c, view_of<P32>(f), f.ls, f.nrhs);
+      k_pack<P32><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, c, view_of<P32>(f), f.ls, n);
       break;
     case QCD_DF64:
-      k_pack<PDF><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, c, view_of<PDF>(f), f.ls, f.nrhs);
+      k_pack<PDF><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, c, view_of<PDF>(f), f.ls, n);
       break;
     default:
-      k_pack<P16><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, c, view_of<P16>(f), f.ls, f.nrhs);
+      k_pack<P16><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, c, view_of<P16>(f), f.ls, n);
   }
   QCD_LAUNCH_CK();
 }
@@ -186,16 +188,16 @@ void unpack_field(const Lattice& lat, int parity, const Field& f, double* canon,
   double2* c = (double2*)canon;
   switch (f.prec) {
     case QCD_F64:
-      k_unpack<P64><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, view_of<P64>(f), c, f.ls, f.nrhs);
+      k_unpack<P64><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, view_of<P64>(f), c, f.ls, n);
       break;
     case QCD_F32:
-      k_unpack<P32><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, view_of<P32>(f), c, f.ls, f.nrhs);
+      k_unpack<P32><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, view_of<P32>(f), c, f.ls, n);
       break;
     case QCD_DF64:
-      k_unpack<PDF><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, view_of<PDF>(f), c, f.ls, f.nrhs);
+      k_unpack<PDF><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, view_of<PDF>(f), c, f.ls, n);
       break;
     default:
-      k_unpack<P16><<<blocks_for(n, 256), 256, 0, st>>>(dg, parity, view_of<P16>(f), c, f.ls, f.nrhs);
+      k_unpack<P16><<<blocks_for(n, kPackThreads), kPackThreads, 0, st>>>(dg, parity, view_of<P16>(f), c, f.ls, n);
   }
   QCD_LAUNCH_CK();
 }

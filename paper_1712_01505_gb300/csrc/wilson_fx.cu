@@ -103,6 +103,24 @@ __global__ void __launch_bounds__(128) k_to_fx(const int4* __restrict__ in, long
   fx_put(w, fx_exponent(w), out, (long)blockIdx.y * out.nsb, cb);
 }
 
+// the same from a canonical field; blockIdx.y: right-hand side, blockIdx.z: parity - parity0
+__global__ void __launch_bounds__(128) k_canon_to_fx(Geom g, const double2* __restrict__ canon, FxField even, FxField odd,
+                                                     int parity0) {
+  __shared__ CanonWarp sm[4];
+  pdl_enter();
+  const int cb = blockIdx.x * blockDim.x + threadIdx.x, parity = parity0 + blockIdx.z;
+  const bool valid = cb < g.Vh;
+  double2 v[12];
+  canon_load(sm[threadIdx.x >> 5], canon, valid ? ((long)blockIdx.y * g.V + canon_index(g, cb, parity)) * 12 : -1, v);
+  if (!valid) return;
+  int4 w[12];
+#pragma unroll
+  for (int k = 0; k < 12; ++k)
+    w[k] = make_int4(__double2loint(v[k].x), __double2hiint(v[k].x), __double2loint(v[k].y), __double2hiint(v[k].y));
+  const FxField& out = parity ? odd : even;
+  fx_put(w, fx_exponent(w), out, (long)blockIdx.y * out.nsb, cb);
+}
+
 // A warp owns 16 sites, lane = 16 sp + site: the lane computes the link products of spin sp of the half
 // spinors (three colours instead of six: half the registers per thread, twice the warps), sums the upper spin
 // sp and, of the lower spins, the one that spin sp of the half spinor feeds: 1 - sp in the x and y hops, sp in the z and
@@ -745,6 +763,53 @@ __global__ void __launch_bounds__(256) k_outer_sums(const double* __restrict__ p
   }
 }
 
+// ----------------------------------------------------------------------------- canonical fields
+// out = [x +] a H in on canonical x and out (complex128, both parities): the operators of qcd_dslash on canonical
+// FP64 fields without FP64 copies of their halves.  Each warp's 16 sites leave through its link buffers, so that
+// whole sites are written in runs; zero: the other site of each pair (the other parity) is zeroed with them.
+// Bound by HBM (1732 B per site and half-dslash).  The full matrix at 24^3 x 48: two packings, two conversions, two
+// stencils and two unpackings 415 us, one conversion (66 us, at the copy rate) and two of these 309 us
+// (96 registers; 327 at 128).  Reading x through shared memory in runs after the hops was slower (368 us): the
+// lanes' own loads of 48 bytes are in flight earlier.
+__global__ void __launch_bounds__(32 * kWarps, 5) k_hop_fx_canon(const __grid_constant__ HA A,
+                                                                    const int4* __restrict__ links,
+                                                                    const __grid_constant__ FxField F,
+                                                                    const double2* __restrict__ x, double2* out, int zero) {
+  extern __shared__ __align__(128) unsigned char smraw[];
+  FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
+  const FxLane L = fx_lane(A);
+  if (!L.warp_valid) return;
+  FxWarp W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
+  pdl_enter();
+  const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+  const long first = (long)L.q * A.g.V * 12;
+  const double2* xs = x + first + (long)canon_index(A.g, L.valid ? L.cb : 0, A.out_parity) * 12;
+  Cx<double> h[6];
+  double a[2];
+  fx_values(A, W, f, L, h, a);
+  double2* buf = reinterpret_cast<double2*>(&sm.w[W.warp][0][0]);  // [site][12]
+  static_assert(sizeof(sm.w[0]) >= kSB * 12 * sizeof(double2), "a warp's sites fit its link buffers");
+  __syncwarp();  // every lane has read the last links
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const int n = 3 * L.sp + (k < 3 ? k : 3 + k);
+    double2 v = make_double2(0.0, 0.0);
+    if (A.xpay) v = __ldg(xs + n);
+    buf[(L.cb - L.cb0) * 12 + n] = make_double2(fma(a[k / 3], h[k].re, v.x), fma(a[k / 3], h[k].im, v.y));
+  }
+  __syncwarp();
+#pragma unroll
+  for (int j = 0; j < kSB * 12 / 32; ++j) {
+    const int u = j * 32 + W.lane, site = u / 12, k = u - 12 * site;
+    if (L.cb0 + site < A.g.Vh) {
+      double2* o = out + first + k;
+      const long c = canon_index(A.g, L.cb0 + site, A.out_parity);
+      o[c * 12] = buf[u];
+      if (zero) o[(c ^ 1) * 12] = make_double2(0.0, 0.0);
+    }
+  }
+}
+
 // ----------------------------------------------------------------------------- links
 // The links of the eight hops as parts, and whether every link has the size the fixed point takes:
 // *flag becomes nonzero if a row or column 2-norm lies outside [kNormMin, kNormMax] (or is NaN).
@@ -1045,6 +1110,60 @@ void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
   launch_k(k_outer_sums, n, 256, 0, st, partial, (int)nb, o.sums, o.sums_stride, (int)!o.x_zero);
   QCD_LAUNCH_CK();
   order.done();
+}
+
+bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* in, double* out, int nrhs,
+              cudaStream_t st) {
+  if (!fx_usable(gh, st)) return false;
+  qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  Field shape;
+  shape.prec = QCD_F64;
+  shape.Vh = g->lat.Vh;
+  shape.nrhs = nrhs;
+  FxField fa, fb;
+  try {
+    fx_scratch(g, "opt.fx.a", shape);
+    fb = fx_scratch(g, "opt.fx.b", shape);
+    if (g->fx_ok) fa = fx_scratch(g, "opt.fx.a", shape);
+  } catch (const Error& e) {
+    if (e.status != QCD_ERR_OOM) throw;
+    return false;
+  }
+  if (!g->fx_ok) return false;
+  static std::atomic<unsigned long long> attr_mask{0};
+  if (first_use_on_device(attr_mask))
+    QCD_CK(cudaFuncSetAttribute(k_hop_fx_canon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared)));
+  const Geom geom = make_geom(g->lat.L, g->lat.bc, g->lat.V, g->lat.Vh);
+  const unsigned nb = (unsigned)((shape.Vh + kWarps * kSB - 1) / (kWarps * kSB)), n = (unsigned)nrhs;
+  const double2 *src = (const double2*)in;
+  const bool full = op == QCD_OP_FULL || op == QCD_OP_FULL_DAG, mhat = op == QCD_OP_MHAT || op == QCD_OP_MHAT_DAG;
+  const int dagger = op == QCD_OP_FULL_DAG || op == QCD_OP_MHAT_DAG;
+  FxOrder order(g, st);
+  // fixed-point halves: both for FULL (even in fa, odd in fb), else the one that the operator reads, in fa
+  const int p0 = full || mhat || op == QCD_OP_D_OE ? 0 : 1;
+  launch_k(k_canon_to_fx, dim3((unsigned)((shape.Vh + 127) / 128), n, full ? 2 : 1), 128, 0, st, geom, src,
+           fa, full ? fb : fa, p0);
+  QCD_LAUNCH_CK();
+  auto hop = [&](const FxField& from, int out_parity, double a, bool xpay, bool zero) {
+    HA A;
+    fx_args(A, g, shape, out_parity, dagger, a);
+    A.stop = nullptr;
+    A.xpay = xpay;
+    launch_k(k_hop_fx_canon, nb * n, 32 * kWarps, sizeof(FxShared), st, A, (const int4*)g->Ufx, from, src,
+             (double2*)out, (int)zero);
+    QCD_LAUNCH_CK();
+  };
+  if (full) {
+    hop(fb, 0, -f.kappa, true, false);
+    hop(fa, 1, -f.kappa, true, false);
+  } else if (mhat) {
+    fx_launch(g, fa, shape, nullptr, &fb, 1, dagger, 1.0, nullptr, st, nullptr, nullptr);
+    hop(fb, 0, -f.kappa * f.kappa, true, true);
+  } else {
+    hop(fa, op == QCD_OP_D_OE, 1.0, false, true);
+  }
+  order.done();
+  return true;
 }
 
 }  // namespace qcd
