@@ -28,6 +28,7 @@ struct ColCoef {
   R pre_d, pre_e, post_d, post_e;
   R ainv, ratio;   // 1 / alpha, beta / alpha
   R apow[kMaxLs];  // beta^k alpha^(-1-k) / den
+  R row0[kMaxLs];  // alpha times row 0 of the inverse: 1 / den, then -m beta^k alpha^-k / den, k = Ls - t
 };
 
 // (d + e T) in place on one column of Ls complex values (stride cs), T = T_lo or T_up
@@ -153,6 +154,77 @@ __device__ __forceinline__ void col_inv_reg(R* re, R* im, int cs, const ColCoef<
   }
 }
 
+// ----------------------------------------------------------------------------- columns in registers
+// The passes of a column operator on several columns of one chirality at once, held in registers from the
+// first slice to the last (Ls <= NR): V is a spin pair of FP32 (complex, or its real or imaginary parts
+// alone) or a complex FP64.  In the order t = s (lower shift) or Ls - 1 - s (upper) both shifts are the same recurrence:
+//   (d + e T): v_t = d x_t + e x_(t-1), x_(-1) = -m x_(Ls-1);
+//   (alpha - beta T)^-1: alpha psi_0 = row0 . x, alpha psi_t = x_t + (beta / alpha) (alpha psi_(t-1)),
+// two multiply-adds per value; the factor 1 / alpha is left to the caller (unit(), in its own scale factor).
+__device__ __forceinline__ P2 vfma(float a, const P2& x, const P2& y) {
+  const float2 b = make_float2(a, a);
+  return {__ffma2_rn(b, x.re, y.re), __ffma2_rn(b, x.im, y.im)};
+}
+__device__ __forceinline__ P2 vmul(float a, const P2& x) {
+  const float2 b = make_float2(a, a);
+  return {__fmul2_rn(b, x.re), __fmul2_rn(b, x.im)};
+}
+__device__ __forceinline__ float2 vfma(float a, float2 x, float2 y) { return __ffma2_rn(make_float2(a, a), x, y); }
+__device__ __forceinline__ float2 vmul(float a, float2 x) { return __fmul2_rn(make_float2(a, a), x); }
+__device__ __forceinline__ Cx<double> vfma(double a, const Cx<double>& x, const Cx<double>& y) {
+  return {fma(a, x.re, y.re), fma(a, x.im, y.im)};
+}
+__device__ __forceinline__ Cx<double> vmul(double a, const Cx<double>& x) { return {a * x.re, a * x.im}; }
+
+// v[t], t < Ls, in the order above; last = v[Ls - 1]
+template <int NR, typename R, typename V>
+__device__ __forceinline__ void col_reg(V (&v)[NR], V last, const ColCoef<R>& c, int dagger) {
+  const int Ls = c.Ls;
+  const bool first = dagger ? (c.flags & kPost) : (c.flags & kPre);
+  const bool then = dagger ? (c.flags & kPre) : (c.flags & kPost);
+  if (first) {
+    const R d = dagger ? c.post_d : c.pre_d, e = dagger ? c.post_e : c.pre_e;
+    V prev = vmul(-c.mf, last);
+#pragma unroll
+    for (int t = 0; t < NR; ++t)
+      if (t < Ls) {
+        const V x = v[t];
+        last = v[t] = vfma(e, prev, vmul(d, x));
+        prev = x;
+      }
+  }
+  if (c.flags & kInv) {
+    V p = vmul(c.row0[0], v[0]);
+#pragma unroll
+    for (int t = 1; t < NR; ++t)
+      if (t < Ls) p = vfma(c.row0[t], v[t], p);
+    v[0] = p;
+#pragma unroll
+    for (int t = 1; t < NR; ++t)
+      if (t < Ls) {
+        p = vfma(c.ratio, p, v[t]);
+        v[t] = p;
+      }
+    last = p;
+  }
+  if (then) {
+    const R d = dagger ? c.pre_d : c.post_d, e = dagger ? c.pre_e : c.post_e;
+    V prev = vmul(-c.mf, last);
+#pragma unroll
+    for (int t = 0; t < NR; ++t)
+      if (t < Ls) {
+        const V x = v[t];
+        v[t] = vfma(e, prev, vmul(d, x));
+        prev = x;
+      }
+  }
+}
+// the factor that col_reg leaves out
+template <typename R>
+__device__ __forceinline__ R col_unit(const ColCoef<R>& c) {
+  return (c.flags & kInv) ? c.ainv : R(1);
+}
+
 // host description of a column operator
 struct ColSpec {
   int flags = 0;
@@ -177,6 +249,10 @@ inline ColCoef<R> make_coef(const DwParams& p, const ColSpec& cs) {
   double w = 1.0 / (cs.alpha * den);
   for (int k = 0; k < p.Ls; ++k) {
     c.apow[k] = (R)w;
+    if (k)
+      c.row0[p.Ls - k] = (R)(-p.mf * w * cs.alpha);
+    else
+      c.row0[0] = (R)(w * cs.alpha);
     w *= ratio;
   }
   return c;

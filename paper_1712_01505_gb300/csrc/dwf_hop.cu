@@ -30,16 +30,20 @@ using namespace dwcol;
 constexpr int kFusedMaxLs = 32;  // tile of 32 sites x Ls slices x 96 B within 96 KB
 
 // PK = 1: the hop with packed FP32x2 arithmetic (stencil.cuh); PK = 2: the same
-// with the links staged as two rows
+// with the links staged as two rows.  The registers are bounded for 24 warps per SM: with the columns of the
+// inverse in registers (one read and one write of the tile; up to Ls = 16) the kernel would take 99 and run
+// 101 us instead of 84 (16^3 x 32 x 16, Mobius adjoint, FP32; 88 with two reads and a write of scalars).
 template <int P, int RECON, int BY, int PK>
-__global__ void __launch_bounds__(32 * BY) k_dw_hop_w(HopArgs<P, RECON> A, ColCoef<float> c) {
+__global__ void __launch_bounds__(32 * BY, 24 / BY) k_dw_hop_w(HopArgs<P, RECON> A, ColCoef<float> c) {
   pdl_enter();
   using R = typename MathType<P>::type;
   static_assert(sizeof(R) == 4, "the fused stencil computes in FP32");
   if (A.stop && *A.stop) return;
   extern __shared__ __align__(16) unsigned char smraw[];
-  R* tile = reinterpret_cast<R*>(smraw);
-  constexpr int cs = 24 * 32;  // stride between slices of the tile
+  // [s][2 * pair + im][32 sites]: the real or imaginary parts of a spin pair in one 8-byte access (whole complex
+  // pairs take the column phase to 154 registers; 24 resident warps need 80)
+  float2* tile = reinterpret_cast<float2*>(smraw);
+  constexpr int cs = 12 * 32;  // stride between slices of the tile
   const int tx = threadIdx.x, ty = threadIdx.y;
   const int r = blockIdx.y;
   const int cb = blockIdx.x * 32 + tx;
@@ -70,14 +74,10 @@ __global__ void __launch_bounds__(32 * BY) k_dw_hop_w(HopArgs<P, RECON> A, ColCo
         hop_link_smp<P, RECON, 6>(A, sm, tx, sg, in, soff, acc);
         hop_link_smp<P, RECON, 7>(A, sm, tx, sg, in, soff, acc);
       }
-      // spin pair q: canonical components b (lane x) and b + 3 (lane y)
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
-        const int b = q < 3 ? q : q + 3;
-        tile[s * cs + (2 * b) * 32 + tx] = acc[q].re.x;
-        tile[s * cs + (2 * b + 1) * 32 + tx] = acc[q].im.x;
-        tile[s * cs + (2 * (b + 3)) * 32 + tx] = acc[q].re.y;
-        tile[s * cs + (2 * (b + 3) + 1) * 32 + tx] = acc[q].im.y;
+        tile[s * cs + 2 * q * 32 + tx] = acc[q].re;
+        tile[s * cs + (2 * q + 1) * 32 + tx] = acc[q].im;
       }
     }
   } else {
@@ -101,39 +101,54 @@ __global__ void __launch_bounds__(32 * BY) k_dw_hop_w(HopArgs<P, RECON> A, ColCo
         hop_link_sm<P, RECON, 1, 7>(A, sm, tx, sg, in, soff, 1, acc);
       }
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        tile[s * cs + (2 * k) * 32 + tx] = acc[0][k].re;
-        tile[s * cs + (2 * k + 1) * 32 + tx] = acc[0][k].im;
+      for (int q = 0; q < 6; ++q) {  // spin pair q: canonical components b and b + 3
+        const int b = q < 3 ? q : q + 3;
+        tile[s * cs + 2 * q * 32 + tx] = make_float2(acc[0][b].re, acc[0][b + 3].re);
+        tile[s * cs + (2 * q + 1) * 32 + tx] = make_float2(acc[0][b].im, acc[0][b + 3].im);
       }
     }
   }
   __syncthreads();
-  for (int k = ty; k < 12; k += BY)
-    if (Ls <= 16)  // the column of the inverse in registers
-      col_apply<R, 16>(tile + (2 * k) * 32 + tx, tile + (2 * k + 1) * 32 + tx, cs, c, (k < 6) != (A.dagger != 0),
-                       A.dagger);
-    else
-      col_apply(tile + (2 * k) * 32 + tx, tile + (2 * k + 1) * 32 + tx, cs, c, (k < 6) != (A.dagger != 0), A.dagger);
+  R unit = R(1);
+  if (Ls <= 16) {  // the columns in registers
+    unit = col_unit(c);
+    for (int k = ty; k < 12; k += BY) {
+      const bool lower = (k < 6) != (A.dagger != 0);
+      float2* p = tile + (lower ? 0 : Ls - 1) * cs + k * 32 + tx;
+      const int ds = lower ? cs : -cs;
+      float2 v[16];
+#pragma unroll
+      for (int t = 0; t < 16; ++t)
+        if (t < Ls) v[t] = p[t * ds];
+      col_reg<16>(v, p[(Ls - 1) * ds], c, A.dagger);
+#pragma unroll
+      for (int t = 0; t < 16; ++t)
+        if (t < Ls) p[t * ds] = v[t];
+    }
+  } else {
+    for (int k = ty; k < 12; k += BY) {
+      const int q = k < 6 ? k % 3 : 3 + k % 3, lane = (k / 3) & 1;  // spin (k / 3) is lane a or b of its pair
+      R* re = reinterpret_cast<R*>(tile + 2 * q * 32 + tx) + lane;
+      col_apply(re, re + 2 * 32, 2 * cs, c, (k < 6) != (A.dagger != 0), A.dagger);
+    }
+  }
   __syncthreads();
   if (!valid) return;
-  const R a = (R)A.a;
+  const float2 a2 = bc2((R)A.a * unit);
   const SpinorView<P> out = A.out.offset_rhs(r);
   for (int s = ty; s < Ls; s += BY) {
     const long site = (long)s * A.g.Vh + cb;
-    Cx<R> o[12];
-    if (A.xpay) {
-      A.x.offset_rhs(r).load(site, o);
+    P2 o[6];
+    if (A.xpay) A.x.offset_rhs(r).load_p(site, o);
 #pragma unroll
-      for (int k = 0; k < 12; ++k) {
-        o[k].re = fma(a, tile[s * cs + (2 * k) * 32 + tx], o[k].re);
-        o[k].im = fma(a, tile[s * cs + (2 * k + 1) * 32 + tx], o[k].im);
-      }
-    } else {
-#pragma unroll
-      for (int k = 0; k < 12; ++k)
-        o[k] = {a * tile[s * cs + (2 * k) * 32 + tx], a * tile[s * cs + (2 * k + 1) * 32 + tx]};
+    for (int q = 0; q < 6; ++q) {
+      const float2 re = tile[s * cs + 2 * q * 32 + tx], im = tile[s * cs + (2 * q + 1) * 32 + tx];
+      if (A.xpay)
+        o[q] = {fma2(a2, re, o[q].re), fma2(a2, im, o[q].im)};
+      else
+        o[q] = {__fmul2_rn(a2, re), __fmul2_rn(a2, im)};
     }
-    out.store(site, o);
+    out.store_p(site, o);
   }
 }
 
