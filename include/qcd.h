@@ -143,8 +143,8 @@ typedef struct {
  *   recomputed and solution accumulated in the outer precision, below).
  * delta: a reliable update is made when the iterated residual has dropped by
  *   this factor since the last one (0 < delta < 1; 0 selects 0.01).
- * use_graph: capture `graph_chunk` inner iterations in one CUDA graph and
- *   check convergence once per graph launch (0 = plain launches).
+ * use_graph: capture up to `graph_chunk` inner iterations in one CUDA graph
+ *   and check convergence once per predicted stop (0 = plain launches).
  * x0_given: x holds an initial guess on entry (warm start).
  * dagger: solve with the adjoint operator (A^dag x = b); Wilson only.
  * outer: precision of the operator applications of the outer steps of a

@@ -699,31 +699,40 @@ struct Solver {
     return std::string(buf) + " x" + std::to_string((uintptr_t)xin.data);
   }
 
-  void run_chunk(int k, bool graph) {
-    if (graph) {
-      std::string key = graph_key(k);
-      auto it = g->graphs.find(key);
-      if (it == g->graphs.end()) {
-        cudaGraph_t gr;
-        long c0 = launches_so_far();
-        QCD_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
-        k_reset<<<1, 1, 0, st>>>(ctl);
-        QCD_LAUNCH_CK();
-        for (int i = 0; i < k; ++i) body();
-        QCD_CK(cudaStreamEndCapture(st, &gr));
-        CachedGraph cg;
-        cg.nodes = launches_so_far() - c0;  // captured, not yet executed
-        set_launches(c0);
-        QCD_CK(cudaGraphInstantiate(&cg.exec, gr, 0));
-        cudaGraphDestroy(gr);
-        it = g->graphs.emplace(key, cg).first;
-      }
-      QCD_CK(cudaGraphLaunch(it->second.exec, st));
-      note_launches(it->second.nodes);
-    } else {
-      k_reset<<<1, 1, 0, st>>>(ctl);
-      QCD_LAUNCH_CK();
+  // one graph of k iterations, built on first use
+  void launch_graph(int k) {
+    std::string key = graph_key(k);
+    auto it = g->graphs.find(key);
+    if (it == g->graphs.end()) {
+      cudaGraph_t gr;
+      long c0 = launches_so_far();
+      QCD_CK(cudaStreamBeginCapture(st, cudaStreamCaptureModeThreadLocal));
       for (int i = 0; i < k; ++i) body();
+      QCD_CK(cudaStreamEndCapture(st, &gr));
+      CachedGraph cg;
+      cg.nodes = launches_so_far() - c0;  // captured, not yet executed
+      set_launches(c0);
+      QCD_CK(cudaGraphInstantiate(&cg.exec, gr, 0));
+      cudaGraphDestroy(gr);
+      it = g->graphs.emplace(key, cg).first;
+    }
+    QCD_CK(cudaGraphLaunch(it->second.exec, st));
+    note_launches(it->second.nodes);
+  }
+
+  // k iterations (in graphs of `chunk`, 8 and 2, hence up to one more); those after
+  // a raised stop word do nothing
+  void run_iterations(int k, bool graph, int chunk) {
+    k_reset<<<1, 1, 0, st>>>(ctl);
+    QCD_LAUNCH_CK();
+    if (!graph) {
+      for (int i = 0; i < k; ++i) body();
+      return;
+    }
+    while (k > 0) {
+      const int n = k >= chunk ? chunk : (k >= 8 && chunk >= 8 ? 8 : std::min(2, chunk));
+      launch_graph(n);
+      k -= n;
     }
   }
 
@@ -1179,11 +1188,29 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   const int chunk = graph ? (prm.graph_chunk > 0 ? prm.graph_chunk : 32) : 16;
   bool first = true;
   int done_reason = QCD_OK;
-  // Chunk length: the iterations between two outer steps are nearly constant
-  // (each removes the same factor delta), so after the first gap has been seen
-  // a chunk stops short of the expected next outer step and the last few
-  // iterations run in chunks of 8 / 2: few launches are wasted after a stop.
-  int last_stop = 0, gap = 0;
+  // How many iterations to launch before the host looks again: as many as the
+  // residual's rate so far predicts up to the next stop, and one.  A launch after
+  // the stop does nothing but costs about 1 us, a look about 15 us of an idle GPU.
+  // Against chunks of 32 up to the first stop and of 8 / 2 towards the later ones
+  // (up to 20 wasted iterations and two more looks per outer step): FP32 with FP64
+  // outer steps, 8^3 x 16 2160 -> 1974 us, 24^3 x 48 FP16 14.7 -> 14.2 ms,
+  // 32^3 x 64 49.5 -> 48.8 ms; a solve without outer steps does not change.
+  std::vector<double> rate(nrhs, 0.0);  // mean decrease of ln |r|^2 per iteration since a restart
+  std::vector<int> start(nrhs, 0);      // iterations at that restart
+  auto look_ahead = [&] {
+    double n = 1e9;
+    for (int r = 0; r < nrhs; ++r) {
+      if (conv[r]) continue;
+      const Scal& s = S.hsc[r];
+      const int done = s.iters - start[r];
+      if (done >= 4 && s.r2 > 0.0 && s.r2 < s.r2_ref) rate[r] = std::log(s.r2_ref / s.r2) / done;
+      const double target = std::max(s.stop2, s.delta2 * s.r2_ref);
+      double m = 8.0;  // nothing known yet
+      if (rate[r] > 0.0 && target > 0.0 && s.r2 > 0.0) m = std::ceil(std::log(s.r2 / target) / rate[r]) + 1.0;
+      n = std::min(n, m);
+    }
+    return (int)std::min(64.0, std::max(2.0, n));
+  };
   // x64 of a right-hand side changed since its last true_residual (plain FP64 solves)
   std::vector<char> stale(nrhs, 0);
   // run `fn(r0, n)` over the maximal runs of consecutive right-hand sides with sel[r]
@@ -1207,19 +1234,15 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       done_reason = QCD_ERR_NOCONV;
       break;
     }
-    int k = chunk;
-    if (gap > 0) {
-      int remaining = last_stop + gap - maxit;
-      k = remaining >= chunk ? chunk : (remaining >= 8 && chunk >= 8 ? 8 : std::min(2, chunk));
-    }
-    const bool capped = k > maxiter - maxit;
-    if (capped) k = maxiter - maxit;
+    int k = look_ahead();
+    const bool capped = k + 2 > maxiter - maxit;  // graphs may hold up to one iteration more than k
+    if (capped) k = std::min(k, maxiter - maxit);
     // the first iteration runs un-captured so that the stencil tuner can time
     if (first) {
-      S.run_chunk(1, false);
+      S.run_iterations(1, false, chunk);
       first = false;
     } else {
-      S.run_chunk(k, graph && !capped);
+      S.run_iterations(k, graph && !capped, chunk);
     }
     // a plain FP64 solve iterates on x64 itself: the outer step's x_o and residual are stale
     if (S.inner == QCD_F64)
@@ -1234,13 +1257,6 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       any = any || due[r];
     }
     if (!any) continue;
-    {
-      int now = 0;
-      for (int r = 0; r < nrhs; ++r)
-        if (!conv[r]) now = std::max(now, S.hsc[r].iters);
-      if (now > last_stop) gap = now - last_stop;
-      last_stop = now;
-    }
     std::vector<char> full(nrhs, 0);
     for (int r = 0; r < nrhs; ++r) {
       if (!due[r]) continue;
@@ -1289,6 +1305,13 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       }
     }
     if (nactive == 0) break;
+    for (int r = 0; r < nrhs; ++r)
+      if (again[r] || again_full[r]) {
+        const Scal& s = S.hsc[r];
+        const int done = s.iters - start[r];
+        if (done >= 4 && s.r2 > 0.0 && s.r2 < s.r2_ref) rate[r] = std::log(s.r2_ref / s.r2) / done;
+        start[r] = s.iters;
+      }
     for_runs(again, [&](int r0, int n) { restart_from_residual(false, r0, n, fxo); });
     for_runs(again_full, [&](int r0, int n) { restart_from_residual(true, r0, n); });
     S.upload();
