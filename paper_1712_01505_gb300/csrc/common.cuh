@@ -577,26 +577,66 @@ __device__ __forceinline__ void canon_store(CanonWarp& w, double2* canon, long b
 }
 
 // ----------------------------------------------------------------------------- block reduction
-// Sum NR doubles over the block (warp shuffles, then shared memory); the
-// result is valid in thread 0.  Deterministic for a fixed block size.
+// An FP64 instruction of a warp holds the SM's FP64 unit for about 19 cycles, so
+// what a sum costs is its warp-level additions: five shuffle steps per value in
+// each of 8 warps and a last round come to 135 for three values (1.3 us per
+// block, and the blocks of an SM take turns).  Here the sums of the lanes across
+// the warps come first, in one warp (21), and the shuffles carry several values
+// at once (6).  With the partials of a kernel's prologue summed by one warp, one
+// division per block and the scalars loaded together (solver.cu): solves of
+// 8^3 x 16 in FP32 1974 -> 1833 us, 24^3 x 48 in FP16 14.2 -> 13.7 ms, twelve
+// right-hand sides there 149 -> 141 ms, domain-wall 16^3 x 32 x 16 173 -> 169 ms.
+
+// v[0 .. NR) summed over the warp (all lanes call it); the result is valid in
+// lane 0.  A step that halves the number of values a lane holds costs half the additions.
+template <int NR>
+__device__ __forceinline__ void warp_sum(double v[NR]) {
+  static_assert(NR >= 1 && NR <= 4, "warp_sum takes up to four values");
+  constexpr unsigned all = 0xffffffffu;
+  const int lane = threadIdx.x & 31;
+  if constexpr (NR == 1) {
+#pragma unroll
+    for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_down_sync(all, v[0], o);
+  } else {
+    const bool h1 = lane & 16, h2 = lane & 8;
+    double a = h1 ? v[1] : v[0];  // NR = 2: values 0 | 1 in the lower | upper half
+    a += __shfl_xor_sync(all, h1 ? v[0] : v[1], 16);
+    if constexpr (NR > 2) {  // and 2 | 3, then the four values one per group of 8 lanes: 0, 2, 1, 3
+      const double v3 = NR > 3 ? v[NR - 1] : 0.0;
+      double b = h1 ? v3 : v[2];
+      b += __shfl_xor_sync(all, h1 ? v[2] : v3, 16);
+      const double send = h2 ? a : b;
+      a = h2 ? b : a;
+      a += __shfl_xor_sync(all, send, 8);
+    } else {
+      a += __shfl_xor_sync(all, a, 8);
+    }
+#pragma unroll
+    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
+    v[0] = a;
+    v[1] = __shfl_sync(all, a, 16);
+    if constexpr (NR > 2) v[2] = __shfl_sync(all, a, 8);
+    if constexpr (NR > 3) v[3] = __shfl_sync(all, a, 24);
+  }
+}
+
+// Sum NR doubles over the block (whole warps, at most 8); the result is valid in
+// thread 0.  Deterministic for a fixed block size.
 template <int NR>
 __device__ __forceinline__ void block_sum(double v[NR]) {
-  __shared__ double sh[32][NR];
-  int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
+  __shared__ double sh[7][NR][32];
+  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5, nw = blockDim.x >> 5;
+  if (warp > 0)
 #pragma unroll
-  for (int k = 0; k < NR; ++k)
-    for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
-  if (lane == 0)
-#pragma unroll
-    for (int k = 0; k < NR; ++k) sh[warp][k] = v[k];
+    for (int k = 0; k < NR; ++k) sh[warp - 1][k][lane] = v[k];
   __syncthreads();
-  int nw = (blockDim.x + 31) >> 5;
   if (warp == 0) {
 #pragma unroll
-    for (int k = 0; k < NR; ++k) v[k] = (lane < nw) ? sh[lane][k] : 0.0;
+    for (int w = 0; w < 7; ++w)
+      if (w < nw - 1)
 #pragma unroll
-    for (int k = 0; k < NR; ++k)
-      for (int o = 16; o > 0; o >>= 1) v[k] += __shfl_down_sync(0xffffffffu, v[k], o);
+        for (int k = 0; k < NR; ++k) v[k] += sh[w][k][lane];
+    warp_sum<NR>(v);
   }
   __syncthreads();
 }

@@ -1,5 +1,6 @@
 // Host-side internals of libqcd shared between translation units.
 #pragma once
+#include <algorithm>
 #include <atomic>
 #include <cuda_runtime.h>
 
@@ -162,9 +163,9 @@ void zero_parity_canon(const Lattice& lat, int parity, double* canon, int nvec, 
 // in order into gpartial[group * 4 + k]; *npartial receives the number of groups.
 // Several slices (FP32: right-hand sides, domain-wall slices): every warp (32
 // sites of one slice q) writes partial[(q * ceil(Vh/32) + site block) * 4 + k]
-// and a second kernel sums each slice in order into gpartial[q * 4 + k]: the ls
-// slice sums of right-hand side r are gpartial[(r * ls + s) * 4 + k] (counters
-// and npartial unused).
+// and a second kernel sums each slice in order into G = red_row_groups(ls, Vh)
+// sums gpartial[(q * G + g) * 4 + k]: those of right-hand side r are the ls * G
+// from gpartial[r * ls * G * 4] on (counters and npartial unused).
 struct RedSpec {
   int mode;
   const Field* rt;
@@ -173,6 +174,13 @@ struct RedSpec {
   int* counters;
   int* npartial;
 };
+// groups of a slice's per-warp partials: one block sums a group, and one block's FP64
+// unit takes 10 us for the 10368 x 3 of 24^3 x 48, so they are spread over up to 16, of
+// 128 partials at least, as long as a right-hand side keeps to 64 sums
+inline int red_row_groups(int ls, long Vh) {
+  const long nsb = (Vh + 31) / 32;
+  return (int)std::max(1L, std::min({16L, 64L / std::max(ls, 1), nsb / 128L}));
+}
 void hop(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int dagger, double a,
          const Field* x, cudaStream_t st, const int* stop = nullptr, bool allow_tuning = true,
          const RedSpec* red = nullptr);

@@ -61,28 +61,35 @@ struct Scal {
 constexpr int kThreads = 256;
 constexpr int kMaxPartial = 4;
 
-__device__ __forceinline__ double2 cdiv(double2 a, double2 b) {
-  double d = b.x * b.x + b.y * b.y;
-  return make_double2((a.x * b.x + a.y * b.y) / d, (a.y * b.x - a.x * b.y) / d);
-}
 __device__ __forceinline__ double2 cmul2(double2 a, double2 b) {
   return make_double2(a.x * b.x - a.y * b.y, a.x * b.y + a.y * b.x);
 }
 __device__ __forceinline__ bool bad(double v) { return !isfinite(v); }
 
 // ----------------------------------------------------------------------------- partial sums
-// Sum the per-block partials of one right-hand side (one block per rhs).
+// Sum the partials of one right-hand side; the result is valid in the first warp.
+// Up to kWarpPartials of them are summed by that warp alone: a block's 8 warps
+// would add zeros most of the time, and FP64 additions are what the sum costs.
+constexpr int kWarpPartials = 256;
 template <int NR>
-__device__ void sum_partials(const double* partial, int nblk, int r, double out[NR]) {
+__device__ __forceinline__ void sum_partials(const double* partial, int nblk, int r, double out[NR]) {
   double v[NR];
 #pragma unroll
   for (int k = 0; k < NR; ++k) v[k] = 0.0;
-  for (int b = threadIdx.x; b < nblk; b += blockDim.x)
+  const bool one_warp = nblk <= kWarpPartials;
+  if (!one_warp || threadIdx.x < 32) {
+    const int step = one_warp ? 32 : blockDim.x;
+#pragma unroll 4
+    for (int b = threadIdx.x; b < nblk; b += step)
 #pragma unroll
-    for (int k = 0; k < NR; ++k) v[k] += partial[((long)r * nblk + b) * kMaxPartial + k];
-  block_sum<NR>(v);
+      for (int k = 0; k < NR; ++k) v[k] += partial[((long)r * nblk + b) * kMaxPartial + k];
+  }
+  if (!one_warp)
+    block_sum<NR>(v);
+  else if (threadIdx.x < 32)
+    warp_sum<NR>(v);
 #pragma unroll
-  for (int k = 0; k < NR; ++k) out[k] = v[k];
+  for (int k = 0; k < NR; ++k) out[k] = threadIdx.x < 32 ? __shfl_sync(0xffffffffu, v[k], 0) : 0.0;
 }
 
 template <int NR>
@@ -94,6 +101,21 @@ __device__ __forceinline__ void write_partial(double v[NR], double* partial, int
 }
 
 #define STOPPED(ctl) (*(ctl) != 0)
+
+// Loads that stay where they are written.  The iteration kernels ask for the stop
+// word and every scalar they need at once: one L2 latency (about 0.4 us) instead of
+// one per test, which counts when a kernel takes 3 us.
+__device__ __forceinline__ int ld_now(const int* p) {
+  int v;
+  asm volatile("ld.global.b32 %0, [%1];" : "=r"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double ld_now(const double* p) {
+  double v;
+  asm volatile("ld.global.f64 %0, [%1];" : "=d"(v) : "l"(p) : "memory");
+  return v;
+}
+__device__ __forceinline__ double2 ld_now2(const double* p) { return make_double2(ld_now(p), ld_now(p + 1)); }
 
 // Loads and stores of the solver's vectors: PV >= 0 fixes the storage precision
 // at compile time (the iteration kernels, which the host instantiates for the
@@ -128,11 +150,12 @@ __host__ __device__ constexpr int x_prec() {
 template <typename R, int PV = -1>
 __global__ void k_bicg_p(AnyView r_, AnyView p_, AnyView v_, long n, Scal* sc, const int* ctl) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.y;
   Scal& s = sc[r];
-  if (!s.active) return;
-  const Cx<R> be = {(R)s.beta[0], (R)s.beta[1]}, om = {(R)s.omega[0], (R)s.omega[1]};
+  const int stop = ld_now(ctl), active = ld_now(&s.active);
+  const double2 be2 = ld_now2(s.beta), om2 = ld_now2(s.omega);
+  if (stop || !active) return;
+  const Cx<R> be = {(R)be2.x, (R)be2.y}, om = {(R)om2.x, (R)om2.y};
   if (blockIdx.x == 0 && threadIdx.x == 0) {  // no block of this kernel reads rho
     s.rho[0] = s.rho_new[0];
     s.rho[1] = s.rho_new[1];
@@ -179,65 +202,78 @@ __global__ void k_cdot(AnyView a_, AnyView b_, long n, double* partial, const Sc
 // This saves a one-block kernel and its launch gap per scalar.
 // nb_dev (may be null): number of partials written by a stencil with a fused reduction.
 
+// The division is made once per block with a lane for each component (a warp's FP64
+// instruction costs the same for one lane as for all).
+
+// component `lane` (0: real part, else imaginary part) of a / b
+__device__ __forceinline__ double cdiv_part(double2 a, double2 b, int lane) {
+  const double p = lane ? a.y : a.x, q = lane ? -a.x : a.y;
+  return (p * b.x + q * b.y) / (b.x * b.x + b.y * b.y);
+}
+
 // alpha = rho / (rt, v); false (for every block) on NaN or breakdown
-__device__ __forceinline__ bool block_alpha(Scal& s, const double* partial, int nb, int r, int* ctl,
+__device__ __forceinline__ bool block_alpha(Scal& s, double2 rho, const double* partial, int nb, int r, int* ctl,
                                             double2* al) {
-  __shared__ double2 sh;
+  __shared__ double sh[2];
   __shared__ int ok;
   double d[2];
   sum_partials<2>(partial, nb, r, d);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 2) {
     const double2 rv = make_double2(d[0], d[1]);
-    const double2 rho = make_double2(s.rho[0], s.rho[1]);
-    const double mag = sqrt(rv.x * rv.x + rv.y * rv.y);
+    // |rv| <= 1e-300 or |rv| < 1e-24 |rho|: the square roots only where the larger components leave it open
+    const double mv = fmax(fabs(rv.x), fabs(rv.y)), mr = fmax(fabs(rho.x), fabs(rho.y));
     int flag = FLAG_NONE;
-    if (bad(rv.x) || bad(rv.y))
+    if (bad(rv.x) || bad(rv.y)) {
       flag = FLAG_NAN;
-    else if (mag <= 1e-300 || mag < 1e-24 * sqrt(rho.x * rho.x + rho.y * rho.y))
-      flag = FLAG_BREAKDOWN;
-    ok = flag == FLAG_NONE;
-    if (ok) sh = cdiv(rho, rv);
+    } else if (!(mv > 1e-299 && mv > 2e-24 * mr)) {
+      const double mag = sqrt(rv.x * rv.x + rv.y * rv.y);
+      if (mag <= 1e-300 || mag < 1e-24 * sqrt(rho.x * rho.x + rho.y * rho.y)) flag = FLAG_BREAKDOWN;
+    }
+    const bool fine = flag == FLAG_NONE;
+    const double q = fine ? cdiv_part(rho, rv, threadIdx.x) : 0.0;
+    sh[threadIdx.x] = q;
+    if (threadIdx.x == 0) ok = fine;
     if (blockIdx.x == 0) {
-      if (ok) {
-        s.alpha[0] = sh.x;
-        s.alpha[1] = sh.y;
-      } else {
+      if (fine) {
+        s.alpha[threadIdx.x] = q;
+      } else if (threadIdx.x == 0) {
         s.flag = flag;
         *ctl = 1;
       }
     }
   }
   __syncthreads();
-  *al = sh;
+  *al = make_double2(sh[0], sh[1]);
   return ok;
 }
 
 // omega = (t, s) / (t, t); false (for every block) on NaN or t = 0
 __device__ __forceinline__ bool block_omega(Scal& s, const double* partial, int nb, int r, int* ctl,
                                             double2* om) {
-  __shared__ double2 sh;
+  __shared__ double sh[2];
   __shared__ int ok;
   double d[3];
   sum_partials<3>(partial, nb, r, d);
-  if (threadIdx.x == 0) {
+  if (threadIdx.x < 2) {
     int flag = FLAG_NONE;
     if (bad(d[0]) || bad(d[1]) || bad(d[2]))
       flag = FLAG_NAN;
     else if (d[2] <= 0.0)  // t = 0: s is (numerically) zero or the operator annihilated it
       flag = FLAG_BREAKDOWN;
-    ok = flag == FLAG_NONE;
-    sh = ok ? make_double2(d[0] / d[2], d[1] / d[2]) : make_double2(0.0, 0.0);
+    const bool fine = flag == FLAG_NONE;
+    const double q = fine ? (threadIdx.x ? d[1] : d[0]) / d[2] : 0.0;
+    sh[threadIdx.x] = q;
+    if (threadIdx.x == 0) ok = fine;
     if (blockIdx.x == 0) {
-      s.omega[0] = sh.x;
-      s.omega[1] = sh.y;
-      if (!ok) {
+      s.omega[threadIdx.x] = q;
+      if (!fine && threadIdx.x == 0) {
         s.flag = flag;
         *ctl = 1;
       }
     }
   }
   __syncthreads();
-  *om = sh;
+  *om = make_double2(sh[0], sh[1]);
   return ok;
 }
 
@@ -246,12 +282,13 @@ template <typename R, int PV = -1>
 __global__ void k_bicg_s(AnyView r_, AnyView v_, AnyView s_, long n, Scal* sc, int* ctl, const double* partial,
                          int nblk, const int* nb_dev) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.y;
   Scal& s = sc[r];
-  if (!s.active) return;
+  const int stop = ld_now(ctl), active = ld_now(&s.active), nb = nb_dev ? ld_now(nb_dev) : nblk;
+  const double2 rho = ld_now2(s.rho);
+  if (stop || !active) return;
   double2 a;
-  if (!block_alpha(s, partial, nb_dev ? *nb_dev : nblk, r, ctl, &a)) return;
+  if (!block_alpha(s, rho, partial, nb, r, ctl, &a)) return;
   const Cx<R> al = {(R)a.x, (R)a.y};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     Cx<R> vr[12], vv[12];
@@ -296,14 +333,15 @@ __global__ void k_bicg_xr(AnyView x_, AnyView p_, AnyView s_, AnyView t_, AnyVie
                           long n, const double* partial_in, int nblk, const int* nb_dev, double* partial_out,
                           Scal* sc, int* ctl) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.y;
   Scal& s = sc[r];
-  if (!s.active) return;
+  const int stop = ld_now(ctl), active = ld_now(&s.active), nb = nb_dev ? ld_now(nb_dev) : nblk;
+  const double2 a = ld_now2(s.alpha);
+  if (stop || !active) return;
   double2 o;
-  if (!block_omega(s, partial_in, nb_dev ? *nb_dev : nblk, r, ctl, &o)) return;
-  const Cx<R> al = {(R)s.alpha[0], (R)s.alpha[1]}, om = {(R)o.x, (R)o.y};
-  const Cx<RX> alx = {(RX)s.alpha[0], (RX)s.alpha[1]}, omx = {(RX)o.x, (RX)o.y};
+  if (!block_omega(s, partial_in, nb, r, ctl, &o)) return;
+  const Cx<R> om = {(R)o.x, (R)o.y};
+  const Cx<RX> alx = {(RX)a.x, (RX)a.y}, omx = {(RX)o.x, (RX)o.y};
   double v[3] = {0.0, 0.0, 0.0};
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     // every input first: the stores below may alias nothing the compiler can prove
@@ -344,12 +382,23 @@ __global__ void k_bicg_xr(AnyView x_, AnyView p_, AnyView s_, AnyView t_, AnyVie
 // 49-53 iterations with a two-iteration wait, 46-49 without)
 __global__ void k_bicg_check(Scal* sc, const double* partial, int nblk, int* ctl, int decide) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.x;
   Scal& s = sc[r];
-  if (!s.active) return;
+  const int stop = ld_now(ctl), active = ld_now(&s.active);
+  const double2 rho = ld_now2(s.rho), alpha = ld_now2(s.alpha), omega = ld_now2(s.omega);
+  if (stop || !active) return;
   double d[3];
   sum_partials<3>(partial, nblk, r, d);
+  if (threadIdx.x >= 32) return;
+  // lanes 0, 1: rho_new / rho, lanes 2, 3: alpha / omega
+  const bool second = threadIdx.x & 2;
+  const double q = cdiv_part(second ? alpha : make_double2(d[0], d[1]), second ? omega : rho, threadIdx.x & 1);
+  double2 f[2];
+#pragma unroll
+  for (int j = 0; j < 2; ++j) {
+    f[j].x = __shfl_sync(0xffffffffu, q, 2 * j);
+    f[j].y = __shfl_sync(0xffffffffu, q, 2 * j + 1);
+  }
   if (threadIdx.x) return;
   s.iters += 1;
   s.rho_new[0] = d[0];
@@ -362,8 +411,7 @@ __global__ void k_bicg_check(Scal* sc, const double* partial, int nblk, int* ctl
   } else if (s.delta2 > 0.0 && d[2] <= s.delta2 * s.r2_ref) {
     s.flag = FLAG_UPDATE;
   }
-  const double2 b = cmul2(cdiv(make_double2(d[0], d[1]), make_double2(s.rho[0], s.rho[1])),
-                          cdiv(make_double2(s.alpha[0], s.alpha[1]), make_double2(s.omega[0], s.omega[1])));
+  const double2 b = cmul2(f[0], f[1]);
   s.beta[0] = b.x;
   s.beta[1] = b.y;
   if (decide && s.flag != FLAG_NONE) *ctl = 1;
@@ -378,11 +426,11 @@ __global__ void k_bicg_check(Scal* sc, const double* partial, int nblk, int* ctl
 template <typename R, int PV = -1>
 __global__ void k_cg_p(AnyView r_, AnyView p_, long n, Scal* sc, const int* ctl) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.y;
   Scal& s = sc[r];
-  if (!s.active) return;
-  const R be = (R)s.beta[0];
+  const int stop = ld_now(ctl), active = ld_now(&s.active);
+  const R be = (R)ld_now(s.beta);
+  if (stop || !active) return;
   if (blockIdx.x == 0 && threadIdx.x == 0) s.rr = s.rr_new;  // no block of this kernel reads rr
   for (long i = blockIdx.x * (long)blockDim.x + threadIdx.x; i < n; i += (long)gridDim.x * blockDim.x) {
     Cx<R> vr[12], vp[12];
@@ -396,16 +444,16 @@ __global__ void k_cg_p(AnyView r_, AnyView p_, long n, Scal* sc, const int* ctl)
 
 // alpha = rr / Re(p, q) from the k_rdot partials, formed by every block (see
 // block_alpha); false (for every block) on NaN or breakdown
-__device__ __forceinline__ bool block_cg_alpha(Scal& s, const double* partial, int nb, int r, int* ctl,
+__device__ __forceinline__ bool block_cg_alpha(Scal& s, double rr, const double* partial, int nb, int r, int* ctl,
                                                double* al) {
   __shared__ double sh;
   __shared__ int ok;
-  double d[2];
-  sum_partials<2>(partial, nb, r, d);
+  double d[1];
+  sum_partials<1>(partial, nb, r, d);
   if (threadIdx.x == 0) {
     const int flag = bad(d[0]) ? FLAG_NAN : (d[0] <= 0.0 ? FLAG_BREAKDOWN : FLAG_NONE);
     ok = flag == FLAG_NONE;
-    sh = ok ? s.rr / d[0] : 0.0;
+    sh = ok ? rr / d[0] : 0.0;
     if (blockIdx.x == 0) {
       if (ok) {
         s.alpha[0] = sh;
@@ -427,12 +475,13 @@ template <typename R, typename RX, int PV = -1>
 __global__ void k_cg_xr(AnyView x_, AnyView p_, AnyView q_, AnyView r_, long n, const double* partial_in,
                         int nblk, const int* nb_dev, double* partial_out, Scal* sc, int* ctl) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.y;
   Scal& s = sc[r];
-  if (!s.active) return;
+  const int stop = ld_now(ctl), active = ld_now(&s.active), nb = nb_dev ? ld_now(nb_dev) : nblk;
+  const double rr_old = ld_now(&s.rr);
+  if (stop || !active) return;
   double a;
-  if (!block_cg_alpha(s, partial_in, nb_dev ? *nb_dev : nblk, r, ctl, &a)) return;
+  if (!block_cg_alpha(s, rr_old, partial_in, nb, r, ctl, &a)) return;
   const R al = (R)a;
   const RX alx = (RX)a;
   double v[1] = {0.0};
@@ -462,10 +511,10 @@ __global__ void k_cg_xr(AnyView x_, AnyView p_, AnyView q_, AnyView r_, long n, 
 // end of an iteration: rr_new, flags and the next beta; decide as in k_bicg_check
 __global__ void k_cg_check(Scal* sc, const double* partial, int nblk, int* ctl, int decide) {
   pdl_enter();
-  if (STOPPED(ctl)) return;
   int r = blockIdx.x;
   Scal& s = sc[r];
-  if (!s.active) return;
+  const int stop = ld_now(ctl), active = ld_now(&s.active);
+  if (stop || !active) return;
   double d[1];
   sum_partials<1>(partial, nblk, r, d);
   if (threadIdx.x) return;
@@ -611,7 +660,7 @@ struct Solver {
   template <typename R, typename RX, int PV>
   void body_t(long nn, int dag) {
     if (bicg()) {
-      int nb_ts = 0;  // partials of (t, s), |t|^2 from k_ts_tt (the unfused path)
+      int nb_ts = 0;  // partials of (t, s), |t|^2 per right-hand side (one: counted by the stencil)
       launch_k(k_bicg_p<R, PV>, wave(k_bicg_p<R, PV>, nn), kThreads, 0, st, any_view(r), any_view(p), any_view(v),
                nn, sc, ctl);
       QCD_LAUNCH_CK();
@@ -626,12 +675,12 @@ struct Solver {
         QCD_LAUNCH_CK();
         apply_mhat(opin, s, t, dag, st, "in", ctl, &red2);
       } else if (fused_multi()) {
-        // per-rhs sums land in partial[rhs * 4 + k]: one partial per right-hand side
+        nb_ts = red_row_groups(ls, g->lat.Vh);  // those of (rt, v) as well (Wilson: ls = 1)
         RedSpec red1{1, &rt, bpartial, partial, nullptr, nullptr};
         RedSpec red2{2, nullptr, bpartial, partial, nullptr, nullptr};
         apply_mhat(opin, p, v, dag, st, "in", ctl, &red1);
         launch_k(k_bicg_s<R, PV>, wave(k_bicg_s<R, PV>, nn), kThreads, 0, st, any_view(r), any_view(v), any_view(s),
-                 nn, sc, ctl, partial, 1, nullptr);
+                 nn, sc, ctl, partial, nb_ts, nullptr);
         QCD_LAUNCH_CK();
         apply_mhat(opin, s, t, dag, st, "in", ctl, &red2);
       } else {
@@ -650,7 +699,7 @@ struct Solver {
       }
       const dim3 gx = wave(k_bicg_xr<R, RX, PV>, nn);
       launch_k(k_bicg_xr<R, RX, PV>, gx, kThreads, 0, st, any_view(xin), any_view(p), any_view(s), any_view(t),
-               any_view(r), any_view(rt), nn, partial, fused_multi() ? 1 : nb_ts, fused() ? ctl + 2 : nullptr,
+               any_view(r), any_view(rt), nn, partial, nb_ts, fused() ? ctl + 2 : nullptr,
                partial2, sc, ctl);
       QCD_LAUNCH_CK();
       launch_k(k_bicg_check, nrhs, kThreads, 0, st, sc, partial2, (int)gx.x, ctl, 1);
@@ -668,7 +717,7 @@ struct Solver {
         if (cg_single())
           nb_dev = npart;
         else
-          nb = ls;  // one sum per slice
+          nb = ls * red_row_groups(ls, g->lat.Vh);
       } else {
         apply_mhat(opin, w, q, 1 - dag, st, "in", ctl);
         const dim3 gr = wave(k_rdot<R, PV>, nn);

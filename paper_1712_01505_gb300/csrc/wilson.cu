@@ -874,19 +874,21 @@ __global__ void __launch_bounds__(32 * BY, 32 / BY) k_hop_sm_occ(HopArgs<P, RECO
   hop_sm<P, RECON, BY, TS, RED>(A);
 }
 
-// per slice q: out[q * 4 + k] = sum over the nsb site blocks of partial[(q * nsb + b) * 4 + k]
-// in a fixed order (one block per slice); the consumer adds the ls slices of a right-hand side
-__global__ void k_red_rows(const double* __restrict__ partial, long nsb, double* __restrict__ out) {
+// per slice q and group g = blockIdx.y of G: out[(q * G + g) * 4 + k] = sum of partial[(q * nsb + b) * 4 + k] over
+// the g-th part of the nsb site blocks, in a fixed order; the consumer adds the sums of a right-hand side
+__global__ void __launch_bounds__(256) k_red_rows(const double* __restrict__ partial, long nsb,
+                                                  double* __restrict__ out) {
   pdl_enter();
   const int q = blockIdx.x;
+  const long per = (nsb + gridDim.y - 1) / gridDim.y, b0 = blockIdx.y * per, b1 = min(nsb, b0 + per);
   double v[3] = {0.0, 0.0, 0.0};
-  for (long b = threadIdx.x; b < nsb; b += blockDim.x)
+  for (long b = b0 + threadIdx.x; b < b1; b += blockDim.x)
 #pragma unroll
     for (int k = 0; k < 3; ++k) v[k] += partial[((long)q * nsb + b) * 4 + k];
   block_sum<3>(v);
   if (threadIdx.x == 0)
 #pragma unroll
-    for (int k = 0; k < 3; ++k) out[(long)q * 4 + k] = v[k];
+    for (int k = 0; k < 3; ++k) out[((long)q * gridDim.y + blockIdx.y) * 4 + k] = v[k];
 }
 
 Geom dev_geom(const Lattice& lat) { return make_geom(lat.L, lat.bc, lat.V, lat.Vh); }
@@ -1211,7 +1213,8 @@ void hop_impl(const qcd_gauge* gh, const void* links, const Field& in, Field& ou
   run_cfg<P, RECON>(&L, cfg);
   QCD_LAUNCH_CK();
   if (multi_red) {  // per right-hand side sums of the per-warp partials
-    launch_k(k_red_rows, (unsigned)A.nslices, 256, 0, st, A.partial, (A.g.Vh + 31) / 32, A.gpartial);
+    launch_k(k_red_rows, dim3((unsigned)A.nslices, (unsigned)red_row_groups(in.ls, A.g.Vh)), 256, 0, st, A.partial,
+             (A.g.Vh + 31) / 32, A.gpartial);
     QCD_LAUNCH_CK();
   }
 }
