@@ -587,36 +587,49 @@ __device__ __forceinline__ void canon_store(CanonWarp& w, double2* canon, long b
 // 8^3 x 16 in FP32 1974 -> 1833 us, 24^3 x 48 in FP16 14.2 -> 13.7 ms, twelve
 // right-hand sides there 149 -> 141 ms, domain-wall 16^3 x 32 x 16 173 -> 169 ms.
 
-// v[0 .. NR) summed over the warp (all lanes call it); the result is valid in
-// lane 0.  A step that halves the number of values a lane holds costs half the additions.
+// v[0 .. NR) summed over the warp (all lanes call it): the sum of value k in the lane 8 j with
+// spread_value(j) = k.  A step that halves the number of values a lane holds costs half the
+// additions; the order of each sum is that of five shuffles by 16, 8, 4, 2, 1.
+__device__ __forceinline__ int spread_value(int j) { return ((j & 1) << 1) | (j >> 1); }  // 0, 2, 1, 3
+template <int NR, typename T>
+__device__ __forceinline__ T warp_sum_spread(const T v[NR]) {
+  static_assert(NR == 3 || NR == 4, "three or four values");
+  constexpr unsigned all = 0xffffffffu;
+  const bool h1 = threadIdx.x & 16, h2 = threadIdx.x & 8;
+  const T v3 = NR > 3 ? v[NR - 1] : T(0);
+  T a = h1 ? v[1] : v[0];  // values 0 and 2 in the lower half, 1 and 3 in the upper
+  T b = h1 ? v3 : v[2];
+  a += __shfl_xor_sync(all, h1 ? v[0] : v[1], 16);
+  b += __shfl_xor_sync(all, h1 ? v[2] : v3, 16);
+  const T send = h2 ? a : b;
+  a = h2 ? b : a;
+  a += __shfl_xor_sync(all, send, 8);
+#pragma unroll
+  for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
+  return a;
+}
+
+// the same for 1 to 3 doubles, the sums valid in lane 0
 template <int NR>
 __device__ __forceinline__ void warp_sum(double v[NR]) {
-  static_assert(NR >= 1 && NR <= 4, "warp_sum takes up to four values");
+  static_assert(NR >= 1 && NR <= 3, "warp_sum takes up to three values");
   constexpr unsigned all = 0xffffffffu;
-  const int lane = threadIdx.x & 31;
   if constexpr (NR == 1) {
 #pragma unroll
     for (int o = 16; o > 0; o >>= 1) v[0] += __shfl_down_sync(all, v[0], o);
-  } else {
-    const bool h1 = lane & 16, h2 = lane & 8;
-    double a = h1 ? v[1] : v[0];  // NR = 2: values 0 | 1 in the lower | upper half
+  } else if constexpr (NR == 2) {
+    const bool h1 = threadIdx.x & 16;
+    double a = h1 ? v[1] : v[0];
     a += __shfl_xor_sync(all, h1 ? v[0] : v[1], 16);
-    if constexpr (NR > 2) {  // and 2 | 3, then the four values one per group of 8 lanes: 0, 2, 1, 3
-      const double v3 = NR > 3 ? v[NR - 1] : 0.0;
-      double b = h1 ? v3 : v[2];
-      b += __shfl_xor_sync(all, h1 ? v[2] : v3, 16);
-      const double send = h2 ? a : b;
-      a = h2 ? b : a;
-      a += __shfl_xor_sync(all, send, 8);
-    } else {
-      a += __shfl_xor_sync(all, a, 8);
-    }
 #pragma unroll
-    for (int o = 4; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
+    for (int o = 8; o > 0; o >>= 1) a += __shfl_xor_sync(all, a, o);
     v[0] = a;
     v[1] = __shfl_sync(all, a, 16);
-    if constexpr (NR > 2) v[2] = __shfl_sync(all, a, 8);
-    if constexpr (NR > 3) v[3] = __shfl_sync(all, a, 24);
+  } else {
+    const double a = warp_sum_spread<3>(v);
+    v[0] = a;
+    v[1] = __shfl_sync(all, a, 16);
+    v[2] = __shfl_sync(all, a, 8);
   }
 }
 

