@@ -15,16 +15,16 @@
 //
 //   sum a h = HH + C,  HH = sum ah hh (64-bit, exact),  C = sum (ah hl + al hh) (FP32),
 //
-// one integer multiply-add and two FP32 ones per real product (sum al hl is
-// below 2^-3 of the last place kept).  HH >> 3 and C / 8 are added into 64-bit sums
-// aligned to the largest e of the eight neighbours; their unit is 2^(e - 1079).
+// one integer multiply-add and two FP32 ones per real product (the sum of six al hl is
+// below 6, less than one unit of the last place kept, which is 8).  HH / 8 and C / 8, rounded to nearest,
+// are added into 64-bit sums aligned to the largest e of the eight neighbours, E; their unit is 2^(E - 1079).
 // Measured against 80-bit arithmetic (tests/test_fixed_point.py), the sum of the
 // eight hops is closer to the exact one than FP64 multiply-adds: relative error
 // 1.0e-16 against 1.5e-16, the same for fields whose sites differ by orders of
 // magnitude.
 //
-// Bounds: with rows of U of 2-norm <= 5/4, |HH| <= 5/4 2^30 sqrt(6) 2^31 < 2^62.7,
-// |C| < 2^33, and the sum of eight hops < 2^62.7.
+// Bounds: with rows of U of 2-norm <= 5/4, |HH| <= 5/4 2^30 sqrt(6) 2^31 < 2^62.7 (with the half that rounds it, at most
+// 2^60, below 2^63), |C| <= 5/4 sqrt(6) 2^30 + 6 2^31 / 2 < 2^33.3 (|hl| <= 1, |al| <= 1/2), and the sum of eight hops < 2^62.7.
 #pragma once
 #include <stdint.h>
 #include <string.h>
@@ -43,6 +43,8 @@ namespace fx {
 // exponent fields (of the largest component) that the fixed-point path takes; sites below kEmin and
 // above kEmax (infinities and NaN included) are stored as FP64 with the field kBad
 constexpr int kEmin = 256, kEmax = 1982, kBad = 0x7000;
+// HH and C are divided by 2^d, d = E - e + 3; from this d on a neighbour is left out (|HH| / 2^d < 1.6 units)
+constexpr int kFar = 62;
 // 2-norms of link rows and columns that it takes
 constexpr double kNormMax = 1.25, kNormMin = 0.5;
 
@@ -85,6 +87,17 @@ FX_FN Part spinor_part(unsigned hi, unsigned lo, int e) {
   l -= up << 27;
   const int s = (int)hi >> 31;
   return {(h ^ s) - s, (float)((l ^ s) - s) * 0x1p-27f};
+}
+
+// (H + C) / 2^d rounded, 3 <= d < kFar; H holds hop_half besides, sc = 2^-d.  Ties of H (one in eight at d = 3) go up in
+// the forward hops and down in the backward ones, so that the eight together have no bias.
+FX_FN int64_t hop_half(int d, int back) { return ((int64_t)1 << (d - 1)) - back; }
+FX_FN int64_t hop_round(int64_t H, float C, float sc, int d) {
+#if defined(__CUDA_ARCH__)
+  return (H >> d) + (int64_t)__float2int_rn(C * sc);
+#else
+  return (H >> d) + (int64_t)lrintf(C * sc);
+#endif
 }
 
 // the value of a part as a double; e as in spinor_part

@@ -218,35 +218,36 @@ __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int s
     gs[c] = swp(g[c]);
     hn[c] = -hi[c];
   }
-  const float sc = __int_as_float((127 - d3) << 23);
   if (!mbar_wait(&W.sm->bar[W.warp][I % kBuf], (unsigned)(I / kBuf) & 1u)) W.failed = true;
-  const int4* w = &W.sm->w[W.warp][I % kBuf][W.lane % kSB];
+  if (d3 < kFar) {
+    const float sc = __int_as_float((127 - d3) << 23);
+    const int4* w = &W.sm->w[W.warp][I % kBuf][W.lane % kSB];
 #pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    int64_t Hr = 0, Hi = 0;
-    float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
+    for (int a = 0; a < 3; ++a) {
+      int64_t Hr = hop_half(d3, HOP & 1), Hi = Hr;
+      float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
 #pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int4 u = w[(a * 3 + b) * kSB];
-      Hr += (int64_t)u.x * hr[b];
-      Hr += (int64_t)u.z * hn[b];
-      Hi += (int64_t)u.x * hi[b];
-      Hi += (int64_t)u.z * hr[b];
-      C = fma2(bc2((float)u.x), y[b], C);
-      C = fma2(bc2(__int_as_float(u.y)), g[b], C);
-      D = fma2(bc2((float)u.z), ys[b], D);
-      D = fma2(bc2(__int_as_float(u.w)), gs[b], D);
-    }
-    const int64_t wr = (Hr >> d3) + (int64_t)__float2int_rn((C.x - D.x) * sc);
-    const int64_t wi = (Hi >> d3) + (int64_t)__float2int_rn((C.y + D.y) * sc);
-    up[2 * a] += wr;
-    up[2 * a + 1] += wi;
-    if (MU == 0 || MU == 2) {  // SG i w
-      lo[2 * a] -= SG * wi;
-      lo[2 * a + 1] += SG * wr;
-    } else {
-      lo[2 * a] += SG * wr;
-      lo[2 * a + 1] += SG * wi;
+      for (int b = 0; b < 3; ++b) {
+        const int4 u = w[(a * 3 + b) * kSB];
+        Hr += (int64_t)u.x * hr[b];
+        Hr += (int64_t)u.z * hn[b];
+        Hi += (int64_t)u.x * hi[b];
+        Hi += (int64_t)u.z * hr[b];
+        C = fma2(bc2((float)u.x), y[b], C);
+        C = fma2(bc2(__int_as_float(u.y)), g[b], C);
+        D = fma2(bc2((float)u.z), ys[b], D);
+        D = fma2(bc2(__int_as_float(u.w)), gs[b], D);
+      }
+      const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
+      up[2 * a] += wr;
+      up[2 * a + 1] += wi;
+      if (MU == 0 || MU == 2) {  // SG i w
+        lo[2 * a] -= SG * wi;
+        lo[2 * a + 1] += SG * wr;
+      } else {
+        lo[2 * a] += SG * wr;
+        lo[2 * a + 1] += SG * wi;
+      }
     }
   }
   __syncwarp();  // every lane has read the buffer
