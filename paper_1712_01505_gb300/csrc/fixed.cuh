@@ -10,7 +10,7 @@
 // where e is the exponent field of the site's largest |component| (which lies in
 // [2^(e - 1023), 2^(e - 1022))), so |xh| < 2^30; a double of exponent e splits without
 // rounding, and smaller ones to within 1.5 2^-56 of 2^(e - 1022) (the shift drops less than 2^-57,
-// the FP32 remainder of 26 bits is rounded by at most 2^-56).
+// the FP32 remainder of 26 bits is rounded by at most 2^-56; what is not zero stays so).
 // Half spinors h = u +- B l are formed part by part (|hh| < 2^31), and
 //
 //   sum a h = HH + C,  HH = sum ah hh (64-bit, exact),  C = sum (ah hl + al hh) (FP32),
@@ -22,6 +22,13 @@
 // eight hops is closer to the exact one than FP64 multiply-adds: relative error
 // 1.0e-16 against 1.5e-16, the same for fields whose sites differ by orders of
 // magnitude.
+//
+// That is an error of 11 units (rms, nearly all of it the FP32 roundings of C) whatever the component is, 4 with one
+// neighbour only, where FP64's is measured by the component's own products.  So a component counts as computed only
+// where S = sum |U| |h|, the magnitudes of its products over the eight hops, shows that the error is small beside it:
+// S >= 2^(E - 1022) / 16 with one neighbour that outweighs the rest, / 8 with several (kSumMin, sum_min); FP64 computes
+// the sites with a component below (wilson_fx.cu).  That leaves at most 5.4 2^-53 S (rms; a chain of FP64 multiply-adds is
+// certain to 16 2^-53 S).  Gaussian fields have S = 4.6 2^(E - 1022), and 0.15 2^-53 S here against 0.29 in FP64.
 //
 // Bounds: with rows of U of 2-norm <= 5/4, |HH| <= 5/4 2^30 sqrt(6) 2^31 < 2^62.7 (with the half that rounds it, at most
 // 2^60, below 2^63), |C| <= 5/4 sqrt(6) 2^30 + 6 2^31 / 2 < 2^33.3 (|hl| <= 1, |al| <= 1/2), and the sum of eight hops < 2^62.7.
@@ -41,10 +48,13 @@ namespace qcd {
 namespace fx {
 
 // exponent fields (of the largest component) that the fixed-point path takes; sites below kEmin and
-// above kEmax (infinities and NaN included) are stored as FP64 with the field kBad
-constexpr int kEmin = 256, kEmax = 1982, kBad = 0x7000;
+// above kEmax (infinities and NaN included) are stored as FP64 with the field kBad; kZero: all components are zero
+constexpr int kEmin = 256, kEmax = 1982, kZero = kEmin - 1, kBad = 0x7000;
 // HH and C are divided by 2^d, d = E - e + 3; from this d on a neighbour is left out (|HH| / 2^d < 1.6 units)
 constexpr int kFar = 62;
+// what the magnitudes of a component's products have to add up to, in units of HH where e = E (2^60 is
+// 2^(E - 1022)): this times the sum of the neighbours' sizes relative to the largest one's, at most 2
+constexpr float kSumMin = 0x1p56f;
 // 2-norms of link rows and columns that it takes
 constexpr double kNormMax = 1.25, kNormMin = 0.5;
 
@@ -82,6 +92,7 @@ FX_FN Part spinor_part(unsigned hi, unsigned lo, int e) {
   const unsigned m = (hi & 0xfffffu) | 0x100000u;
   const uint64_t p = shr64(((uint64_t)m << 36) | ((uint64_t)lo << 4), d);  // |v| 2^(1079 - e), 57 bits
   int h = (int)(p >> 27), l = (int)(p & 0x7ffffffu);
+  l |= (p == 0) & (((hi << 1) | lo) != 0);  // not zero: the last unit
   const int up = (l >> 26) & (h != 0x3fffffff);  // round h to nearest, but keep it below 2^30
   h += up;
   l -= up << 27;
@@ -99,6 +110,8 @@ FX_FN int64_t hop_round(int64_t H, float C, float sc, int d) {
   return (H >> d) + (int64_t)lrintf(C * sc);
 #endif
 }
+// the least sum of magnitudes for neighbours whose sizes relative to the largest one's add up to `size` (1 to 8)
+FX_FN float sum_min(float size) { return size < 2.f ? kSumMin * size : kSumMin * 2.f; }
 
 // the value of a part as a double; e as in spinor_part
 FX_FN double part_value(const Part& p, int e) { return ldexp((double)p.h + (double)p.l, e - 1052); }

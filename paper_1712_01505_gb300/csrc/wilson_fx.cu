@@ -46,7 +46,7 @@ struct FxField {
 // the exponent field of a site's 12 components (words of doubles); kBad out of range
 __device__ __forceinline__ int fx_field_of(unsigned mx, unsigned low) {
   const int e = (int)(mx >> 20);
-  if (mx == 0) return low ? kBad : kEmin;  // subnormals below 2^-1042 / all zero
+  if (mx == 0) return low ? kBad : kZero;  // subnormals below 2^-1042 / all zero
   return e < kEmin || e > kEmax ? kBad : e;
 }
 template <int N>
@@ -170,22 +170,16 @@ __device__ __forceinline__ void fx_abandon(FxWarp& W) {  // wait for the copies 
   for (int b = 0; b < kBuf; ++b) mbar_wait(&W.sm->bar[W.warp][b], 0u);
 }
 
-// Hop number I (of fx_order) added to up (upper spin sp) and lo (a lower spin; up to the sign that the caller
-// applies).  m: the sign of the lower input spin.  Packed FP32 lanes: (re, im).
-template <int I>
-__device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int sp, int m, int64_t (&up)[6],
-                                       int64_t (&lo)[6]) {
-  constexpr int HOP = fx_order(I), MU = HOP >> 1;
-  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
-  const int nbw = W.sm->nb[HOP][W.warp * kSB + W.lane % kSB], ncb = nbw & 0x7fffffff;
+// The half spinor of a hop in direction MU that the lane multiplies (upper spin sp, the lower spin that it meets times
+// m): integer and FP32 parts.  nbw: the neighbour's index, negative with the antiperiodic factor.
+template <int MU>
+__device__ __forceinline__ void fx_half(const FxField& f, int nbw, int sp, int m, int (&hr)[3], int (&hi)[3],
+                                        float2 (&y)[3]) {
+  const int ncb = nbw & 0x7fffffff;
   const int4* q = f.p + (long)(ncb / kSB) * kSiteUnits + ncb % kSB;
   const int4* qu = q + sp * (3 * kSB);
   const int4* ql = q + 6 * kSB + (MU < 2 ? 1 - sp : sp) * (3 * kSB);  // the lower spin that meets upper spin sp
-  const int d3 = min(E - __ldg(f.e + ncb), 100) + 3;
-  m *= SG;
   const float mf = (float)m;
-  int hr[3], hi[3];
-  float2 y[3];  // the FP32 parts
 #pragma unroll
   for (int c = 0; c < 3; ++c) {
     const int4 a = __ldg(qu + c * kSB), b = __ldg(ql + c * kSB);
@@ -209,6 +203,26 @@ __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int s
       y[c] = make_float2(-y[c].x, -y[c].y);
     }
   }
+}
+
+// What the eight hops add up to in a lane: upper spin sp and a lower spin (up to the sign that fx_sum applies), and
+// beside each component the sum of |hop| in units of 2^48 (2^(E - 1022) is 2^9 of them), a component's real and
+// imaginary part in one word.
+struct FxSum {
+  int64_t up[6], lo[6];
+  unsigned su[3], sl[3];
+};
+
+// Hop number I (of fx_order) added to a.  m: the sign of the lower input spin.  Packed FP32 lanes: (re, im).
+template <int I>
+__device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int sp, int m, FxSum& S) {
+  constexpr int HOP = fx_order(I), MU = HOP >> 1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
+  const int nbw = W.sm->nb[HOP][W.warp * kSB + W.lane % kSB];
+  const int d3 = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100) + 3;
+  int hr[3], hi[3];
+  float2 y[3];  // the FP32 parts
+  fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
   int hn[3];
   float2 g[3], ys[3], gs[3];  // the integer parts as FP32; both with the lanes exchanged
 #pragma unroll
@@ -239,14 +253,18 @@ __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int s
         D = fma2(bc2(__int_as_float(u.w)), gs[b], D);
       }
       const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
-      up[2 * a] += wr;
-      up[2 * a + 1] += wi;
+      const unsigned size = __byte_perm(abs((int)(wr >> 32)), abs((int)(wi >> 32)), 0x7632);
+      S.up[2 * a] += wr;
+      S.up[2 * a + 1] += wi;
+      S.su[a] += size;
       if (MU == 0 || MU == 2) {  // SG i w
-        lo[2 * a] -= SG * wi;
-        lo[2 * a + 1] += SG * wr;
+        S.lo[2 * a] -= SG * wi;
+        S.lo[2 * a + 1] += SG * wr;
+        S.sl[a] += __byte_perm(size, size, 0x1032);
       } else {
-        lo[2 * a] += SG * wr;
-        lo[2 * a + 1] += SG * wi;
+        S.lo[2 * a] += SG * wr;
+        S.lo[2 * a + 1] += SG * wi;
+        S.sl[a] += size;
       }
     }
   }
@@ -254,9 +272,75 @@ __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int s
   if (I + kBuf < 8) W.issue(fx_order(I + kBuf < 8 ? I + kBuf : 0), I % kBuf);
 }
 
-// The hop sum of one site in FP64 from the fixed-point field (neighbours whose values are kept in
-// FP64), added to acc.
-__device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int cb, Cx<double>* out) {
+// The magnitudes of the products of hop number I, per component of the lane: upper spin sp in s, the lower spin in t;
+// bits of nz, nt: a product is not zero.  links: of the lane's site.
+template <int I>
+__device__ __forceinline__ void fx_magnitudes(const int* nb, const FxField& f, const int4* links, int E, int sp, int m,
+                                              float (&s)[6], float (&t)[6], unsigned& nz, unsigned& nt, float& size) {
+  constexpr int HOP = fx_order(I), MU = HOP >> 1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;
+  const int nbw = nb[HOP * (kWarps * kSB)];
+  const int d = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100);
+  const float sc = __int_as_float((127 - d) << 23);
+  int hr[3], hi[3];
+  float2 y[3];
+  fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
+  size += sc;
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    float mr = 0.f, mi = 0.f;
+    unsigned br = 0, bi = 0;
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 u = __ldg(links + HOP * kHopUnits + (a * 3 + b) * kSB);
+      const float ur = fabsf((float)u.x + __int_as_float(u.y)), ui = fabsf((float)u.z + __int_as_float(u.w));
+      const float xr = fabsf((float)hr[b] + y[b].x), xi = fabsf((float)hi[b] + y[b].y);
+      mr = fmaf(ur, xr, fmaf(ui, xi, mr));
+      mi = fmaf(ur, xi, fmaf(ui, xr, mi));
+      br |= (ur != 0.f && xr != 0.f) || (ui != 0.f && xi != 0.f);
+      bi |= (ur != 0.f && xi != 0.f) || (ui != 0.f && xr != 0.f);
+    }
+    constexpr int x = (MU == 0 || MU == 2) ? 1 : 0;  // i w
+    s[2 * a] = fmaf(mr, sc, s[2 * a]);
+    s[2 * a + 1] = fmaf(mi, sc, s[2 * a + 1]);
+    t[2 * a + x] = fmaf(mr, sc, t[2 * a + x]);
+    t[2 * a + 1 - x] = fmaf(mi, sc, t[2 * a + 1 - x]);
+    nz |= (br | bi << 1) << (2 * a);
+    nt |= (x ? (bi | br << 1) : (br | bi << 1)) << (2 * a);
+  }
+}
+
+// Whether every component of the lane is as exact from the fixed-point parts as FP64 would have it (fixed.cuh), or has
+// no product that is not zero.  The whole warp calls it.
+__device__ __noinline__ bool fx_exact(const int* nb, const FxField& f, const int4* links, int E, int sp, int g5) {
+  const int gs = sp ? -g5 : g5;
+  float s[6] = {}, t[6] = {}, size = 0.f;
+  unsigned nz = 0, nt = 0;
+  fx_magnitudes<0>(nb, f, links, E, sp, -gs, s, t, nz, nt, size);
+  fx_magnitudes<1>(nb, f, links, E, sp, -gs, s, t, nz, nt, size);
+  fx_magnitudes<2>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
+  fx_magnitudes<3>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) t[k] = __shfl_xor_sync(0xffffffffu, t[k], kSB);  // the lower spins change lanes (fx_sum)
+  nt = __shfl_xor_sync(0xffffffffu, nt, kSB);
+  fx_magnitudes<4>(nb, f, links, E, sp, gs, s, t, nz, nt, size);
+  fx_magnitudes<5>(nb, f, links, E, sp, gs, s, t, nz, nt, size);
+  fx_magnitudes<6>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
+  fx_magnitudes<7>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
+  const float least = sum_min(size);
+  bool ok = true;
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    ok = ok && (s[k] >= least || !(nz >> k & 1)) && (t[k] >= least || !(nt >> k & 1));
+  return ok;
+}
+
+// The hop sum of one site in FP64: from the FP64 field that was converted to f where A.in names it (slice q of an internal
+// field, or with A.in.stride 1 of a canonical one), else from the parts (the first half-dslash of Mhat left no other form).
+__device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int q, int cb, Cx<double>* out) {
+  const double2* src = A.in.p;
+  const bool canon = A.in.stride == 1;
+  if (src) src += canon ? (long)q * A.g.V * 12 : (long)(q / A.ls) * 12 * A.in.stride + (long)(q % A.ls) * A.g.Vh;
   const SiteCoords c = cb_to_site(A.g, cb, A.out_parity);
   const double sg = A.dagger ? 1.0 : -1.0;
   Cx<double> acc[12];
@@ -271,6 +355,11 @@ __device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int cb, Cx
     Cx<double> U[9], psi[12], h[6], gg[6];
     A.U.load(back ? 1 - A.out_parity : A.out_parity, MU, back ? n : cb, U);
     for (int k = 0; k < 12; ++k) {
+      if (src) {
+        const double2 v = src[canon ? (long)canon_index(A.g, n, 1 - A.out_parity) * 12 + k : k * A.in.stride + n];
+        psi[k] = {v.x, v.y};
+        continue;
+      }
       const int4 u = f.p[(long)(n / kSB) * kSiteUnits + k * kSB + n % kSB];
       if (e == kBad)
         psi[k] = {__hiloint2double(u.y, u.x), __hiloint2double(u.w, u.z)};
@@ -294,9 +383,9 @@ __device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int cb, Cx
 }
 
 // [x +] a H in of one site in FP64, stored
-__device__ __noinline__ void fp64_site_store(const HA& A, const FxField& f, int cb, int r, long site) {
+__device__ __noinline__ void fp64_site_store(const HA& A, const FxField& f, int q, int cb, int r, long site) {
   Cx<double> acc[12], o[12];
-  fp64_site(A, f, cb, acc);
+  fp64_site(A, f, q, cb, acc);
   if (A.xpay) {
     A.x.offset_rhs(r).load(site, o);
     for (int k = 0; k < 12; ++k) o[k] = fmac(A.a, acc[k], o[k]);
@@ -307,9 +396,9 @@ __device__ __noinline__ void fp64_site_store(const HA& A, const FxField& f, int 
 }
 
 // H in of one site in FP64, stored in the fixed-point field o as a kBad site
-__device__ __noinline__ void fp64_site_store_fx(const HA& A, const FxField& f, const FxField& o, int cb) {
+__device__ __noinline__ void fp64_site_store_fx(const HA& A, const FxField& f, const FxField& o, int q, int cb) {
   Cx<double> acc[12];
-  fp64_site(A, f, cb, acc);
+  fp64_site(A, f, q, cb, acc);
   int4* p = o.p + (long)(cb / kSB) * kSiteUnits + cb % kSB;
   for (int k = 0; k < 12; ++k)
     p[k * kSB] = make_int4(__double2loint(acc[k].re), __double2hiint(acc[k].re), __double2loint(acc[k].im),
@@ -320,7 +409,7 @@ __device__ __noinline__ void fp64_site_store_fx(const HA& A, const FxField& f, c
 // The exponent field of the site's largest neighbour (its neighbour indices go to shared memory).
 __device__ __forceinline__ int fx_neighbours(const HA& A, FxWarp& W, const FxField& f, int cb) {
   const SiteCoords c = cb_to_site(A.g, cb, A.out_parity);
-  int E = kEmin;
+  int E = kZero;
   const bool back = W.lane >= kSB;  // the site's other lane does the forward hops
 #pragma unroll
   for (int mu = 0; mu < 4; ++mu) {
@@ -340,26 +429,44 @@ __device__ __forceinline__ void flip(int64_t (&v)[6], bool minus) {
   for (int k = 0; k < 6; ++k) v[k] = (v[k] ^ n) - n;
 }
 
-// up, lo = the sum of the eight hops for spins sp and 2 + sp, in units of the returned value
-// (lo: times -1 for H^dag = g5 H g5); the whole warp calls it
-__device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, int64_t (&up)[6],
-                                         int64_t (&lo)[6]) {
+// S.up, S.lo = the sum of the eight hops for spins sp and 2 + sp, in units of the returned value
+// (lo: times -1 for H^dag = g5 H g5); the whole warp calls it.  slow: the site is FP64's, for a neighbour that is
+// kept in FP64 or a component that the parts do not hold well enough.
+//
+// The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
+// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Only then are the magnitudes formed (fx_exact, a
+// second walk over the hops), which settles all but fields with components far smaller than others that the links hardly
+// mix with them.  Without any of this the full matrix on 24^3 x 48 took 309 us instead of 319, a solve on 12x10x14x18 3.61 ms
+// instead of 3.75, and twelve point sources on 24^3 x 48, around which spins and colours differ most, 139 ms instead of 146.
+__device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S, bool& slow) {
   const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) up[k] = lo[k] = 0;
-  fx_hop<0>(W, f, E, sp, -gs, up, lo);  // y: B = (-l1, l0)
-  fx_hop<1>(W, f, E, sp, -gs, up, lo);
-  flip(lo, sp == 0);                    // B^dag = (g1, -g0)
-  fx_hop<2>(W, f, E, sp, g5, up, lo);   // x: B = -i (l1, l0)
-  fx_hop<3>(W, f, E, sp, g5, up, lo);
+  for (int k = 0; k < 6; ++k) S.up[k] = S.lo[k] = 0;
 #pragma unroll
-  for (int k = 0; k < 6; ++k) lo[k] = __shfl_xor_sync(0xffffffffu, lo[k], kSB);
-  flip(lo, sp != 0);
-  fx_hop<4>(W, f, E, sp, gs, up, lo);   // z: B = (-i l0, i l1)
-  fx_hop<5>(W, f, E, sp, gs, up, lo);
-  flip(lo, sp != 0);
-  fx_hop<6>(W, f, E, sp, g5, up, lo);   // t: B = 1
-  fx_hop<7>(W, f, E, sp, g5, up, lo);
+  for (int k = 0; k < 3; ++k) S.su[k] = S.sl[k] = 0;
+  fx_hop<0>(W, f, E, sp, -gs, S);  // y: B = (-l1, l0)
+  fx_hop<1>(W, f, E, sp, -gs, S);
+  flip(S.lo, sp == 0);             // B^dag = (g1, -g0)
+  fx_hop<2>(W, f, E, sp, g5, S);   // x: B = -i (l1, l0)
+  fx_hop<3>(W, f, E, sp, g5, S);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) S.lo[k] = __shfl_xor_sync(0xffffffffu, S.lo[k], kSB);
+#pragma unroll
+  for (int k = 0; k < 3; ++k) S.sl[k] = __shfl_xor_sync(0xffffffffu, S.sl[k], kSB);
+  flip(S.lo, sp != 0);
+  fx_hop<4>(W, f, E, sp, gs, S);   // z: B = (-i l0, i l1)
+  fx_hop<5>(W, f, E, sp, gs, S);
+  flip(S.lo, sp != 0);
+  fx_hop<6>(W, f, E, sp, g5, S);   // t: B = 1
+  fx_hop<7>(W, f, E, sp, g5, S);
+  unsigned least = 0xffffffffu;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) least = __vminu2(least, __vminu2(S.su[k], S.sl[k]));
+  bool weak = min(least & 0xffffu, least >> 16) < 64u && E > kZero && E < kBad;  // kZero: all neighbours are zero
+  if (__any_sync(0xffffffffu, weak))
+    weak = !fx_exact(&W.sm->nb[0][W.warp * kSB + W.lane % kSB], f, W.links + W.lane % kSB, E, sp, g5) && weak;
+  const unsigned any = __ballot_sync(0xffffffffu, weak);
+  slow = E == kBad || ((any | any >> kSB) >> (W.lane % kSB) & 1);  // of either lane
   if (W.failed) return __longlong_as_double(0x7ff8000000000000ll);  // a copy that never arrived: NaN output
   return __hiloint2double((E - 56) << 20, 0);  // 2^(E - 1079)
 }
@@ -367,7 +474,7 @@ __device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& 
 // The sums as a fixed-point field of their own (a = 1, no x term: the first half-dslash of Mhat, whose
 // result only the second one reads): both lanes of a site find its largest sum.
 __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, bool valid, int E, bool minus_lo, bool nan,
-                                         int64_t (&up)[6], int64_t (&lo)[6]) {
+                                         bool slow, int64_t (&up)[6], int64_t (&lo)[6]) {
   flip(lo, minus_lo);
   uint64_t mx = 0;
 #pragma unroll
@@ -376,11 +483,11 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
     mx |= (uint64_t)(lo[k] ^ (lo[k] >> 63));
   }
   mx |= __shfl_xor_sync(0xffffffffu, mx, kSB);
-  if (!valid || E == kBad) return;  // kBad: fp64_site_store_fx
+  if (!valid || slow) return;  // slow: fp64_site_store_fx
   const int b = 64 - __clzll((long long)mx);  // -2^b <= every sum < 2^b
-  const int e = mx ? b + E - 57 : kEmin, shift = b - 30;
+  const int e = mx ? b + E - 57 : kZero, shift = b - 30;
   int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
-  const bool wide = nan || e < kEmin || e > kEmax;
+  const bool wide = nan || (mx && (e < kEmin || e > kEmax));
   const double unit = nan ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double((E - 56) << 20, 0);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
@@ -423,17 +530,19 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_const
   const long site = (long)s * A.g.Vh + cb;
   const FxField f{F.p + (long)q * F.nsb * kSiteUnits, F.e + (long)q * F.nsb * kSB, F.nsb};
   const int E = fx_neighbours(A, W, f, valid ? cb : 0);
-  int64_t up[6], lo[6];
-  const double unit = fx_sum(A, W, f, E, sp, up, lo);
+  FxSum S;
+  bool slow;
+  const double unit = fx_sum(A, W, f, E, sp, S, slow);
+  int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
   if constexpr (OUT == 1) {
     const FxField o{O.p + (long)q * O.nsb * kSiteUnits, O.e + (long)q * O.nsb * kSB, O.nsb};
-    fx_store(o, cb, sp, valid, E, A.dagger != 0, W.failed, up, lo);
-    if (E == kBad && valid && sp == 0) fp64_site_store_fx(A, f, o, cb);
+    fx_store(o, cb, sp, valid, E, A.dagger != 0, W.failed, slow, up, lo);
+    if (slow && valid && sp == 0) fp64_site_store_fx(A, f, o, q, cb);
     return;
   }
   if (!valid) return;
-  if (E == kBad) {
-    if (sp == 0) fp64_site_store(A, f, cb, r, site);
+  if (slow) {
+    if (sp == 0) fp64_site_store(A, f, q, cb, r, site);
     return;
   }
   const double au = A.a * unit, al = A.dagger ? -au : au;
@@ -476,11 +585,12 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx_red(const __grid_c
   double red[3] = {0.0, 0.0, 0.0};
   if (warp_valid) {
     const int E = fx_neighbours(A, W, F, valid ? cb : 0);
-    const bool bad = E == kBad;
-    if (bad && valid && sp == 0) fp64_site_store(A, F, cb, 0, cb);
+    FxSum S;
+    bool bad;
+    const double unit = fx_sum(A, W, F, E, sp, S, bad);
+    if (bad && valid && sp == 0) fp64_site_store(A, F, 0, cb, 0, cb);
     __syncwarp();
-    int64_t up[6], lo[6];
-    const double unit = fx_sum(A, W, F, E, sp, up, lo);
+    int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
     const double au = A.a * unit, al = A.dagger ? -au : au;
     if (valid) {
       const double2* x = A.x.p + 3 * sp * A.x.stride + cb;
@@ -591,11 +701,10 @@ __device__ __forceinline__ FxLane fx_lane(const HA& A) {
 __device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField& f, const FxLane& L, Cx<double> v[6],
                                           double a[2]) {
   const int E = fx_neighbours(A, W, f, L.valid ? L.cb : 0);
-  Cx<double> slow[12];
-  const bool bad = E == kBad && L.valid;
-  if (bad) fp64_site(A, f, L.cb, slow);  // both lanes of the site
-  int64_t up[6], lo[6];
-  const double unit = fx_sum(A, W, f, E, L.sp, up, lo);
+  FxSum S;
+  bool bad;
+  const double unit = fx_sum(A, W, f, E, L.sp, S, bad);
+  int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
   a[0] = A.a * unit;
   a[1] = A.dagger ? -a[0] : a[0];
 #pragma unroll
@@ -603,7 +712,9 @@ __device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField&
     v[c] = {(double)up[2 * c], (double)up[2 * c + 1]};
     v[3 + c] = {(double)lo[2 * c], (double)lo[2 * c + 1]};
   }
-  if (bad) {
+  if (bad && L.valid) {
+    Cx<double> slow[12];
+    fp64_site(A, f, L.q, L.cb, slow);  // both lanes of the site
     a[0] = a[1] = A.a;
     const Cx<double>* w = slow + 3 * L.sp;
 #pragma unroll
@@ -830,6 +941,7 @@ __global__ void __launch_bounds__(128) k_links_fx(Geom g, const double2* __restr
   int4* wf = W + (((long)par * nsb + cb / kSB) * 8 + 2 * mu) * kHopUnits + cb % kSB;
   int4* wb = W + (((long)(1 - par) * nsb + j / kSB) * 8 + 2 * mu + 1) * kHopUnits + j % kSB;
   float row[3] = {0.f, 0.f, 0.f}, col[3] = {0.f, 0.f, 0.f};
+  bool ok = true;
 #pragma unroll
   for (int k = 0; k < 9; ++k) {
     const double2 u = u64[k * Vh];
@@ -837,10 +949,10 @@ __global__ void __launch_bounds__(128) k_links_fx(Geom g, const double2* __restr
     row[k / 3] += n;
     col[k % 3] += n;
     const Part re = link_part(u.x), im = link_part(u.y);
+    ok = ok && (re.h || re.l != 0.f || u.x == 0.0) && (im.h || im.l != 0.f || u.y == 0.0);  // not lost
     wf[k * kSB] = make_int4(re.h, __float_as_int(re.l), im.h, __float_as_int(im.l));
     wb[((k % 3) * 3 + k / 3) * kSB] = make_int4(re.h, __float_as_int(re.l), -im.h, __float_as_int(-im.l));
   }
-  bool ok = true;
 #pragma unroll
   for (int k = 0; k < 3; ++k) {
     constexpr float lo = (float)(kNormMin * kNormMin), hi = (float)(kNormMax * kNormMax);
@@ -917,10 +1029,12 @@ void fx_args(HA& A, const qcd_gauge* gh, const Field& shape, int out_parity, int
   A.a = a;
   A.U.p = (const double2*)gh->U64;
   A.U.Vh = gh->lat.Vh;
+  A.in = {nullptr, nullptr, 0};  // no FP64 form of the input
 }
+SpinorView<P64> canon_view(const double2* p) { return {const_cast<double2*>(p), nullptr, 1}; }
 
-// out = [x +] a H in (out FP64), or the fixed-point field fout = H in (a = 1, x null)
-void fx_launch(const qcd_gauge* gh, const FxField& in, const Field& shape, Field* out, const FxField* fout,
+// out = [x +] a H in (out FP64), or the fixed-point field fout = H in (a = 1, x null); src: the FP64 form of `in`
+void fx_launch(const qcd_gauge* gh, const FxField& in, const SpinorView<P64>* src, const Field& shape, Field* out, const FxField* fout,
                int out_parity, int dagger, double a, const Field* x, cudaStream_t st, const int* stop,
                const RedSpec* red) {
   FxLaunch L;
@@ -940,7 +1054,7 @@ void fx_launch(const qcd_gauge* gh, const FxField& in, const Field& shape, Field
   fx_args(A, gh, shape, out_parity, dagger, a);
   A.xpay = x != nullptr;
   A.out = out ? fx_view(*out) : fx_view(shape);
-  A.in = A.out;  // not read: the input is L.F
+  if (src) A.in = *src;
   A.x = x ? fx_view(*x) : A.out;
   A.rt = red && red->rt ? fx_view(*red->rt) : A.out;
   A.stop = stop;
@@ -1019,7 +1133,8 @@ bool hop_fx(const qcd_gauge* gh, const Field& in, Field& out, int out_parity, in
   if (!g->fx_ok) return false;  // the links gave way to another allocation
   FxOrder order(g, st);
   fx_pack(in, f, st, stop);
-  fx_launch(g, f, in, &out, nullptr, out_parity, dagger, a, x, st, stop, red);
+  const SpinorView<P64> src = fx_view(in);
+  fx_launch(g, f, &src, in, &out, nullptr, out_parity, dagger, a, x, st, stop, red);
   order.done();
   return true;
 }
@@ -1040,8 +1155,9 @@ bool mhat_fx(const qcd_gauge* gh, const Field& in, Field& out, int dagger, doubl
   if (!g->fx_ok) return false;
   FxOrder order(g, st);
   fx_pack(in, f, st, stop);
-  fx_launch(g, f, in, nullptr, &t, 1, dagger, 1.0, nullptr, st, stop, nullptr);
-  fx_launch(g, t, in, &out, nullptr, 0, dagger, -k2, &in, st, stop, red);
+  const SpinorView<P64> src = fx_view(in);
+  fx_launch(g, f, &src, in, nullptr, &t, 1, dagger, 1.0, nullptr, st, stop, nullptr);
+  fx_launch(g, t, nullptr, in, &out, nullptr, 0, dagger, -k2, &in, st, stop, red);
   order.done();
   return true;
 }
@@ -1086,6 +1202,7 @@ void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
     fx_args(A, g, shape, 1, o.dagger, o.kappa);
     A.stop = nullptr;
     A.partial = partial;
+    A.in = fx_view(o.x);
     A.x = fx_view(o.b_o);
     A.out = fx_view(o.x_o);
     launch_k(k_outer_odd, nb * n, 32 * kWarps, sizeof(FxShared), st, A, links, fa, fb);
@@ -1096,6 +1213,7 @@ void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
   A.stop = nullptr;
   A.partial = partial;
   A.xpay = o.x_zero ? 1 : 2;
+  A.in = fx_view(o.x_zero ? o.b_o : o.x_o);
   A.rt = fx_view(o.b_e);
   A.x = fx_view(o.x);
   if (o.r.prec == QCD_F64) {
@@ -1145,9 +1263,11 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
   launch_k(k_canon_to_fx, dim3((unsigned)((shape.Vh + 127) / 128), n, full ? 2 : 1), 128, 0, st, geom, src,
            fa, full ? fb : fa, p0);
   QCD_LAUNCH_CK();
-  auto hop = [&](const FxField& from, int out_parity, double a, bool xpay, bool zero) {
+  const SpinorView<P64> cv = canon_view(src);
+  auto hop = [&](const FxField& from, bool converted, int out_parity, double a, bool xpay, bool zero) {
     HA A;
     fx_args(A, g, shape, out_parity, dagger, a);
+    if (converted) A.in = cv;
     A.stop = nullptr;
     A.xpay = xpay;
     launch_k(k_hop_fx_canon, nb * n, 32 * kWarps, sizeof(FxShared), st, A, (const int4*)g->Ufx, from, src,
@@ -1155,13 +1275,13 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
     QCD_LAUNCH_CK();
   };
   if (full) {
-    hop(fb, 0, -f.kappa, true, false);
-    hop(fa, 1, -f.kappa, true, false);
+    hop(fb, true, 0, -f.kappa, true, false);
+    hop(fa, true, 1, -f.kappa, true, false);
   } else if (mhat) {
-    fx_launch(g, fa, shape, nullptr, &fb, 1, dagger, 1.0, nullptr, st, nullptr, nullptr);
-    hop(fb, 0, -f.kappa * f.kappa, true, true);
+    fx_launch(g, fa, &cv, shape, nullptr, &fb, 1, dagger, 1.0, nullptr, st, nullptr, nullptr);
+    hop(fb, false, 0, -f.kappa * f.kappa, true, true);
   } else {
-    hop(fa, op == QCD_OP_D_OE, 1.0, false, true);
+    hop(fa, true, op == QCD_OP_D_OE, 1.0, false, true);
   }
   order.done();
   return true;
