@@ -335,75 +335,94 @@ __device__ __noinline__ bool fx_exact(const int* nb, const FxField& f, const int
   return ok;
 }
 
-// The hop sum of one site in FP64: from the FP64 field that was converted to f where A.in names it (slice q of an internal
-// field, or with A.in.stride 1 of a canonical one), else from the parts (the first half-dslash of Mhat left no other form).
-__device__ __noinline__ void fp64_site(const HA& A, const FxField& f, int q, int cb, Cx<double>* out) {
-  const double2* src = A.in.p;
-  const bool canon = A.in.stride == 1;
-  if (src) src += canon ? (long)q * A.g.V * 12 : (long)(q / A.ls) * 12 * A.in.stride + (long)(q % A.ls) * A.g.Vh;
-  const SiteCoords c = cb_to_site(A.g, cb, A.out_parity);
-  const double sg = A.dagger ? 1.0 : -1.0;
-  Cx<double> acc[12];
+// Hop number I in FP64, added to the lane's sums as fx_hop does: from the FP64 field that was converted to f where A.in
+// names it (src: its slice; of a canonical field if A.in.stride is 1), else from the parts (the first half-dslash of Mhat
+// left no other form).
+template <int I>
+__device__ __forceinline__ void fp64_hop(const HA& A, const FxField& f, const double2* src, const int* nb, int cb, int sp,
+                                         int m, Cx<double> (&v)[6]) {
+  constexpr int HOP = fx_order(I), MU = HOP >> 1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;
+  const int nbw = nb[HOP * (kWarps * kSB)], n = nbw & 0x7fffffff;
+  const int ku = 3 * sp, kl = 6 + 3 * (MU < 2 ? 1 - sp : sp);  // the first components of the two spins
+  Cx<double> u[3], l[3], h[3], U[9];
+  if (src) {
+    const bool canon = A.in.stride == 1;
+    const double2* p = src + (canon ? (long)canon_index(A.g, n, 1 - A.out_parity) * 12 : n);
 #pragma unroll
-  for (int k = 0; k < 12; ++k) acc[k] = {0.0, 0.0};
-  auto hop = [&](auto mu, bool back) {
-    constexpr int MU = decltype(mu)::value;
-    int wrap;
-    const int n = neighbour_index(A.g, c, MU, back ? -1 : +1, &wrap) >> 1;
-    const double sf = (wrap && A.g.apbc[MU]) ? -1.0 : 1.0, sgn = back ? -sg : sg;
-    const int e = f.e[n];
-    Cx<double> U[9], psi[12], h[6], gg[6];
-    A.U.load(back ? 1 - A.out_parity : A.out_parity, MU, back ? n : cb, U);
-    for (int k = 0; k < 12; ++k) {
-      if (src) {
-        const double2 v = src[canon ? (long)canon_index(A.g, n, 1 - A.out_parity) * 12 + k : k * A.in.stride + n];
-        psi[k] = {v.x, v.y};
-        continue;
-      }
-      const int4 u = f.p[(long)(n / kSB) * kSiteUnits + k * kSB + n % kSB];
-      if (e == kBad)
-        psi[k] = {__hiloint2double(u.y, u.x), __hiloint2double(u.w, u.z)};
-      else
-        psi[k] = {part_value({u.x, __int_as_float(u.y)}, e), part_value({u.z, __int_as_float(u.w)}, e)};
+    for (int c = 0; c < 3; ++c) {
+      const double2 x = __ldg(p + (ku + c) * A.in.stride), y = __ldg(p + (kl + c) * A.in.stride);
+      u[c] = {x.x, x.y};
+      l[c] = {y.x, y.y};
     }
-    project<MU>(psi, sgn, h);
-    if (back)
-      link_mul<true>(U, h, gg);
-    else
-      link_mul<false>(U, h, gg);
-    reconstruct_add<MU>(gg, sgn, sf, acc);
-  };
-  for (int back = 0; back < 2; ++back) {
-    hop(std::integral_constant<int, 0>{}, back);
-    hop(std::integral_constant<int, 1>{}, back);
-    hop(std::integral_constant<int, 2>{}, back);
-    hop(std::integral_constant<int, 3>{}, back);
-  }
-  for (int k = 0; k < 12; ++k) out[k] = acc[k];
-}
-
-// [x +] a H in of one site in FP64, stored
-__device__ __noinline__ void fp64_site_store(const HA& A, const FxField& f, int q, int cb, int r, long site) {
-  Cx<double> acc[12], o[12];
-  fp64_site(A, f, q, cb, acc);
-  if (A.xpay) {
-    A.x.offset_rhs(r).load(site, o);
-    for (int k = 0; k < 12; ++k) o[k] = fmac(A.a, acc[k], o[k]);
   } else {
-    for (int k = 0; k < 12; ++k) o[k] = A.a * acc[k];
+    const int e = f.e[n];
+    const int4* p = f.p + (long)(n / kSB) * kSiteUnits + n % kSB;
+    auto value = [&](int k) {
+      const int4 w = p[k * kSB];
+      return e == kBad ? Cx<double>{__hiloint2double(w.y, w.x), __hiloint2double(w.w, w.z)}
+                       : Cx<double>{part_value({w.x, __int_as_float(w.y)}, e), part_value({w.z, __int_as_float(w.w)}, e)};
+    };
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      u[c] = value(ku + c);
+      l[c] = value(kl + c);
+    }
   }
-  A.out.offset_rhs(r).store(site, o);
+  const double s = m * SG, sign = nbw < 0 ? -1.0 : 1.0;
+#pragma unroll
+  for (int c = 0; c < 3; ++c) {
+    if (MU == 0 || MU == 2)
+      h[c] = {sign * fma(s, l[c].im, u[c].re), sign * fma(-s, l[c].re, u[c].im)};
+    else
+      h[c] = {sign * fma(s, l[c].re, u[c].re), sign * fma(s, l[c].im, u[c].im)};
+  }
+  A.U.load((HOP & 1) ? 1 - A.out_parity : A.out_parity, MU, (HOP & 1) ? n : cb, U);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    Cx<double> w = {0.0, 0.0};
+#pragma unroll
+    for (int b = 0; b < 3; ++b) w = (HOP & 1) ? cjmadd(U[b * 3 + a], h[b], w) : cmadd(U[a * 3 + b], h[b], w);
+    v[a] = v[a] + w;
+    v[3 + a] = v[3 + a] + ((MU == 0 || MU == 2) ? Cx<double>{-SG * w.im, SG * w.re} : Cx<double>{SG * w.re, SG * w.im});
+  }
 }
 
-// H in of one site in FP64, stored in the fixed-point field o as a kBad site
-__device__ __noinline__ void fp64_site_store_fx(const HA& A, const FxField& f, const FxField& o, int q, int cb) {
-  Cx<double> acc[12];
-  fp64_site(A, f, q, cb, acc);
-  int4* p = o.p + (long)(cb / kSB) * kSiteUnits + cb % kSB;
-  for (int k = 0; k < 12; ++k)
-    p[k * kSB] = make_int4(__double2loint(acc[k].re), __double2hiint(acc[k].re), __double2loint(acc[k].im),
-                           __double2hiint(acc[k].im));
-  o.e[cb] = kBad;
+// The hop sums of the lane (upper spin sp, lower spin 2 + sp, the latter times -1 for H^dag) in FP64; the whole warp calls
+// it, since a site's two lanes share the work.  Bound by the FP64 pipe.  The full matrix on 24^3 x 32 where every site comes
+// here (a point source's solution, links within 1e-4 of 1): 1.11 ms, of which 0.82 are the FP64 kernel's; one
+// lane per site, 2.04.
+__device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, const int* nb, int cb, int sp,
+                                      Cx<double> (&out)[6]) {
+  const double2* src = A.in.p;
+  if (src) {
+    const int r = fdiv(q, A.d_ls);
+    src += A.in.stride == 1 ? (long)q * A.g.V * 12 : (long)r * 12 * A.in.stride + (long)(q - r * A.ls) * A.g.Vh;
+  }
+  const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
+  Cx<double> v[6];
+#pragma unroll
+  for (int k = 0; k < 6; ++k) v[k] = {0.0, 0.0};
+  auto turn = [&](bool minus) {
+#pragma unroll
+    for (int k = 3; k < 6; ++k) v[k] = minus ? -v[k] : v[k];
+  };
+  fp64_hop<0>(A, f, src, nb, cb, sp, -gs, v);  // signs and lanes as in fx_sum
+  fp64_hop<1>(A, f, src, nb, cb, sp, -gs, v);
+  turn(sp == 0);
+  fp64_hop<2>(A, f, src, nb, cb, sp, g5, v);
+  fp64_hop<3>(A, f, src, nb, cb, sp, g5, v);
+#pragma unroll
+  for (int k = 3; k < 6; ++k)
+    v[k] = {__shfl_xor_sync(0xffffffffu, v[k].re, kSB), __shfl_xor_sync(0xffffffffu, v[k].im, kSB)};
+  turn(sp != 0);
+  fp64_hop<4>(A, f, src, nb, cb, sp, gs, v);
+  fp64_hop<5>(A, f, src, nb, cb, sp, gs, v);
+  turn(sp != 0);
+  fp64_hop<6>(A, f, src, nb, cb, sp, g5, v);
+  fp64_hop<7>(A, f, src, nb, cb, sp, g5, v);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) out[k] = v[k];
 }
 
 // The exponent field of the site's largest neighbour (its neighbour indices go to shared memory).
@@ -436,8 +455,8 @@ __device__ __forceinline__ void flip(int64_t (&v)[6], bool minus) {
 // The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
 // 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Only then are the magnitudes formed (fx_exact, a
 // second walk over the hops), which settles all but fields with components far smaller than others that the links hardly
-// mix with them.  Without any of this the full matrix on 24^3 x 48 took 309 us instead of 319, a solve on 12x10x14x18 3.61 ms
-// instead of 3.75, and twelve point sources on 24^3 x 48, around which spins and colours differ most, 139 ms instead of 146.
+// mix with them.  Without any of this the full matrix on 24^3 x 48 took 309 us instead of 317, a solve on 12x10x14x18 3.56 ms
+// instead of 3.72, and twelve point sources on 24^3 x 48, around which spins and colours differ most, 138 ms instead of 144.
 __device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S, bool& slow) {
   const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
 #pragma unroll
@@ -483,7 +502,7 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
     mx |= (uint64_t)(lo[k] ^ (lo[k] >> 63));
   }
   mx |= __shfl_xor_sync(0xffffffffu, mx, kSB);
-  if (!valid || slow) return;  // slow: fp64_site_store_fx
+  if (!valid || slow) return;  // slow: fx_store_fp64
   const int b = 64 - __clzll((long long)mx);  // -2^b <= every sum < 2^b
   const int e = mx ? b + E - 57 : kZero, shift = b - 30;
   int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
@@ -506,6 +525,64 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
   if (sp == 0) out.e[cb] = wide ? kBad : e;
 }
 
+// a slow site's sums as a kBad site of that field
+__device__ __forceinline__ void fx_store_fp64(const FxField& out, int cb, int sp, bool minus_lo, const Cx<double> (&v)[6]) {
+  int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    const Cx<double> x = k >= 3 && minus_lo ? -v[k] : v[k];
+    o[(k < 3 ? k : 3 + k) * kSB] =
+        make_int4(__double2loint(x.re), __double2hiint(x.re), __double2loint(x.im), __double2hiint(x.im));
+  }
+  if (sp == 0) out.e[cb] = kBad;
+}
+
+// the sites and the slice of a lane
+struct FxLane {
+  int cb0, cb, sp, q, r;
+  bool valid, warp_valid;
+};
+__device__ __forceinline__ FxLane fx_lane(const HA& A) {
+  FxLane L;
+  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
+  L.q = blockIdx.x - sblock * A.ntiles;
+  L.r = fdiv(L.q, A.d_ls);
+  L.cb0 = (sblock * kWarps + (threadIdx.x >> 5)) * kSB;
+  L.cb = L.cb0 + threadIdx.x % kSB;
+  L.sp = (threadIdx.x & 31) / kSB;
+  L.valid = L.cb < A.g.Vh;
+  L.warp_valid = L.cb0 < A.g.Vh;
+  return L;
+}
+__device__ __forceinline__ FxField fx_slice(const FxField& F, int q) {
+  return {F.p + (long)q * F.nsb * kSiteUnits, F.e + (long)q * F.nsb * kSB, F.nsb};
+}
+
+// a H in for the lane's six components (upper spin sp, lower spin 2 + sp) as a[k / 3] v[k]; the whole warp calls it
+__device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField& f, const FxLane& L, Cx<double> (&v)[6],
+                                          double (&a)[2]) {
+  const int cb = L.valid ? L.cb : 0;
+  const int E = fx_neighbours(A, W, f, cb);
+  FxSum S;
+  bool slow;
+  const double unit = fx_sum(A, W, f, E, L.sp, S, slow);
+  if (__any_sync(0xffffffffu, slow)) {  // the warp's sites together: nothing of theirs has to be kept meanwhile
+    Cx<double> w[6];  // in memory, for the call: v stays in registers
+    fp64_sum(A, f, L.q, &W.sm->nb[0][W.warp * kSB + W.lane % kSB], cb, L.sp, w);
+    a[0] = A.a;
+#pragma unroll
+    for (int k = 0; k < 6; ++k) v[k] = w[k];
+  } else {
+    a[0] = A.a * unit;
+#pragma unroll
+    for (int c = 0; c < 3; ++c) {
+      v[c] = {(double)S.up[2 * c], (double)S.up[2 * c + 1]};
+      v[3 + c] = {(double)S.lo[2 * c], (double)S.lo[2 * c + 1]};
+    }
+  }
+  a[1] = A.dagger ? -a[0] : a[0];
+}
+
 // OUT = 0: [x +] a H in as FP64; OUT = 1: H in as the fixed-point field O
 template <int MINB, int OUT>
 __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_constant__ HA A,
@@ -514,53 +591,46 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_const
                                                               const __grid_constant__ FxField O) {
   extern __shared__ __align__(128) unsigned char smraw[];
   FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
-  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
-  const int q = blockIdx.x - sblock * A.ntiles;
-  const int cb0 = (sblock * kWarps + (threadIdx.x >> 5)) * kSB;  // the warp's first site
-  if (cb0 >= A.g.Vh) return;                                   // a whole warp
-  const int cb = cb0 + threadIdx.x % kSB, sp = (threadIdx.x & 31) / kSB;
-  const bool valid = cb < A.g.Vh;
-  FxWarp W = fx_begin(sm, links, (long)A.out_parity * F.nsb + cb0 / kSB);
+  const FxLane L = fx_lane(A);
+  if (!L.warp_valid) return;
+  FxWarp W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
   pdl_enter();
   if (A.stop && *A.stop) {
     fx_abandon(W);
     return;
   }
-  const int r = fdiv(q, A.d_ls), s = q - r * A.ls;
-  const long site = (long)s * A.g.Vh + cb;
-  const FxField f{F.p + (long)q * F.nsb * kSiteUnits, F.e + (long)q * F.nsb * kSB, F.nsb};
-  const int E = fx_neighbours(A, W, f, valid ? cb : 0);
-  FxSum S;
-  bool slow;
-  const double unit = fx_sum(A, W, f, E, sp, S, slow);
-  int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
+  const FxField f = fx_slice(F, L.q);
   if constexpr (OUT == 1) {
-    const FxField o{O.p + (long)q * O.nsb * kSiteUnits, O.e + (long)q * O.nsb * kSB, O.nsb};
-    fx_store(o, cb, sp, valid, E, A.dagger != 0, W.failed, slow, up, lo);
-    if (slow && valid && sp == 0) fp64_site_store_fx(A, f, o, q, cb);
-    return;
-  }
-  if (!valid) return;
-  if (slow) {
-    if (sp == 0) fp64_site_store(A, f, q, cb, r, site);
-    return;
-  }
-  const double au = A.a * unit, al = A.dagger ? -au : au;
-  const long xstr = A.x.stride, ostr = A.out.stride;
-  const double2* x = A.x.offset_rhs(r).p + 3 * sp * xstr + site;
-  double2* o = A.out.offset_rhs(r).p + 3 * sp * ostr + site;
-  if (A.xpay) {
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      const double2 xu = __ldg(x + c * xstr), xl = __ldg(x + (6 + c) * xstr);
-      o[c * ostr] = make_double2(fma(au, (double)up[2 * c], xu.x), fma(au, (double)up[2 * c + 1], xu.y));
-      o[(6 + c) * ostr] = make_double2(fma(al, (double)lo[2 * c], xl.x), fma(al, (double)lo[2 * c + 1], xl.y));
+    const int cb = L.valid ? L.cb : 0;
+    const int E = fx_neighbours(A, W, f, cb);
+    FxSum S;
+    bool slow;
+    fx_sum(A, W, f, E, L.sp, S, slow);
+    const FxField o = fx_slice(O, L.q);
+    fx_store(o, L.cb, L.sp, L.valid, E, A.dagger != 0, W.failed, slow, S.up, S.lo);
+    if (__any_sync(0xffffffffu, slow)) {
+      Cx<double> v[6];
+      fp64_sum(A, f, L.q, &sm.nb[0][W.warp * kSB + W.lane % kSB], cb, L.sp, v);
+      if (slow && L.valid) fx_store_fp64(o, L.cb, L.sp, A.dagger != 0, v);
     }
-  } else {
+    return;
+  }
+  Cx<double> v[6];
+  double a[2];
+  fx_values(A, W, f, L, v, a);
+  if (!L.valid) return;
+  const long site = (long)(L.q - L.r * A.ls) * A.g.Vh + L.cb;
+  const long xstr = A.x.stride, ostr = A.out.stride;
+  const double2* x = A.x.offset_rhs(L.r).p + 3 * L.sp * xstr + site;
+  double2* o = A.out.offset_rhs(L.r).p + 3 * L.sp * ostr + site;
 #pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      o[c * ostr] = make_double2(au * (double)up[2 * c], au * (double)up[2 * c + 1]);
-      o[(6 + c) * ostr] = make_double2(al * (double)lo[2 * c], al * (double)lo[2 * c + 1]);
+  for (int k = 0; k < 6; ++k) {
+    const int n = k < 3 ? k : 3 + k;
+    if (A.xpay) {
+      const double2 xs = __ldg(x + n * xstr);
+      o[n * ostr] = make_double2(fma(a[k / 3], v[k].re, xs.x), fma(a[k / 3], v[k].im, xs.y));
+    } else {
+      o[n * ostr] = make_double2(a[k / 3] * v[k].re, a[k / 3] * v[k].im);
     }
   }
 }
@@ -572,44 +642,30 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx_red(const __grid_c
                                                                   const __grid_constant__ FxField F) {
   extern __shared__ __align__(128) unsigned char smraw[];
   FxShared& sm = *reinterpret_cast<FxShared*>(smraw);
-  const int cb0 = (blockIdx.x * kWarps + (threadIdx.x >> 5)) * kSB;
-  const int cb = cb0 + threadIdx.x % kSB, sp = (threadIdx.x & 31) / kSB;
-  const bool valid = cb < A.g.Vh, warp_valid = cb0 < A.g.Vh;
+  const FxLane L = fx_lane(A);  // one slice
   FxWarp W;
-  if (warp_valid) W = fx_begin(sm, links, (long)A.out_parity * F.nsb + cb0 / kSB);
+  if (L.warp_valid) W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
   pdl_enter();
   if (A.stop && *A.stop) {
-    if (warp_valid) fx_abandon(W);
+    if (L.warp_valid) fx_abandon(W);
     return;
   }
   double red[3] = {0.0, 0.0, 0.0};
-  if (warp_valid) {
-    const int E = fx_neighbours(A, W, F, valid ? cb : 0);
-    FxSum S;
-    bool bad;
-    const double unit = fx_sum(A, W, F, E, sp, S, bad);
-    if (bad && valid && sp == 0) fp64_site_store(A, F, 0, cb, 0, cb);
-    __syncwarp();
-    int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
-    const double au = A.a * unit, al = A.dagger ? -au : au;
-    if (valid) {
-      const double2* x = A.x.p + 3 * sp * A.x.stride + cb;
-      const double2* rt = A.rt.p + 3 * sp * A.rt.stride + cb;
-      double2* out = A.out.p + 3 * sp * A.out.stride + cb;
+  if (L.warp_valid) {
+    Cx<double> v[6];
+    double a[2];
+    fx_values(A, W, F, L, v, a);
+    if (L.valid) {
+      const double2* x = A.x.p + 3 * L.sp * A.x.stride + L.cb;
+      const double2* rt = A.rt.p + 3 * L.sp * A.rt.stride + L.cb;
+      double2* out = A.out.p + 3 * L.sp * A.out.stride + L.cb;
       Cx<double> d = {0.0, 0.0};
 #pragma unroll
       for (int k = 0; k < 6; ++k) {  // colour k of spin sp, colour k - 3 of spin 2 + sp
-        const int c = k % 3, n = k < 3 ? c : 6 + c;
-        const double a = k < 3 ? au : al;
-        const double vr = (double)(k < 3 ? up[2 * c] : lo[2 * c]), vi = (double)(k < 3 ? up[2 * c + 1] : lo[2 * c + 1]);
+        const int n = k < 3 ? k : 3 + k;
         const double2 xs = __ldg(x + n * A.x.stride);
-        Cx<double> o = {fma(a, vr, xs.x), fma(a, vi, xs.y)};
-        if (bad) {  // as stored above
-          const volatile double2* w = out + n * A.out.stride;
-          o = {w->x, w->y};
-        } else {
-          out[n * A.out.stride] = make_double2(o.re, o.im);
-        }
+        const Cx<double> o = {fma(a[k / 3], v[k].re, xs.x), fma(a[k / 3], v[k].im, xs.y)};
+        out[n * A.out.stride] = make_double2(o.re, o.im);
         if (RED == 1) {  // (rt, out)
           const double2 w = __ldg(rt + n * A.rt.stride);
           d = cjmadd(Cx<double>{w.x, w.y}, o, d);
@@ -678,50 +734,6 @@ __global__ void __launch_bounds__(128) k_outer_x(SpinorView<P64> x, SpinorView<P
   fx_put(w, e, out, (long)blockIdx.y * out.nsb, cb);
 }
 
-// acc = the sum of the eight hops in FP64 values with factor a (slow path: fp64_site); the lane's six components,
-// upper spin sp then lower spin 2 + sp.  false: the warp has no such site.
-struct FxLane {
-  int cb0, cb, sp, q, r;
-  bool valid, warp_valid;
-};
-__device__ __forceinline__ FxLane fx_lane(const HA& A) {
-  FxLane L;
-  const int sblock = fdiv(blockIdx.x, A.d_ntiles);
-  L.q = blockIdx.x - sblock * A.ntiles;
-  L.r = L.q;  // Wilson: one slice per right-hand side
-  L.cb0 = (sblock * kWarps + (threadIdx.x >> 5)) * kSB;
-  L.cb = L.cb0 + threadIdx.x % kSB;
-  L.sp = (threadIdx.x & 31) / kSB;
-  L.valid = L.cb < A.g.Vh;
-  L.warp_valid = L.cb0 < A.g.Vh;
-  return L;
-}
-
-// a H in for the lane's six components (upper spin sp, lower spin 2 + sp) as a[k / 3] v[k]
-__device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField& f, const FxLane& L, Cx<double> v[6],
-                                          double a[2]) {
-  const int E = fx_neighbours(A, W, f, L.valid ? L.cb : 0);
-  FxSum S;
-  bool bad;
-  const double unit = fx_sum(A, W, f, E, L.sp, S, bad);
-  int64_t(&up)[6] = S.up, (&lo)[6] = S.lo;
-  a[0] = A.a * unit;
-  a[1] = A.dagger ? -a[0] : a[0];
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    v[c] = {(double)up[2 * c], (double)up[2 * c + 1]};
-    v[3 + c] = {(double)lo[2 * c], (double)lo[2 * c + 1]};
-  }
-  if (bad && L.valid) {
-    Cx<double> slow[12];
-    fp64_site(A, f, L.q, L.cb, slow);  // both lanes of the site
-    a[0] = a[1] = A.a;
-    const Cx<double>* w = slow + 3 * L.sp;
-#pragma unroll
-    for (int n = 0; n < 6; ++n) v[n] = w[n < 3 ? n : 3 + n];
-  }
-}
-
 // out = x + a H in, FP64 and as the fixed-point field O; partial k = 1: |x - out + a H in|^2, the rounding of out
 __global__ void __launch_bounds__(32 * kWarps, 4) k_outer_odd(const __grid_constant__ HA A,
                                                               const int4* __restrict__ links,
@@ -735,7 +747,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_outer_odd(const __grid_const
   pdl_enter();
   double res = 0.0;
   if (L.warp_valid) {
-    const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+    const FxField f = fx_slice(F, L.q);
     Cx<double> h[6];
     double a[2];
     fx_values(A, W, f, L, h, a);
@@ -791,7 +803,7 @@ __global__ void __launch_bounds__(32 * kWarps, 4) k_outer_res(const __grid_const
   pdl_enter();
   double res = 0.0;
   if (L.warp_valid) {
-    const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+    const FxField f = fx_slice(F, L.q);
     Cx<double> h[6];
     double a[2];
     fx_values(A, W, f, L, h, a);
@@ -893,7 +905,7 @@ __global__ void __launch_bounds__(32 * kWarps, 5) k_hop_fx_canon(const __grid_co
   if (!L.warp_valid) return;
   FxWarp W = fx_begin(sm, links, (long)A.out_parity * F.nsb + L.cb0 / kSB);
   pdl_enter();
-  const FxField f{F.p + (long)L.q * F.nsb * kSiteUnits, F.e + (long)L.q * F.nsb * kSB, F.nsb};
+  const FxField f = fx_slice(F, L.q);
   const long first = (long)L.q * A.g.V * 12;
   const double2* xs = x + first + (long)canon_index(A.g, L.valid ? L.cb : 0, A.out_parity) * 12;
   Cx<double> h[6];
