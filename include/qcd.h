@@ -311,6 +311,9 @@ qcd_status qcd_norm2(const qcd_gauge* g, const qcd_fermion* fermion, const void*
  *                          scheduled while its predecessor drains; results are
  *                          the same either way);
  *   QCD_FAULT=alloc        every device workspace allocation fails (QCD_ERR_OOM);
+ *   QCD_FAULT=oom          CUDA refuses the first attempt at every device workspace
+ *                          allocation: buffers that are only for speed are done
+ *                          without or given back, the others are then allocated;
  *   QCD_FAULT=nan          qcd_solve poisons its inner residual with NaN after the
  *                          first restart, which the device reductions must report
  *                          (QCD_ERR_NAN);

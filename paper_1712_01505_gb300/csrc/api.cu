@@ -79,6 +79,10 @@ Field Field::rhs_range(int r0, int n) const {
   return f;
 }
 
+namespace {
+bool is_optional(const std::string& name) { return name.compare(0, 4, "opt.") == 0; }
+}  // namespace
+
 void* Workspace::get(const std::string& name, size_t bytes) {
   if (bytes == 0) bytes = 16;
   auto it = bufs.find(name);
@@ -86,25 +90,36 @@ void* Workspace::get(const std::string& name, size_t bytes) {
   if (it != bufs.end()) {
     QCD_CK(cudaFree(it->second.p));
     bufs.erase(it);
+    ++generation;  // also if the new one is refused
   }
-  if (getenv("QCD_FAULT") && strcmp(getenv("QCD_FAULT"), "alloc") == 0)
+  const char* fault = getenv("QCD_FAULT");
+  if (fault && strcmp(fault, "alloc") == 0)
     raise(QCD_ERR_OOM, "workspace allocation of %zu bytes refused (QCD_FAULT=alloc)", bytes);
+  // QCD_FAULT=oom: the first attempt asks for more than any device has
+  const bool refuse = fault && strcmp(fault, "oom") == 0;
   void* p = nullptr;
-  cudaError_t e = cudaMalloc(&p, bytes);
-  if (e == cudaErrorMemoryAllocation && drop_optional()) {
-    cudaGetLastError();
-    e = cudaMalloc(&p, bytes);
+  cudaError_t e = cudaMalloc(&p, refuse ? (size_t)1 << 60 : bytes);
+  if (e == cudaErrorMemoryAllocation) {
+    cudaGetLastError();  // else the next launch check would report it
+    // an optional buffer is done without; for any other the optional ones give way
+    if (!is_optional(name) && (drop_optional() || refuse)) e = cudaMalloc(&p, bytes);
   }
+  if (e != cudaSuccess) cudaGetLastError();
   QCD_CK(e);
   bufs[name] = {p, bytes};
   ++generation;
   return p;
 }
 
+bool Workspace::has(const std::string& name, size_t bytes) const {
+  auto it = bufs.find(name);
+  return it != bufs.end() && it->second.bytes >= bytes;
+}
+
 bool Workspace::drop_optional() {
   bool any = false;
   for (auto it = bufs.begin(); it != bufs.end();) {
-    if (it->first.compare(0, 4, "opt.") == 0) {
+    if (is_optional(it->first)) {
       cudaFree(it->second.p);  // waits for the device
       it = bufs.erase(it);
       any = true;
@@ -315,7 +330,6 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
       QCD_CK(cudaMemcpyAsync(&fx_bad, fx_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
     } catch (const Error& e) {
       if (e.status != QCD_ERR_OOM) throw;
-      cudaGetLastError();
     }
     QCD_CK(cudaStreamSynchronize(st));
     g->fx_ok = fx_bad == 0;

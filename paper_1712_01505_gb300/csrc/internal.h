@@ -101,9 +101,10 @@ struct Workspace {
   std::map<std::string, Buf> bufs;
   long generation = 0;  // bumped whenever a buffer is (re)allocated or freed
   // Buffers named "opt.*" speed things up but are not needed: when the device is out of memory they are
-  // given back (and *opt_in_use cleared) before an allocation fails.
+  // given back (and *opt_in_use cleared) before an allocation of another buffer fails.
   bool* opt_in_use = nullptr;
   void* get(const std::string& name, size_t bytes);
+  bool has(const std::string& name, size_t bytes) const;  // get() would return it as it is
   bool drop_optional();
   void release();
 };

@@ -1016,10 +1016,18 @@ SpinorView<P64> fx_view(const Field& f) {
   return v;
 }
 
-// A scratch field of the handle.
-FxField fx_scratch(qcd_gauge* g, const char* name, const Field& like) {
+bool capturing(cudaStream_t st) {
+  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
+  QCD_CK(cudaStreamIsCapturing(st, &cs));
+  return cs != cudaStreamCaptureStatusNone;
+}
+
+// A scratch field of the handle; not allocated while the solver captures its iterations, which then run
+// without it as the uncaptured first one did.
+FxField fx_scratch(qcd_gauge* g, const char* name, const Field& like, cudaStream_t st) {
   const long nsb = (like.Vh + kSB - 1) / kSB, nq = (long)like.ls * like.nrhs;
   const size_t data = (size_t)nq * nsb * kSiteUnits * sizeof(int4), exps = (size_t)nq * nsb * kSB * sizeof(int);
+  if (!g->ws.has(name, data + exps) && capturing(st)) raise(QCD_ERR_OOM, "no scratch for the fixed-point stencil");
   char* p = (char*)g->ws.get(name, data + exps);
   return {(int4*)p, (int*)(p + data), nsb};
 }
@@ -1113,10 +1121,7 @@ struct FxOrder {
 // outlives the call must not hold the handle's scratch).
 bool fx_usable(const qcd_gauge* g, cudaStream_t st) {
   if (!g->fx_ok) return false;
-  if (st == g->work) return true;
-  cudaStreamCaptureStatus cs = cudaStreamCaptureStatusNone;
-  QCD_CK(cudaStreamIsCapturing(st, &cs));
-  return cs == cudaStreamCaptureStatusNone;
+  return st == g->work || !capturing(st);
 }
 
 }  // namespace
@@ -1137,12 +1142,11 @@ bool hop_fx(const qcd_gauge* gh, const Field& in, Field& out, int out_parity, in
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   FxField f;
   try {
-    f = fx_scratch(g, "opt.fx.a", in);
+    f = fx_scratch(g, "opt.fx.a", in, st);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  if (!g->fx_ok) return false;  // the links gave way to another allocation
   FxOrder order(g, st);
   fx_pack(in, f, st, stop);
   const SpinorView<P64> src = fx_view(in);
@@ -1157,14 +1161,12 @@ bool mhat_fx(const qcd_gauge* gh, const Field& in, Field& out, int dagger, doubl
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   FxField f, t;
   try {
-    fx_scratch(g, "opt.fx.a", in);
-    t = fx_scratch(g, "opt.fx.b", in);
-    if (g->fx_ok) f = fx_scratch(g, "opt.fx.a", in);
+    f = fx_scratch(g, "opt.fx.a", in, st);
+    t = fx_scratch(g, "opt.fx.b", in, st);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  if (!g->fx_ok) return false;
   FxOrder order(g, st);
   fx_pack(in, f, st, stop);
   const SpinorView<P64> src = fx_view(in);
@@ -1178,23 +1180,23 @@ bool outer_fx_ready(const qcd_gauge* gh, const Field& shape, cudaStream_t st) {
   if (!fx_usable(gh, st)) return false;
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   try {
-    fx_scratch(g, "opt.fx.a", shape);
-    fx_scratch(g, "opt.fx.b", shape);
+    fx_scratch(g, "opt.fx.a", shape, st);
+    fx_scratch(g, "opt.fx.b", shape, st);
     const size_t nb = (size_t)(shape.Vh + kWarps * kSB - 1) / (kWarps * kSB);
-    g->ws.get("s.outer", sizeof(double) * 4 * nb * shape.nrhs);
+    g->ws.get("opt.fx.sums", sizeof(double) * 4 * nb * shape.nrhs);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  return g->fx_ok;
+  return true;
 }
 
 void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   const Field& shape = o.x;
-  const FxField fa = fx_scratch(g, "opt.fx.a", shape), fb = fx_scratch(g, "opt.fx.b", shape);
+  const FxField fa = fx_scratch(g, "opt.fx.a", shape, st), fb = fx_scratch(g, "opt.fx.b", shape, st);
   const unsigned nb = (unsigned)((shape.Vh + kWarps * kSB - 1) / (kWarps * kSB)), n = (unsigned)shape.nrhs;
-  double* partial = (double*)g->ws.get("s.outer", sizeof(double) * 4 * nb * n);
+  double* partial = (double*)g->ws.get("opt.fx.sums", sizeof(double) * 4 * nb * n);
   const int4* links = (const int4*)g->Ufx;
   static std::atomic<unsigned long long> attr_mask{0};
   if (first_use_on_device(attr_mask))
@@ -1253,14 +1255,12 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
   shape.nrhs = nrhs;
   FxField fa, fb;
   try {
-    fx_scratch(g, "opt.fx.a", shape);
-    fb = fx_scratch(g, "opt.fx.b", shape);
-    if (g->fx_ok) fa = fx_scratch(g, "opt.fx.a", shape);
+    fa = fx_scratch(g, "opt.fx.a", shape, st);
+    fb = fx_scratch(g, "opt.fx.b", shape, st);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  if (!g->fx_ok) return false;
   static std::atomic<unsigned long long> attr_mask{0};
   if (first_use_on_device(attr_mask))
     QCD_CK(cudaFuncSetAttribute(k_hop_fx_canon, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared)));
