@@ -270,30 +270,8 @@ Field internal_field(const qcd_gauge* g, int prec, int ls, int nrhs, const void*
 }
 
 }  // namespace
-}  // namespace qcd
 
-using namespace qcd;
-
-extern "C" {
-
-const char* qcd_last_error(void) { return t_err.c_str(); }
-
-qcd_status qcd_kernel_launches(uint64_t* count) {
-  return guarded([&] {
-    if (!count) raise(QCD_ERR_ARG, "count is NULL");
-    *count = (uint64_t)launches_so_far();
-  });
-}
-
-qcd_status qcd_set_tuning(int32_t mode) {
-  return guarded([&] {
-    if (mode != 0 && mode != 1) raise(QCD_ERR_ARG, "tuning mode must be 0 or 1");
-    set_tuning(mode);
-  });
-}
-
-qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd_gauge** out) {
-  NvtxRange nvtx_range("qcd_gauge_load");
+qcd_status gauge_load(const qcd_geom* geom, const void* U, void* stream, bool fixed_point, qcd_gauge** out) {
   qcd_gauge* g = nullptr;
   qcd_status s = guarded([&] {
     check_geom(geom);
@@ -322,18 +300,20 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
     gauge_reorder(g, su.dev, st);
     links_to_df(g, st);
     int fx_bad = 1;
-    g->ws.opt_in_use = &g->fx_ok;
-    try {  // optional: without it the FP64 stencil runs on U64
-      g->Ufx = g->ws.get("opt.Ufx", fx_link_bytes(lat) + sizeof(int));
-      int* fx_flag = (int*)((char*)g->Ufx + fx_link_bytes(lat));
-      links_to_fx(g, fx_flag, st);
-      QCD_CK(cudaMemcpyAsync(&fx_bad, fx_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
-    } catch (const Error& e) {
-      if (e.status != QCD_ERR_OOM) throw;
+    if (fixed_point) {
+      g->ws.opt_in_use = &g->fx_ok;
+      try {  // optional: without it the FP64 stencil runs on U64
+        g->Ufx = g->ws.get("opt.Ufx", fx_link_bytes(lat) + sizeof(int));
+        int* fx_flag = (int*)((char*)g->Ufx + fx_link_bytes(lat));
+        links_to_fx(g, fx_flag, st);
+        QCD_CK(cudaMemcpyAsync(&fx_bad, fx_flag, sizeof(int), cudaMemcpyDeviceToHost, st));
+      } catch (const Error& e) {
+        if (e.status != QCD_ERR_OOM) throw;
+      }
     }
     QCD_CK(cudaStreamSynchronize(st));
     g->fx_ok = fx_bad == 0;
-    if (!g->fx_ok) g->ws.drop_optional();  // links that are not of unit size
+    if (fixed_point && !g->fx_ok) g->ws.drop_optional();  // links that are not of unit size
   });
   if (s != QCD_OK) {
     if (g) {
@@ -352,6 +332,33 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
   }
   *out = g;
   return QCD_OK;
+}
+
+}  // namespace qcd
+
+using namespace qcd;
+
+extern "C" {
+
+const char* qcd_last_error(void) { return t_err.c_str(); }
+
+qcd_status qcd_kernel_launches(uint64_t* count) {
+  return guarded([&] {
+    if (!count) raise(QCD_ERR_ARG, "count is NULL");
+    *count = (uint64_t)launches_so_far();
+  });
+}
+
+qcd_status qcd_set_tuning(int32_t mode) {
+  return guarded([&] {
+    if (mode != 0 && mode != 1) raise(QCD_ERR_ARG, "tuning mode must be 0 or 1");
+    set_tuning(mode);
+  });
+}
+
+qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd_gauge** out) {
+  NvtxRange nvtx_range("qcd_gauge_load");
+  return gauge_load(geom, U, stream, true, out);
 }
 
 qcd_status qcd_gauge_free(qcd_gauge* g) {

@@ -828,9 +828,9 @@ void dd_create(const qcd_dd_geom* geom, int nlocal, const int32_t* ids, const vo
         lg.bc[m] = ((d->cut >> m) & 1) ? 1 : d->bc[m];  // cut directions never wrap locally
       }
       lg.recon = d->recon;
-      const qcd_status stt = qcd_gauge_load(&lg, U[k], st, &s.g);
+      // the subdomains' stencils run on the plain link copies
+      const qcd_status stt = gauge_load(&lg, U[k], st, false, &s.g);
       if (stt != QCD_OK) raise(stt, "subdomain %d: %s", s.id, qcd_last_error());
-      s.g->ws.drop_optional();  // the subdomains' stencils run on the plain link copies
       d->subs.push_back(s);  // owned from here on (freed with the handle)
       Sub& sb = d->subs.back();
       sb.halo = sb.g->ws.get("dd.halo", halo_bytes(d, QCD_F64));

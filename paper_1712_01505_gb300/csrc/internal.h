@@ -213,6 +213,8 @@ struct OuterStep {
 };
 bool outer_fx_ready(const qcd_gauge* g, const Field& shape, cudaStream_t st);
 void outer_fx(const qcd_gauge* g, const OuterStep& o, cudaStream_t st);
+// qcd_gauge_load; without the fixed-point form of the links if the handle's FP64 stencils will not use it
+qcd_status gauge_load(const qcd_geom* geom, const void* U, void* stream, bool fixed_point, qcd_gauge** out);
 // Ufx from U64; *flag (device) becomes nonzero if a link's size is outside the fixed-point range
 size_t fx_link_bytes(const Lattice& lat);
 void links_to_fx(qcd_gauge* g, int* flag, cudaStream_t st);
