@@ -183,9 +183,12 @@ typedef struct qcd_gauge qcd_gauge;
  * even-odd reordered copies in FP64 (18 reals), in FP32 and FP16 (geom->recon
  * reals), in double-float (18 hi/lo FP32 pairs) and, where every link row and
  * column has a 2-norm in [1/2, 5/4], in fixed point for both ends of each link
- * (used by the FP64 operators; given back when device memory runs out, the FP64
- * operators then use the FP64 copy); the caller's buffer is not referenced after
- * the call returns.
+ * (1152 bytes per site, used by the FP64 operators).  The fixed-point form is
+ * done without if it does not fit, and is given back, until the handle is freed,
+ * when a workspace of this handle, or of another one while no call uses this one,
+ * does not fit otherwise; the FP64 operators then use the FP64 copy.  Other
+ * allocators of the process do not get it back.  The caller's buffer is not
+ * referenced after the call returns.
  * Errors: QCD_ERR_ARG for a NULL pointer, odd or non-positive extents, bc not
  * +-1, recon not 12/18, or V >= 2^31; QCD_ERR_OOM if the copies do not fit. */
 qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd_gauge** out);

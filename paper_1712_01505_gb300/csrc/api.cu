@@ -6,6 +6,8 @@
 #include <cstdarg>
 #include <cstdio>
 #include <cstring>
+#include <mutex>
+#include <set>
 #include <string>
 
 #include <nvtx3/nvToolsExt.h>
@@ -80,8 +82,46 @@ Field Field::rhs_range(int r0, int n) const {
 }
 
 namespace {
+// Every workspace of the process, for giving optional buffers back between handles.  Never destroyed: handles may
+// be freed while the process exits.
+std::mutex& registry_mutex() {
+  static std::mutex* m = new std::mutex;
+  return *m;
+}
+std::set<Workspace*>& registry() {
+  static std::set<Workspace*>* s = new std::set<Workspace*>;
+  return *s;
+}
+
+// the optional buffers of the other handles on the device that have some (opt_in_use) and that no call is using
+bool drop_others(const Workspace* self) {
+  std::lock_guard<std::mutex> lk(registry_mutex());
+  bool any = false;
+  for (Workspace* w : registry())
+    if (w != self && w->device == self->device && w->users == 0 && w->opt_in_use && w->drop_optional()) any = true;
+  return any;
+}
+
 bool is_optional(const std::string& name) { return name.compare(0, 4, "opt.") == 0; }
 }  // namespace
+
+Workspace::Workspace() {
+  std::lock_guard<std::mutex> lk(registry_mutex());
+  registry().insert(this);
+}
+Workspace::~Workspace() {
+  std::lock_guard<std::mutex> lk(registry_mutex());
+  registry().erase(this);
+}
+
+OptUse::OptUse(const qcd_gauge* g) : ws_(const_cast<qcd_gauge*>(g)->ws) {
+  std::lock_guard<std::mutex> lk(registry_mutex());
+  ++ws_.users;
+}
+OptUse::~OptUse() {
+  std::lock_guard<std::mutex> lk(registry_mutex());
+  --ws_.users;
+}
 
 void* Workspace::get(const std::string& name, size_t bytes) {
   if (bytes == 0) bytes = 16;
@@ -102,7 +142,13 @@ void* Workspace::get(const std::string& name, size_t bytes) {
   if (e == cudaErrorMemoryAllocation) {
     cudaGetLastError();  // else the next launch check would report it
     // an optional buffer is done without; for any other the optional ones give way
-    if (!is_optional(name) && (drop_optional() || refuse)) e = cudaMalloc(&p, bytes);
+    if (!is_optional(name)) {
+      if (drop_optional()) e = cudaMalloc(&p, bytes);
+      if (e == cudaErrorMemoryAllocation && (drop_others(this) || refuse)) {
+        cudaGetLastError();
+        e = cudaMalloc(&p, bytes);
+      }
+    }
   }
   if (e != cudaSuccess) cudaGetLastError();
   QCD_CK(e);
@@ -269,6 +315,21 @@ Field internal_field(const qcd_gauge* g, int prec, int ls, int nrhs, const void*
   return f;
 }
 
+void destroy(qcd_gauge* g) {
+  {
+    OptUse use(g);
+    cudaDeviceSynchronize();
+    for (auto& kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
+    g->graphs.clear();
+    g->ws.release();
+  }
+  if (g->work) cudaStreamDestroy(g->work);
+  if (g->ev_in) cudaEventDestroy(g->ev_in);
+  if (g->ev_out) cudaEventDestroy(g->ev_out);
+  if (g->fx_ev) cudaEventDestroy(g->fx_ev);
+  delete g;
+}
+
 }  // namespace
 
 qcd_status gauge_load(const qcd_geom* geom, const void* U, void* stream, bool fixed_point, qcd_gauge** out) {
@@ -279,6 +340,8 @@ qcd_status gauge_load(const qcd_geom* geom, const void* U, void* stream, bool fi
     cudaStream_t st = (cudaStream_t)stream;
     g = new qcd_gauge();
     QCD_CK(cudaGetDevice(&g->device));
+    g->ws.device = g->device;
+    OptUse use(g);
     Lattice& lat = g->lat;
     for (int m = 0; m < 4; ++m) {
       lat.L[m] = geom->L[m];
@@ -316,17 +379,7 @@ qcd_status gauge_load(const qcd_geom* geom, const void* U, void* stream, bool fi
     if (fixed_point && !g->fx_ok) g->ws.drop_optional();  // links that are not of unit size
   });
   if (s != QCD_OK) {
-    if (g) {
-      cudaDeviceSynchronize();
-      for (auto& kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
-      g->graphs.clear();
-      g->ws.release();
-      if (g->work) cudaStreamDestroy(g->work);
-      if (g->ev_in) cudaEventDestroy(g->ev_in);
-      if (g->ev_out) cudaEventDestroy(g->ev_out);
-      if (g->fx_ev) cudaEventDestroy(g->fx_ev);
-      delete g;
-    }
+    if (g) destroy(g);
     if (out) *out = nullptr;
     return s;
   }
@@ -363,16 +416,7 @@ qcd_status qcd_gauge_load(const qcd_geom* geom, const void* U, void* stream, qcd
 
 qcd_status qcd_gauge_free(qcd_gauge* g) {
   return guarded([&] {
-    if (!g) return;
-    cudaDeviceSynchronize();
-    for (auto& kv : g->graphs) cudaGraphExecDestroy(kv.second.exec);
-    g->graphs.clear();
-    g->ws.release();
-    cudaStreamDestroy(g->work);
-    cudaEventDestroy(g->ev_in);
-    cudaEventDestroy(g->ev_out);
-    if (g->fx_ev) cudaEventDestroy(g->fx_ev);
-    delete g;
+    if (g) destroy(g);
   });
 }
 
@@ -398,6 +442,7 @@ qcd_status qcd_field_pack(const qcd_gauge* gc, const qcd_fermion* fermion, qcd_p
   NvtxRange nvtx_range("qcd_field_pack");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     qcd_gauge* g = const_cast<qcd_gauge*>(gc);
     int ls = check_fermion(fermion);
     check_prec(prec);
@@ -418,6 +463,7 @@ qcd_status qcd_field_unpack(const qcd_gauge* gc, const qcd_fermion* fermion, qcd
   NvtxRange nvtx_range("qcd_field_unpack");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     qcd_gauge* g = const_cast<qcd_gauge*>(gc);
     int ls = check_fermion(fermion);
     check_prec(prec);
@@ -439,6 +485,7 @@ qcd_status qcd_dslash(const qcd_gauge* gc, const qcd_fermion* fermion, qcd_prec 
   NvtxRange nvtx_range("qcd_dslash");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     qcd_gauge* g = const_cast<qcd_gauge*>(gc);
     int ls = check_fermion(fermion);
     check_prec(prec);
@@ -512,6 +559,7 @@ qcd_status qcd_solve(const qcd_gauge* gc, const qcd_fermion* fermion, const qcd_
   NvtxRange nvtx_range("qcd_solve");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     qcd_gauge* g = const_cast<qcd_gauge*>(gc);
     int ls = check_fermion(fermion);
     if (!params || !b || !x || !info) raise(QCD_ERR_ARG, "NULL argument");
@@ -553,6 +601,7 @@ qcd_status qcd_norm2(const qcd_gauge* gc, const qcd_fermion* fermion, const void
   NvtxRange nvtx_range("qcd_norm2");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     qcd_gauge* g = const_cast<qcd_gauge*>(gc);
     int ls = check_fermion(fermion);
     if (!psi || !out) raise(QCD_ERR_ARG, "NULL argument");
@@ -569,6 +618,7 @@ qcd_status qcd_mhat_noalloc(const qcd_gauge* gc, const qcd_fermion* fermion, qcd
                             int32_t dagger, const void* in, void* out, int32_t nrhs, void* stream) {
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     check_fermion(fermion);
     if (fermion->type != QCD_WILSON) raise(QCD_ERR_UNSUPPORTED, "qcd_mhat_noalloc is for Wilson fermions");
     check_prec(prec);
@@ -588,6 +638,7 @@ qcd_status qcd_force(const qcd_gauge* gc, const qcd_fermion* fermion, const void
   NvtxRange nvtx_range("qcd_force");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     check_fermion(fermion);
     if (fermion->type != QCD_WILSON) raise(QCD_ERR_UNSUPPORTED, "the force is implemented for Wilson fermions");
     if (!X || !eta || !dSdU) raise(QCD_ERR_ARG, "NULL argument");
@@ -602,6 +653,7 @@ qcd_status qcd_force_eo(const qcd_gauge* gc, const qcd_fermion* fermion, const v
   NvtxRange nvtx_range("qcd_force_eo");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     check_fermion(fermion);
     if (fermion->type != QCD_WILSON) raise(QCD_ERR_UNSUPPORTED, "the force is implemented for Wilson fermions");
     if (!X || !Y || !dSdU) raise(QCD_ERR_ARG, "NULL argument");
@@ -616,6 +668,7 @@ qcd_status qcd_force_project(const qcd_gauge* gc, const void* dSdU, void* F, voi
   NvtxRange nvtx_range("qcd_force_project");
   return guarded([&] {
     check_gauge(gc);
+    OptUse use(gc);
     if (!dSdU || !F) raise(QCD_ERR_ARG, "NULL argument");
     if (dSdU == F) raise(QCD_ERR_ARG, "dSdU and F must not overlap");
     if (!is_device_ptr(dSdU) || !is_device_ptr(F)) raise(QCD_ERR_ARG, "qcd_force_project takes device buffers");

@@ -101,12 +101,29 @@ struct Workspace {
   std::map<std::string, Buf> bufs;
   long generation = 0;  // bumped whenever a buffer is (re)allocated or freed
   // Buffers named "opt.*" speed things up but are not needed: when the device is out of memory they are
-  // given back (and *opt_in_use cleared) before an allocation of another buffer fails.
+  // given back (and *opt_in_use cleared) before an allocation of another buffer fails, those of this
+  // handle first, then those of the process's other handles that no call is using.
   bool* opt_in_use = nullptr;
+  int device = 0;
+  int users = 0;  // calls that are using the handle (OptUse)
+  Workspace();
+  ~Workspace();
+  Workspace(const Workspace&) = delete;
+  Workspace& operator=(const Workspace&) = delete;
   void* get(const std::string& name, size_t bytes);
   bool has(const std::string& name, size_t bytes) const;  // get() would return it as it is
   bool drop_optional();
   void release();
+};
+
+// While it lives, no other handle's allocation takes the optional buffers of this one.
+class OptUse {
+ public:
+  explicit OptUse(const qcd_gauge* g);
+  ~OptUse();
+
+ private:
+  Workspace& ws_;
 };
 
 }  // namespace qcd

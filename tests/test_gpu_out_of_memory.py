@@ -99,3 +99,81 @@ def test_solve_whose_allocations_take_the_links_back(monkeypatch, inner, method,
             qcd.solve(g, f, to_dev(b), x.zero_(), nrhs=nrhs, tol=1e-11, inner=inner, method=method, use_graph=True)
             check(x.cpu().numpy())
     g.free()
+
+
+def test_another_handle_gives_its_links_back(monkeypatch):
+    """An allocation that only fits without the fixed-point links of an idle handle gets their memory; that handle
+    answers as before."""
+    device()
+    big = (16, 16, 16, 16)
+    Vb = int(np.prod(big))
+    Ub = inputs.gauge_field(big, 0.3, 37)
+    U, g = _load(38)
+    gb = qcd.Gauge.load(to_dev(Ub), big, BC)
+    f = qcd.wilson(KAPPA)
+    psi = inputs.gaussian_source((Vb, 4, 3), 39)
+    d = to_dev(psi)
+    ref = ora.wilson(big, BC, KAPPA, Ub, psi)
+
+    def full():
+        out = torch.empty_like(d)
+        qcd.dslash(gb, f, "FULL", d, out, prec="f64")
+        torch.cuda.synchronize()
+        return max_err(out, ref)
+
+    assert full() < TOL
+    torch.cuda.synchronize()
+    free = torch.cuda.mem_get_info()[0]
+    monkeypatch.setenv("QCD_FAULT", "oom")
+    b = to_dev(inputs.gaussian_source((V, 4, 3), 40))
+    x = torch.zeros_like(b)
+    qcd.solve(g, f, b, x, tol=1e-10, inner="f32")  # a lattice of 768 sites
+    monkeypatch.delenv("QCD_FAULT")
+    assert torch.cuda.mem_get_info()[0] - free >= 1152 * Vb // 2  # 1152 bytes per site came back, a little was used
+    assert full() < TOL
+    x = torch.zeros_like(d)
+    qcd.solve(gb, f, d, x, tol=1e-11, inner="f64", use_graph=True)
+    res = np.linalg.norm(psi - ora.wilson(big, BC, KAPPA, Ub, x.cpu().numpy())) / np.linalg.norm(psi)
+    assert res <= 1.01e-11
+    g.free()
+    gb.free()
+
+
+def test_handles_of_two_threads(monkeypatch):
+    """While a call uses a handle, no other thread's allocation takes its links."""
+    import threading
+
+    dev = device()
+    f = qcd.wilson(KAPPA)
+    sets, errors = [_load(41 + k) for k in range(2)], []
+    monkeypatch.setenv("QCD_FAULT", "oom")
+
+    def work(k):
+        try:
+            U, g = sets[k]
+            stream = torch.cuda.Stream(dev)
+            with torch.cuda.stream(stream):
+                for rep in range(6):
+                    n = 1 + (rep + k) % 3
+                    b = inputs.gaussian_source((n, V, 4, 3), 50 + rep)
+                    x = torch.zeros(b.shape, dtype=torch.complex128, device=dev)
+                    src = to_dev(b)
+                    qcd.solve(g, f, src, x, nrhs=n, tol=1e-11, inner="f64")
+                    out = torch.empty_like(x)
+                    qcd.dslash(g, f, "FULL", x, out, prec="f64", nrhs=n)
+                    stream.synchronize()
+                    for r in range(n):
+                        assert max_err(out[r], b[r]) < 1e-9
+                    if rep == 3:  # loaded again, with its fixed-point form
+                        g.free()
+                        g = qcd.Gauge.load(to_dev(U), L, BC)
+            g.free()
+        except BaseException as e:  # noqa: BLE001
+            errors.append(e)
+
+    threads = [threading.Thread(target=work, args=(k,)) for k in range(2)]
+    for t in threads:
+        t.start()
+    for t in threads:
+        t.join()
+    assert not errors, errors
