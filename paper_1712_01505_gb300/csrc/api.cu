@@ -326,7 +326,8 @@ void destroy(qcd_gauge* g) {
   if (g->work) cudaStreamDestroy(g->work);
   if (g->ev_in) cudaEventDestroy(g->ev_in);
   if (g->ev_out) cudaEventDestroy(g->ev_out);
-  if (g->fx_ev) cudaEventDestroy(g->fx_ev);
+  for (auto& set : g->fx_set)
+    if (set.done) cudaEventDestroy(set.done);
   delete g;
 }
 

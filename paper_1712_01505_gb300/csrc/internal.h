@@ -146,11 +146,20 @@ struct qcd_gauge {
   void* Udf = nullptr;  // double-float, 18 reals as hi/lo FP32 pairs
   void* Ufx = nullptr;  // the FP64 links of the eight hops of every site in fixed point (fixed.cuh)
   bool fx_ok = false;   // Ufx is there and every link has the size the fixed-point stencil takes
-  bool fx_used = false;             // the fixed-point scratch has been used, last on fx_stream
-  cudaStream_t fx_stream = nullptr;
+  // The fixed-point scratch, one set for each of the caller's streams up to kFxSets, so that operators on several
+  // streams overlap; the solver's stream shares the first.
+  struct FxSet {
+    bool owned = false, used = false;
+    bool on_work = false;           // the last use was on `work`, the event not recorded
+    cudaStream_t owner = nullptr;   // a name only: the stream may be gone, or another by now
+    cudaEvent_t done = nullptr;
+  };
+  static constexpr int kFxSets = 4;
+  FxSet fx_set[kFxSets];
+  int fx_next = 0;
   qcd::Workspace ws;
   cudaStream_t work = nullptr;  // private stream (capturable) for the solver
-  cudaEvent_t ev_in = nullptr, ev_out = nullptr, fx_ev = nullptr;
+  cudaEvent_t ev_in = nullptr, ev_out = nullptr;
   int device = 0;
 };
 

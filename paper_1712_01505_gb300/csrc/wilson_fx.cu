@@ -1099,22 +1099,47 @@ void fx_launch(const qcd_gauge* gh, const FxField& in, const SpinorView<P64>* sr
 }
 
 // The scratch fields belong to the handle, and calls on device buffers are asynchronous on the caller's
-// stream: work on another stream than the last user's waits for that user's event.  (The solver's own
-// stream is recorded only when another stream follows it: the handle owns it.)
-struct FxOrder {
-  qcd_gauge* g;
-  cudaStream_t st;
-  FxOrder(qcd_gauge* g_, cudaStream_t st_) : g(g_), st(st_) {
-    if (!g->fx_ev) QCD_CK(cudaEventCreateWithFlags(&g->fx_ev, cudaEventDisableTiming));
-    if (!g->fx_used || g->fx_stream == st) return;
-    if (g->fx_stream == g->work) QCD_CK(cudaEventRecord(g->fx_ev, g->work));
-    QCD_CK(cudaStreamWaitEvent(st, g->fx_ev, 0));
+// stream.  A stream has a set of its own while there are sets (kFxSets), and always waits for the event of the set's last
+// use: a stream's address says nothing about which stream that was (it may have been destroyed with the work
+// pending and another one created there, and cudaStreamPerThread is one address for every thread's).  Only the solver's
+// own stream is known; its use is recorded when another stream follows.
+class FxOrder {
+ public:
+  FxOrder(qcd_gauge* g, cudaStream_t st) : g_(g), st_(st), set_(g->fx_set[pick(g, st)]) {
+    if (!set_.done) QCD_CK(cudaEventCreateWithFlags(&set_.done, cudaEventDisableTiming));
+    if (!set_.used || (set_.on_work && st == g->work)) return;
+    if (set_.on_work) QCD_CK(cudaEventRecord(set_.done, g->work));
+    QCD_CK(cudaStreamWaitEvent(st, set_.done, 0));
   }
-  void done() {
-    g->fx_used = true;
-    g->fx_stream = st;
-    if (st != g->work) QCD_CK(cudaEventRecord(g->fx_ev, st));
+  ~FxOrder() {
+    set_.used = true;
+    set_.on_work = st_ == g_->work;
+    if (!set_.on_work) cudaEventRecord(set_.done, st_);
   }
+  FxOrder(const FxOrder&) = delete;
+  FxOrder& operator=(const FxOrder&) = delete;
+  // scratch field 'a' or 'b' of the set
+  FxField field(char which, const Field& like) const {
+    const char name[] = {'o', 'p', 't', '.', 'f', 'x', '.', which, (char)('0' + (&set_ - g_->fx_set)), 0};
+    return fx_scratch(g_, name, like, st_);
+  }
+
+ private:
+  static int pick(qcd_gauge* g, cudaStream_t st) {
+    if (st == g->work) return 0;
+    for (int k = 0; k < qcd_gauge::kFxSets; ++k)
+      if (!g->fx_set[k].owned || g->fx_set[k].owner == st) {
+        g->fx_set[k].owned = true;
+        g->fx_set[k].owner = st;
+        return k;
+      }
+    const int k = g->fx_next++ % qcd_gauge::kFxSets;
+    g->fx_set[k].owner = st;
+    return k;
+  }
+  qcd_gauge* g_;
+  cudaStream_t st_;
+  qcd_gauge::FxSet& set_;
 };
 
 // Whether the fixed-point path may run on `st`: never under a caller's stream capture (a graph that
@@ -1140,18 +1165,17 @@ bool hop_fx(const qcd_gauge* gh, const Field& in, Field& out, int out_parity, in
             cudaStream_t st, const int* stop, const RedSpec* red) {
   if (!fx_usable(gh, st)) return false;
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  FxOrder order(g, st);
   FxField f;
   try {
-    f = fx_scratch(g, "opt.fx.a", in, st);
+    f = order.field('a', in);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  FxOrder order(g, st);
   fx_pack(in, f, st, stop);
   const SpinorView<P64> src = fx_view(in);
   fx_launch(g, f, &src, in, &out, nullptr, out_parity, dagger, a, x, st, stop, red);
-  order.done();
   return true;
 }
 
@@ -1159,20 +1183,19 @@ bool mhat_fx(const qcd_gauge* gh, const Field& in, Field& out, int dagger, doubl
              const RedSpec* red) {
   if (!fx_usable(gh, st)) return false;
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
+  FxOrder order(g, st);
   FxField f, t;
   try {
-    f = fx_scratch(g, "opt.fx.a", in, st);
-    t = fx_scratch(g, "opt.fx.b", in, st);
+    f = order.field('a', in);
+    t = order.field('b', in);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
   }
-  FxOrder order(g, st);
   fx_pack(in, f, st, stop);
   const SpinorView<P64> src = fx_view(in);
   fx_launch(g, f, &src, in, nullptr, &t, 1, dagger, 1.0, nullptr, st, stop, nullptr);
   fx_launch(g, t, nullptr, in, &out, nullptr, 0, dagger, -k2, &in, st, stop, red);
-  order.done();
   return true;
 }
 
@@ -1180,8 +1203,9 @@ bool outer_fx_ready(const qcd_gauge* gh, const Field& shape, cudaStream_t st) {
   if (!fx_usable(gh, st)) return false;
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   try {
-    fx_scratch(g, "opt.fx.a", shape, st);
-    fx_scratch(g, "opt.fx.b", shape, st);
+    FxOrder order(g, st);
+    order.field('a', shape);
+    order.field('b', shape);
     const size_t nb = (size_t)(shape.Vh + kWarps * kSB - 1) / (kWarps * kSB);
     g->ws.get("opt.fx.sums", sizeof(double) * 4 * nb * shape.nrhs);
   } catch (const Error& e) {
@@ -1194,7 +1218,8 @@ bool outer_fx_ready(const qcd_gauge* gh, const Field& shape, cudaStream_t st) {
 void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
   qcd_gauge* g = const_cast<qcd_gauge*>(gh);
   const Field& shape = o.x;
-  const FxField fa = fx_scratch(g, "opt.fx.a", shape, st), fb = fx_scratch(g, "opt.fx.b", shape, st);
+  FxOrder order(g, st);
+  const FxField fa = order.field('a', shape), fb = order.field('b', shape);
   const unsigned nb = (unsigned)((shape.Vh + kWarps * kSB - 1) / (kWarps * kSB)), n = (unsigned)shape.nrhs;
   double* partial = (double*)g->ws.get("opt.fx.sums", sizeof(double) * 4 * nb * n);
   const int4* links = (const int4*)g->Ufx;
@@ -1203,7 +1228,6 @@ void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
     for (const void* k : {(const void*)k_outer_odd, (const void*)k_outer_res<P64>, (const void*)k_outer_res<P32>,
                           (const void*)k_outer_res<P16>})
       QCD_CK(cudaFuncSetAttribute(k, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(FxShared)));
-  FxOrder order(g, st);
   const dim3 sites((unsigned)((shape.Vh + 127) / 128), n);
   if (o.x_zero) {
     fx_pack(o.b_o, fb, st, nullptr);  // x_o = b_o
@@ -1242,7 +1266,6 @@ void outer_fx(const qcd_gauge* gh, const OuterStep& o, cudaStream_t st) {
   QCD_LAUNCH_CK();
   launch_k(k_outer_sums, n, 256, 0, st, partial, (int)nb, o.sums, o.sums_stride, (int)!o.x_zero);
   QCD_LAUNCH_CK();
-  order.done();
 }
 
 bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* in, double* out, int nrhs,
@@ -1253,10 +1276,11 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
   shape.prec = QCD_F64;
   shape.Vh = g->lat.Vh;
   shape.nrhs = nrhs;
+  FxOrder order(g, st);
   FxField fa, fb;
   try {
-    fa = fx_scratch(g, "opt.fx.a", shape, st);
-    fb = fx_scratch(g, "opt.fx.b", shape, st);
+    fa = order.field('a', shape);
+    fb = order.field('b', shape);
   } catch (const Error& e) {
     if (e.status != QCD_ERR_OOM) throw;
     return false;
@@ -1269,7 +1293,6 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
   const double2 *src = (const double2*)in;
   const bool full = op == QCD_OP_FULL || op == QCD_OP_FULL_DAG, mhat = op == QCD_OP_MHAT || op == QCD_OP_MHAT_DAG;
   const int dagger = op == QCD_OP_FULL_DAG || op == QCD_OP_MHAT_DAG;
-  FxOrder order(g, st);
   // fixed-point halves: both for FULL (even in fa, odd in fb), else the one that the operator reads, in fa
   const int p0 = full || mhat || op == QCD_OP_D_OE ? 0 : 1;
   launch_k(k_canon_to_fx, dim3((unsigned)((shape.Vh + 127) / 128), n, full ? 2 : 1), 128, 0, st, geom, src,
@@ -1295,7 +1318,6 @@ bool canon_fx(const qcd_gauge* gh, const qcd_fermion& f, int op, const double* i
   } else {
     hop(fa, true, op == QCD_OP_D_OE, 1.0, false, true);
   }
-  order.done();
   return true;
 }
 
