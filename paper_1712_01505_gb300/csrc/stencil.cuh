@@ -457,9 +457,8 @@ __device__ __forceinline__ void red_epilogue(const HA& A, R v[3]) {
     double b = 0.0;
     for (int w = 0; w < (int)(blockDim.x >> 5); ++w) b += wsum[w][threadIdx.x];
     A.partial[(long)blockIdx.x * 4 + threadIdx.x] = b;
-    __threadfence();
   }
-  if (spread && warp == 0) __syncwarp();
+  if (spread && warp == 0) __syncwarp();  // the lanes' stores before thread 0's fence
   if (threadIdx.x == 0) {
     if constexpr (!spread) {
       double b[3] = {0.0, 0.0, 0.0};
@@ -468,8 +467,8 @@ __device__ __forceinline__ void red_epilogue(const HA& A, R v[3]) {
         for (int k = 0; k < 3; ++k) b[k] += wsum[w][k];
 #pragma unroll
       for (int k = 0; k < 3; ++k) A.partial[(long)blockIdx.x * 4 + k] = b[k];
-      __threadfence();
     }
+    __threadfence();
     const int members = min(kRedGroup, (int)gridDim.x - grp * kRedGroup);
     last = (atomicAdd(&A.counters[grp], 1) == members - 1);
     if (blockIdx.x == 0) *A.npartial = ngroups;
