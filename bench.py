@@ -10,7 +10,7 @@ One step = one pass of the hot path on that input:
   1. the standalone even-odd hopping stencil D_eo in FP32 (NDSLASH launches)
      and in FP64 (one launch), on internal-layout device buffers;
   2. the mixed-precision even-odd BiCGStab solve (FP32 inner iterations,
-     IEEE-FP64 reliable updates: true residual, solution accumulation and
+     FP64 reliable updates: true residual, solution accumulation and
      reductions in FP64) to |b - M x| / |b| <= 1e-10 on the full system,
      from canonical device buffers (source preparation, solve, reconstruction
      and the final FP64 true residual included).
@@ -239,8 +239,8 @@ def main():
                     help="wilson32 (default, the bench line); the others characterise the other "
                          "configurations (domain-wall CG, 12-rhs propagator, force) and print their own line")
     ap.add_argument("--outer", default="f64", choices=["f64", "df64"],
-                    help="precision of the outer steps of the mixed solve: f64 = IEEE FP64 stencil (the "
-                         "default), df64 = double-float stencil (FP32 pairs); the final residual is IEEE FP64 "
+                    help="precision of the outer steps of the mixed solve: f64 = FP64 stencil (the "
+                         "default), df64 = double-float stencil (FP32 pairs); the final residual is FP64 "
                          "either way")
     ap.add_argument("--delta", type=float, default=None,
                     help="reliable-update factor of the mixed solves (default: 1e-5 for the FP32 Wilson solves "
@@ -368,7 +368,7 @@ def main():
 
     def hops_in_solve(inf, outer=args.outer):
         # 4 inner half-dslashes per BiCGStab iteration, 1 for the source and 2 per outer step
-        # (none before the first since x0 = 0).  IEEE-FP64 outer steps reconstruct x_o and form
+        # (none before the first since x0 = 0).  FP64 outer steps reconstruct x_o and form
         # the full-system residual themselves, so the last one ends the solve; double-float
         # outer steps add the reconstruction and the even half of the final FP64 residual.
         return 4 * inf["iters"] + 1 + 2 * inf["outer_updates"] + (2 if outer == "df64" else 0)
@@ -488,7 +488,7 @@ def main():
         "data": "synthetic: smoothed-random SU(3) links and Z2 noise source (seeded)",
         "config": {"workload": WORKLOAD, "lattice": list(L), "kappa": KAPPA, "eps": EPS, "recon": RECON,
                    "solver": "EO BiCGStab, FP32 inner + reliable updates in "
-                             + ("double-float (FP32 pairs)" if args.outer == "df64" else "IEEE FP64")
+                             + ("double-float (FP32 pairs)" if args.outer == "df64" else "FP64 (link products in fixed point)")
                              + " (FP64 solution and reductions), FP64 final residual, CUDA graph chunks of 32",
                    "outer": args.outer,
                    "tol": TOL, "ndslash_per_step": NDSLASH, "delta": delta,

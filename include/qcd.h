@@ -71,6 +71,16 @@ typedef enum {
 } qcd_status;
 
 /* Storage / arithmetic precision of internal fields and operator applications.
+ * QCD_F64 is double in storage, sums and results.  The Wilson hopping term
+ * multiplies the links in fixed point (integers with an FP32 remainder, 64-bit
+ * sums) wherever an output component comes out as good as from FP64
+ * arithmetic: its error is then below 2^-48 S, S the sum of the magnitudes of
+ * its own products (rms at most 2^-50.5 S; on Gaussian fields 2^-55.7 S, FP64
+ * 2^-54.8 S).  Components with too small an S beside their neighbours' values,
+ * infinities, NaN, links whose rows and columns are not of unit size (see
+ * qcd_gauge_load), calls under a caller's stream capture, qcd_mhat_noalloc, the
+ * domain decomposition and calls short of memory get FP64 arithmetic; results
+ * of the two kinds differ in their last bits.
  * QCD_DF64 ("double-float") keeps every real as an unevaluated sum hi + lo of
  * two FP32 numbers (|lo| <= ulp(hi)/2 on store) and multiplies and sums with
  * error-free transformations (TwoSum, TwoProd by FMA; the compensated dot
@@ -149,10 +159,10 @@ typedef struct {
  * dagger: solve with the adjoint operator (A^dag x = b); Wilson only.
  * outer: precision of the operator applications of the outer steps of a
  *   mixed solve (source preparation, reliable-update residuals b - Mhat x,
- *   reconstruction of the odd sites): QCD_F64 (IEEE double, the default when
+ *   reconstruction of the odd sites): QCD_F64 (the default when
  *   zero-initialised) or QCD_DF64 (double-float; the solution is then also
- *   accumulated in double-float).  The final true_resid is computed with IEEE
- *   FP64 operators either way; ignored when inner = QCD_F64. */
+ *   accumulated in double-float).  The final true_resid is computed with the
+ *   QCD_F64 operators either way; ignored when inner = QCD_F64. */
 typedef struct {
   int32_t method;
   double tol;

@@ -13,7 +13,7 @@
 // the true-residual recomputation, the solution accumulation and the global
 // sums of the dot products.  With outer = QCD_DF64 (Wilson) the outer steps
 // run in double-float instead (FP32 pairs, about 48 bits; see wilson_df.cu),
-// and only the final true residual uses the IEEE-FP64 stencil.
+// and only the final true residual uses the FP64 stencil.
 //
 // The scalars (alpha, beta, omega, rho, |r|^2) never leave the device during
 // the inner iteration: per-block partial sums become scalars in the prologue of
@@ -863,7 +863,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   S.b_e = ws_field(g, "s.b_e", QCD_F64, ls, nrhs);
   S.b_o = ws_field(g, "s.b_o", QCD_F64, ls, nrhs);
   S.x64 = ws_field(g, "s.x64", QCD_F64, ls, nrhs);
-  // IEEE-FP64 outer steps of the Wilson solve keep the reconstructed odd half of x
+  // FP64 outer steps of the Wilson solve keep the reconstructed odd half of x
   const bool wil64 = !dwf && !(prm.outer == QCD_DF64 && S.inner != QCD_F64);
   if (wil64) S.xo64 = ws_field(g, "s.xo64", QCD_F64, ls, nrhs);
   // ... and the even half r_e of the full-system residual: the inner residual itself for
@@ -903,7 +903,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
     if (g->ws.generation != gen) QCD_CK(cudaMemsetAsync(S.counters, 0, sizeof(int) * ngroups, st));
   }
   S.hsc.assign(nrhs, Scal{});
-  // BiCGStab with IEEE-FP64 outer steps: the steps in fixed point (three fused kernels, wilson_fx.cu) where
+  // BiCGStab with FP64 outer steps: the steps in fixed point (three fused kernels, wilson_fx.cu) where
   // that path is available, else the separate operators below.  Everything the solve allocates on the
   // device is allocated by here, so that no later allocation can take the links of that path back.
   bool fxo = false;
@@ -926,7 +926,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
   // Double-float outer steps (mixed solves): the prepared source, the solution
   // and the outer residual live in FP32 pairs and the outer operator
   // applications use the double-float stencil (and A^-1 for domain-wall); the
-  // true residual reported at the end is recomputed with the IEEE-FP64
+  // true residual reported at the end is recomputed with the FP64
   // operator all the same.
   const bool dfo = prm.outer == QCD_DF64 && S.inner != QCD_F64;
   const OpCtx opdf{g, f, QCD_DF64};
@@ -1038,7 +1038,7 @@ void solve_device(qcd_gauge* g, const qcd_fermion& f, const qcd_solver_params& p
       return;
     }
     if (wil64) {
-      // Wilson with IEEE-FP64 outer steps: reconstruct x_o = b_o + kappa h, h = H_oe x_e,
+      // Wilson with FP64 outer steps: reconstruct x_o = b_o + kappa h, h = H_oe x_e,
       // and form the even half of the full-system residual,
       //   r_e = b_e - x_e + kappa H_eo x_o  (= bhat - Mhat x_e; the odd half is zero up to
       // the rounding of x_o), so that the outer step that reaches the target has already

@@ -201,3 +201,20 @@ def test_reconstructed_half_of_a_solve(links, field, dagger):
     assert np.array_equal(_half(got, 0), _half(x0, 0))
     _close(_half(got, 1), KAPPA * _half(h, 1), KAPPA * (TOL * _half(S, 1) + 2.0 ** -52 * np.abs(_half(h, 1))), "odd half")
     g.free()
+
+
+@pytest.mark.parametrize("inner", ["f64", "f32", "f16"])
+@pytest.mark.parametrize("scale", [3.0, 0.3])
+def test_solves_on_links_of_other_size(inner, scale):
+    """Links outside the fixed-point range: plain and mixed solves on the FP64 kernels, judged in extended precision."""
+    device()
+    U = scale * _links("interacting")
+    kappa = 0.1 / scale
+    b = inputs.gaussian_source((V, 4, 3), 28)
+    g = qcd.Gauge.load(to_dev(U), L, BC)
+    x = torch.zeros((V, 4, 3), dtype=torch.complex128, device=device())
+    info, _ = qcd.solve(g, qcd.wilson(kappa), to_dev(b), x, tol=1e-12, inner=inner, use_graph=True)
+    x = x.cpu().numpy()
+    res = np.linalg.norm(b - (x - kappa * _hop(U, x)[0])) / np.linalg.norm(b)
+    assert res <= 1.01e-12 and abs(res - info[0]["true_resid"]) <= 1e-2 * res + 2e-15
+    g.free()
