@@ -489,7 +489,7 @@ def main():
         "config": {"workload": WORKLOAD, "lattice": list(L), "kappa": KAPPA, "eps": EPS, "recon": RECON,
                    "solver": "EO BiCGStab, FP32 inner + reliable updates in "
                              + ("double-float (FP32 pairs)" if args.outer == "df64" else "FP64 (link products in fixed point)")
-                             + " (FP64 solution and reductions), FP64 final residual, CUDA graph chunks of 32",
+                             + " (FP64 solution and reductions), FP64 final residual, CUDA graphs of up to 32 iterations",
                    "outer": args.outer,
                    "tol": TOL, "ndslash_per_step": NDSLASH, "delta": delta,
                    "l2": "inputs larger than L2 (links 403 MB, each parity vector 101 MB)",

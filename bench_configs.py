@@ -123,7 +123,7 @@ def run_dwf(args):
         o_ = torch.empty(nb, dtype=torch.uint8, device=dev)
         qcd.field_pack(g, f, prec, 1, bd, a_)
         if args.profile == "cg":  # ncu: one warmed-up CG solve (inner precision --profile-prec, FP32 or
-            # FP16, at the reliable-update factor of the measured solve; IEEE-FP64 outer steps)
+            # FP16, at the reliable-update factor of the measured solve; FP64 outer steps)
             pin = "f16" if args.profile_prec == "f16" else "f32"
             kw = dict(method=qcd.CG_NORMAL, tol=1e-10, inner=pin, use_graph=True, graph_chunk=32,
                       delta=(args.delta or (1e-4 if pin == "f32" else 0.0)), outer=args.outer)
@@ -252,7 +252,7 @@ def run_dwf(args):
     out = {"workload": "dwf_16x16x16x32_Ls16_M5_1.8_mf0.02", "hop": hop, "cg": res, "roofline": roof,
            "cpu_baseline": cpu,
            "bicgstab_f32_df": bicg, "mobius_b5_1.5_c5_0.5": mob,
-           "note": "cg keys: inner precision, _df = double-float outer steps (else IEEE FP64)",
+           "note": "cg keys: inner precision, _df = double-float outer steps (else FP64)",
            "speedup_f16_vs_f64": round(res["f64"]["ms"] / res["f16"]["ms"], 3),
            "speedup_f32_vs_f64": round(res["f64"]["ms"] / res["f32"]["ms"], 3),
            "speedup_f16_df_vs_f64": round(res["f64"]["ms"] / res["f16_df"]["ms"], 3),

@@ -30,7 +30,8 @@ using namespace dwcol;
 constexpr int kFusedMaxLs = 32;  // tile of 32 sites x Ls slices x 96 B within 96 KB
 
 // PK = 1: the hop with packed FP32x2 arithmetic (stencil.cuh); PK = 2: the same
-// with the links staged as two rows.  The registers are bounded for 24 warps per SM: with the columns of the
+// with the links staged as two rows.  The registers are bounded for 24 warps per SM (BY 4 and 8: 80 registers, up to
+// 48 bytes spilled; BY 16: one block of 16 warps, 128 registers): with the columns of the
 // inverse in registers (one read and one write of the tile; up to Ls = 16) the kernel would take 99 and run
 // 101 us instead of 84 (16^3 x 32 x 16, Mobius adjoint, FP32; 88 with two reads and a write of scalars).
 template <int P, int RECON, int BY, int PK>

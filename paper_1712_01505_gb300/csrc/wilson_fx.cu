@@ -6,12 +6,13 @@
 //
 // The input is first rewritten as fixed-point parts with one exponent per site (k_to_fx), the links
 // are kept that way from the loading of the gauge field, and only the final sum goes through the
-// FP64 pipe: 24 conversions and 24 multiply-adds per site instead of 864.  Measured at 32^3 x 64:
-// FP64 kernel 1.57 ms (FP64 pipe), here 0.315 ms, 5.8 TB/s = 85% of the copy rate (HBM: links 1152 B, input
-// 196 B, x and output 192 B each per site), and 0.063 ms for k_to_fx (HBM); 16^3 x 32 x 16 slices
-// 1.56 -> 0.28 + 0.07 ms (issue slots).  Forms that were slower: the conversion inside the stencil (8 times per
-// site: 0.555 ms), three integer products per real one instead of one and two FP32 ones (0.355 ms, the
-// integer multiply pipe), one thread per site (0.333 ms at 168 registers, 12 warps per SM).
+// FP64 pipe: 24 conversions and 24 multiply-adds per site instead of 864.  Sites whose components the parts do not
+// hold as well as FP64 would are computed in FP64 (fx_sum, fx_careful).  Measured at 32^3 x 64:
+// FP64 kernel 1.56 ms (FP64 pipe), here 0.31 ms, 5.3 TB/s = 79% of the copy rate (links 1152 B, input 196 B, x and output
+// 192 B each per site; HBM and issue slots), and 0.056 ms for k_to_fx (HBM); 16^3 x 32 x 16 slices 1.56 -> 0.35 ms with
+// the conversion (issue slots).  Forms that were slower than 0.315 ms, all without the sums of magnitudes: the conversion
+// inside the stencil (8 times per site: 0.555 ms), three integer products per real one instead of one and two FP32
+// ones (0.355 ms, the integer multiply pipe), one thread per site (0.333 ms at 168 registers, 12 warps per SM).
 #include <cstdio>
 #include <vector>
 
@@ -30,9 +31,9 @@ using namespace fx;
 using HA = HopArgs<P64, 18>;
 
 // Layouts.  Links: the matrices of all eight hops of a site, W[2 mu] = U_mu(x) and
-// W[2 mu + 1] = U_mu(x - mu)^dag, as [parity][block of 32 sites][hop][element][32] (each link is stored
+// W[2 mu + 1] = U_mu(x - mu)^dag, as [parity][block of 16 sites][hop][element][16] (each link is stored
 // for both of its ends: a half-dslash reads as many bytes as from one copy, contiguously and with
-// no transposition).  Spinors: [slice][block of 32 sites][component][32] and one exponent field per
+// no transposition).  Spinors: [slice][block of 16 sites][component][16] and one exponent field per
 // site.  A unit is int4 (re.h, re.l, im.h, im.l).  A site of exponent field kBad holds its FP64 values.
 constexpr int kSB = 16;  // sites per block of the layouts
 constexpr int kHopUnits = 9 * kSB, kSiteUnits = 12 * kSB;
@@ -213,87 +214,98 @@ struct FxSum {
   unsigned su[3], sl[3];
 };
 
-// Hop number I (of fx_order) added to a.  m: the sign of the lower input spin.  Packed FP32 lanes: (re, im).
+// The products of a hop, added to S; link(k): element k of its matrix.  Packed FP32 lanes: (re, im).
+template <int HOP, typename LINK>
+__device__ __forceinline__ void fx_products(LINK link, int d3, const int (&hr)[3], const int (&hi)[3], const float2 (&y)[3],
+                                            FxSum& S) {
+  constexpr int MU = HOP >> 1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
+  const float sc = __int_as_float((127 - d3) << 23);
+#pragma unroll
+  for (int a = 0; a < 3; ++a) {
+    int64_t Hr = hop_half(d3, HOP & 1), Hi = Hr;
+    float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
+#pragma unroll
+    for (int b = 0; b < 3; ++b) {
+      const int4 u = link(a * 3 + b);
+      const float2 g = make_float2((float)hr[b], (float)hi[b]);  // the integer parts as FP32
+      Hr += (int64_t)u.x * hr[b];
+      Hr += (int64_t)u.z * -hi[b];
+      Hi += (int64_t)u.x * hi[b];
+      Hi += (int64_t)u.z * hr[b];
+      C = fma2(bc2((float)u.x), y[b], C);
+      C = fma2(bc2(__int_as_float(u.y)), g, C);
+      D = fma2(bc2((float)u.z), swp(y[b]), D);
+      D = fma2(bc2(__int_as_float(u.w)), swp(g), D);
+    }
+    const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
+    const unsigned size = __byte_perm(abs((int)(wr >> 32)), abs((int)(wi >> 32)), 0x7632);
+    S.up[2 * a] += wr;
+    S.up[2 * a + 1] += wi;
+    S.su[a] += size;
+    if (MU == 0 || MU == 2) {  // SG i w
+      S.lo[2 * a] -= SG * wi;
+      S.lo[2 * a + 1] += SG * wr;
+      S.sl[a] += __byte_perm(size, size, 0x1032);
+    } else {
+      S.lo[2 * a] += SG * wr;
+      S.lo[2 * a + 1] += SG * wi;
+      S.sl[a] += size;
+    }
+  }
+}
+
+// Hop number I (of fx_order) added to S.  m: the sign of the lower input spin.
 template <int I>
 __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int sp, int m, FxSum& S) {
   constexpr int HOP = fx_order(I), MU = HOP >> 1;
-  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
+  constexpr int SG = (HOP & 1) ? 1 : -1;
   const int nbw = W.sm->nb[HOP][W.warp * kSB + W.lane % kSB];
   const int d3 = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100) + 3;
   int hr[3], hi[3];
   float2 y[3];  // the FP32 parts
   fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
-  int hn[3];
-  float2 g[3], ys[3], gs[3];  // the integer parts as FP32; both with the lanes exchanged
-#pragma unroll
-  for (int c = 0; c < 3; ++c) {
-    g[c] = make_float2((float)hr[c], (float)hi[c]);
-    ys[c] = swp(y[c]);
-    gs[c] = swp(g[c]);
-    hn[c] = -hi[c];
-  }
   if (!mbar_wait(&W.sm->bar[W.warp][I % kBuf], (unsigned)(I / kBuf) & 1u)) W.failed = true;
   if (d3 < kFar) {
-    const float sc = __int_as_float((127 - d3) << 23);
     const int4* w = &W.sm->w[W.warp][I % kBuf][W.lane % kSB];
-#pragma unroll
-    for (int a = 0; a < 3; ++a) {
-      int64_t Hr = hop_half(d3, HOP & 1), Hi = Hr;
-      float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
-#pragma unroll
-      for (int b = 0; b < 3; ++b) {
-        const int4 u = w[(a * 3 + b) * kSB];
-        Hr += (int64_t)u.x * hr[b];
-        Hr += (int64_t)u.z * hn[b];
-        Hi += (int64_t)u.x * hi[b];
-        Hi += (int64_t)u.z * hr[b];
-        C = fma2(bc2((float)u.x), y[b], C);
-        C = fma2(bc2(__int_as_float(u.y)), g[b], C);
-        D = fma2(bc2((float)u.z), ys[b], D);
-        D = fma2(bc2(__int_as_float(u.w)), gs[b], D);
-      }
-      const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
-      const unsigned size = __byte_perm(abs((int)(wr >> 32)), abs((int)(wi >> 32)), 0x7632);
-      S.up[2 * a] += wr;
-      S.up[2 * a + 1] += wi;
-      S.su[a] += size;
-      if (MU == 0 || MU == 2) {  // SG i w
-        S.lo[2 * a] -= SG * wi;
-        S.lo[2 * a + 1] += SG * wr;
-        S.sl[a] += __byte_perm(size, size, 0x1032);
-      } else {
-        S.lo[2 * a] += SG * wr;
-        S.lo[2 * a + 1] += SG * wi;
-        S.sl[a] += size;
-      }
-    }
+    fx_products<HOP>([&](int k) { return w[k * kSB]; }, d3, hr, hi, y, S);
   }
   __syncwarp();  // every lane has read the buffer
   if (I + kBuf < 8) W.issue(fx_order(I + kBuf < 8 ? I + kBuf : 0), I % kBuf);
 }
 
-// The magnitudes of the products of hop number I, per component of the lane: upper spin sp in s, the lower spin in t;
-// bits of nz, nt: a product is not zero.  links: of the lane's site.
+// The magnitudes of a lane's products, per component (upper spin sp in s, the lower spin in t), the neighbours' sizes relative
+// to the largest one's, and bits of nz, nt: a product is not zero.
+struct FxMagnitudes {
+  float s[6], t[6], size;
+  unsigned nz, nt;
+};
+
+// Hop number I and its magnitudes.  links: of the lane's site.
 template <int I>
-__device__ __forceinline__ void fx_magnitudes(const int* nb, const FxField& f, const int4* links, int E, int sp, int m,
-                                              float (&s)[6], float (&t)[6], unsigned& nz, unsigned& nt, float& size) {
+__device__ __forceinline__ void fx_careful_hop(const int* nb, const FxField& f, const int4* links, int E, int sp, int m,
+                                               FxSum& S, FxMagnitudes& M) {
   constexpr int HOP = fx_order(I), MU = HOP >> 1;
   constexpr int SG = (HOP & 1) ? 1 : -1;
   const int nbw = nb[HOP * (kWarps * kSB)];
   const int d = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100);
-  const float sc = __int_as_float((127 - d) << 23);
   int hr[3], hi[3];
   float2 y[3];
   fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
-  size += sc;
+  int4 u[9];
+#pragma unroll
+  for (int k = 0; k < 9; ++k) u[k] = __ldg(links + HOP * kHopUnits + k * kSB);
+  if (d + 3 < kFar) fx_products<HOP>([&](int k) { return u[k]; }, d + 3, hr, hi, y, S);
+  const float sc = __int_as_float((127 - d) << 23);
+  M.size += sc;
 #pragma unroll
   for (int a = 0; a < 3; ++a) {
     float mr = 0.f, mi = 0.f;
     unsigned br = 0, bi = 0;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const int4 u = __ldg(links + HOP * kHopUnits + (a * 3 + b) * kSB);
-      const float ur = fabsf((float)u.x + __int_as_float(u.y)), ui = fabsf((float)u.z + __int_as_float(u.w));
+      const int4 v = u[a * 3 + b];
+      const float ur = fabsf((float)v.x + __int_as_float(v.y)), ui = fabsf((float)v.z + __int_as_float(v.w));
       const float xr = fabsf((float)hr[b] + y[b].x), xi = fabsf((float)hi[b] + y[b].y);
       mr = fmaf(ur, xr, fmaf(ui, xi, mr));
       mi = fmaf(ur, xi, fmaf(ui, xr, mi));
@@ -301,38 +313,13 @@ __device__ __forceinline__ void fx_magnitudes(const int* nb, const FxField& f, c
       bi |= (ur != 0.f && xi != 0.f) || (ui != 0.f && xr != 0.f);
     }
     constexpr int x = (MU == 0 || MU == 2) ? 1 : 0;  // i w
-    s[2 * a] = fmaf(mr, sc, s[2 * a]);
-    s[2 * a + 1] = fmaf(mi, sc, s[2 * a + 1]);
-    t[2 * a + x] = fmaf(mr, sc, t[2 * a + x]);
-    t[2 * a + 1 - x] = fmaf(mi, sc, t[2 * a + 1 - x]);
-    nz |= (br | bi << 1) << (2 * a);
-    nt |= (x ? (bi | br << 1) : (br | bi << 1)) << (2 * a);
+    M.s[2 * a] = fmaf(mr, sc, M.s[2 * a]);
+    M.s[2 * a + 1] = fmaf(mi, sc, M.s[2 * a + 1]);
+    M.t[2 * a + x] = fmaf(mr, sc, M.t[2 * a + x]);
+    M.t[2 * a + 1 - x] = fmaf(mi, sc, M.t[2 * a + 1 - x]);
+    M.nz |= (br | bi << 1) << (2 * a);
+    M.nt |= (x ? (bi | br << 1) : (br | bi << 1)) << (2 * a);
   }
-}
-
-// Whether every component of the lane is as exact from the fixed-point parts as FP64 would have it (fixed.cuh), or has
-// no product that is not zero.  The whole warp calls it.
-__device__ __noinline__ bool fx_exact(const int* nb, const FxField& f, const int4* links, int E, int sp, int g5) {
-  const int gs = sp ? -g5 : g5;
-  float s[6] = {}, t[6] = {}, size = 0.f;
-  unsigned nz = 0, nt = 0;
-  fx_magnitudes<0>(nb, f, links, E, sp, -gs, s, t, nz, nt, size);
-  fx_magnitudes<1>(nb, f, links, E, sp, -gs, s, t, nz, nt, size);
-  fx_magnitudes<2>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
-  fx_magnitudes<3>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
-#pragma unroll
-  for (int k = 0; k < 6; ++k) t[k] = __shfl_xor_sync(0xffffffffu, t[k], kSB);  // the lower spins change lanes (fx_sum)
-  nt = __shfl_xor_sync(0xffffffffu, nt, kSB);
-  fx_magnitudes<4>(nb, f, links, E, sp, gs, s, t, nz, nt, size);
-  fx_magnitudes<5>(nb, f, links, E, sp, gs, s, t, nz, nt, size);
-  fx_magnitudes<6>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
-  fx_magnitudes<7>(nb, f, links, E, sp, g5, s, t, nz, nt, size);
-  const float least = sum_min(size);
-  bool ok = true;
-#pragma unroll
-  for (int k = 0; k < 6; ++k)
-    ok = ok && (s[k] >= least || !(nz >> k & 1)) && (t[k] >= least || !(nt >> k & 1));
-  return ok;
 }
 
 // Hop number I in FP64, added to the lane's sums as fx_hop does: from the FP64 field that was converted to f where A.in
@@ -389,11 +376,11 @@ __device__ __forceinline__ void fp64_hop(const HA& A, const FxField& f, const do
 }
 
 // The hop sums of the lane (upper spin sp, lower spin 2 + sp, the latter times -1 for H^dag) in FP64; the whole warp calls
-// it, since a site's two lanes share the work.  Bound by the FP64 pipe.  The full matrix on 24^3 x 32 where every site comes
-// here (a point source's solution, links within 1e-4 of 1): 1.11 ms, of which 0.82 are the FP64 kernel's; one
-// lane per site, 2.04.
+// it, since a site's two lanes share the work; as bits of FP64 numbers.  Bound by the FP64 pipe.  The full matrix on
+// 24^3 x 32 where every site comes here (a point source's solution, links within 1e-4 of 1): 1.34 ms with the two walks
+// before; the FP64 kernel, 0.82.
 __device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, const int* nb, int cb, int sp,
-                                      Cx<double> (&out)[6]) {
+                                      int64_t (&out)[12]) {
   const double2* src = A.in.p;
   if (src) {
     const int r = fdiv(q, A.d_ls);
@@ -422,7 +409,10 @@ __device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, cons
   fp64_hop<6>(A, f, src, nb, cb, sp, g5, v);
   fp64_hop<7>(A, f, src, nb, cb, sp, g5, v);
 #pragma unroll
-  for (int k = 0; k < 6; ++k) out[k] = v[k];
+  for (int k = 0; k < 6; ++k) {
+    out[2 * k] = __double_as_longlong(v[k].re);
+    out[2 * k + 1] = __double_as_longlong(v[k].im);
+  }
 }
 
 // The exponent field of the site's largest neighbour (its neighbour indices go to shared memory).
@@ -448,52 +438,99 @@ __device__ __forceinline__ void flip(int64_t (&v)[6], bool minus) {
   for (int k = 0; k < 6; ++k) v[k] = (v[k] ^ n) - n;
 }
 
-// S.up, S.lo = the sum of the eight hops for spins sp and 2 + sp, in units of the returned value
-// (lo: times -1 for H^dag = g5 H g5); the whole warp calls it.  slow: the site is FP64's, for a neighbour that is
-// kept in FP64 or a component that the parts do not hold well enough.
-//
-// The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
-// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Only then are the magnitudes formed (fx_exact, a
-// second walk over the hops), which settles all but fields with components far smaller than others that the links hardly
-// mix with them.  Without any of this the full matrix on 24^3 x 48 took 309 us instead of 317, a solve on 12x10x14x18 3.56 ms
-// instead of 3.72, and twelve point sources on 24^3 x 48, around which spins and colours differ most, 138 ms instead of 144.
-__device__ __forceinline__ double fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S, bool& slow) {
-  const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) S.up[k] = S.lo[k] = 0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) S.su[k] = S.sl[k] = 0;
-  fx_hop<0>(W, f, E, sp, -gs, S);  // y: B = (-l1, l0)
-  fx_hop<1>(W, f, E, sp, -gs, S);
-  flip(S.lo, sp == 0);             // B^dag = (g1, -g0)
-  fx_hop<2>(W, f, E, sp, g5, S);   // x: B = -i (l1, l0)
-  fx_hop<3>(W, f, E, sp, g5, S);
+// the hops of both walks, in order: H(number, sign of the lower input spin); the lower spins' signs and lanes between them
+template <typename H>
+__device__ __forceinline__ void fx_walk(int sp, int g5, FxSum& S, H hop) {
+  const int gs = sp ? -g5 : g5;
+  hop(std::integral_constant<int, 0>{}, -gs);  // y: B = (-l1, l0)
+  hop(std::integral_constant<int, 1>{}, -gs);
+  flip(S.lo, sp == 0);                         // B^dag = (g1, -g0)
+  hop(std::integral_constant<int, 2>{}, g5);   // x: B = -i (l1, l0)
+  hop(std::integral_constant<int, 3>{}, g5);
 #pragma unroll
   for (int k = 0; k < 6; ++k) S.lo[k] = __shfl_xor_sync(0xffffffffu, S.lo[k], kSB);
 #pragma unroll
   for (int k = 0; k < 3; ++k) S.sl[k] = __shfl_xor_sync(0xffffffffu, S.sl[k], kSB);
   flip(S.lo, sp != 0);
-  fx_hop<4>(W, f, E, sp, gs, S);   // z: B = (-i l0, i l1)
-  fx_hop<5>(W, f, E, sp, gs, S);
+  hop(std::integral_constant<int, 4>{}, gs);   // z: B = (-i l0, i l1)
+  hop(std::integral_constant<int, 5>{}, gs);
   flip(S.lo, sp != 0);
-  fx_hop<6>(W, f, E, sp, g5, S);   // t: B = 1
-  fx_hop<7>(W, f, E, sp, g5, S);
+  hop(std::integral_constant<int, 6>{}, g5);   // t: B = 1
+  hop(std::integral_constant<int, 7>{}, g5);
+}
+__device__ __forceinline__ void fx_clear(FxSum& S) {
+#pragma unroll
+  for (int k = 0; k < 6; ++k) S.up[k] = S.lo[k] = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) S.su[k] = S.sl[k] = 0;
+}
+
+// S.up, S.lo = the sum of the eight hops for spins sp and 2 + sp, in units of 2^(E - 1079) (lo: times -1 for
+// H^dag = g5 H g5); the whole warp calls it.  true (for the whole warp): the sums do not show that they are exact
+// enough, or a neighbour is kept in FP64; fx_careful then computes the sites.
+//
+// The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
+// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Without it a half-dslash on 32^3 x 64 took 352 us instead of 365,
+// the full matrix on 24^3 x 48 309 instead of 316, a solve on 12x10x14x18 3.53 ms instead of 3.79, and twelve point sources on
+// 24^3 x 48, around which spins and colours differ most, 138 ms instead of 145.
+__device__ __forceinline__ bool fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S) {
+  fx_clear(S);
+  fx_walk(sp, A.dagger ? -1 : 1, S,
+          [&](auto i, int m) { fx_hop<decltype(i)::value>(W, f, E, sp, m, S); });
   unsigned least = 0xffffffffu;
 #pragma unroll
   for (int k = 0; k < 3; ++k) least = __vminu2(least, __vminu2(S.su[k], S.sl[k]));
-  bool weak = min(least & 0xffffu, least >> 16) < 64u && E > kZero && E < kBad;  // kZero: all neighbours are zero
-  if (__any_sync(0xffffffffu, weak))
-    weak = !fx_exact(&W.sm->nb[0][W.warp * kSB + W.lane % kSB], f, W.links + W.lane % kSB, E, sp, g5) && weak;
-  const unsigned any = __ballot_sync(0xffffffffu, weak);
-  slow = E == kBad || ((any | any >> kSB) >> (W.lane % kSB) & 1);  // of either lane
-  if (W.failed) return __longlong_as_double(0x7ff8000000000000ll);  // a copy that never arrived: NaN output
-  return __hiloint2double((E - 56) << 20, 0);  // 2^(E - 1079)
+  const bool weak = (min(least & 0xffffu, least >> 16) < 64u && E > kZero) || E == kBad;  // kZero: all neighbours are zero
+  return __any_sync(0xffffffffu, weak);
+}
+__device__ __forceinline__ double fx_unit(int E) { return __hiloint2double((E - 56) << 20, 0); }  // 2^(E - 1079)
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// The same sums once more with the magnitudes of their products, in out (up, then lo); of a site with a neighbour that
+// is kept in FP64, or with a component that is neither as exact as FP64 would have it (fixed.cuh) nor without a
+// product that is not zero, as FP64 numbers: true, for both lanes of the site.  A walk of its own, so that the
+// kernels' registers hold nothing meanwhile (with the first walk's sums kept, their spills added 110 MB to the
+// DRAM traffic of a half-dslash on 32^3 x 64, and 9 us).  It settles all but fields with components far smaller than others that the
+// links hardly mix with them.
+__device__ __noinline__ bool fx_careful(const HA& A, const FxField& f, const int4* links, const int* nb, int q, int E, int cb,
+                                        int sp, int64_t (&out)[12]) {
+  FxSum S;
+  FxMagnitudes M = {};
+  fx_clear(S);
+  fx_walk(sp, A.dagger ? -1 : 1, S, [&](auto i, int m) {
+    constexpr int I = decltype(i)::value;
+    if constexpr (I == 4) {  // the lower spins have changed lanes
+#pragma unroll
+      for (int k = 0; k < 6; ++k) M.t[k] = __shfl_xor_sync(0xffffffffu, M.t[k], kSB);
+      M.nt = __shfl_xor_sync(0xffffffffu, M.nt, kSB);
+    }
+    fx_careful_hop<I>(nb, f, links, E, sp, m, S, M);
+  });
+  const float least = sum_min(M.size);
+  bool bad = E == kBad;
+#pragma unroll
+  for (int k = 0; k < 6; ++k)
+    bad = bad || (M.s[k] < least && (M.nz >> k & 1)) || (M.t[k] < least && (M.nt >> k & 1));
+  const unsigned all = __ballot_sync(0xffffffffu, bad), site = (all | all >> kSB) & 0xffffu;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    out[k] = S.up[k];
+    out[6 + k] = S.lo[k];
+  }
+  if (!site) return false;
+  bad = site >> (threadIdx.x % kSB) & 1;
+  int64_t w[12];
+  fp64_sum(A, f, q, nb, cb, sp, w);
+  if (bad)
+#pragma unroll
+    for (int k = 0; k < 12; ++k) out[k] = w[k];
+  return bad;
 }
 
 // The sums as a fixed-point field of their own (a = 1, no x term: the first half-dslash of Mhat, whose
 // result only the second one reads): both lanes of a site find its largest sum.
 __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, bool valid, int E, bool minus_lo, bool nan,
-                                         bool slow, int64_t (&up)[6], int64_t (&lo)[6]) {
+                                         int64_t (&up)[6], int64_t (&lo)[6]) {
   flip(lo, minus_lo);
   uint64_t mx = 0;
 #pragma unroll
@@ -502,12 +539,12 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
     mx |= (uint64_t)(lo[k] ^ (lo[k] >> 63));
   }
   mx |= __shfl_xor_sync(0xffffffffu, mx, kSB);
-  if (!valid || slow) return;  // slow: fx_store_fp64
+  if (!valid) return;
   const int b = 64 - __clzll((long long)mx);  // -2^b <= every sum < 2^b
   const int e = mx ? b + E - 57 : kZero, shift = b - 30;
   int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
   const bool wide = nan || (mx && (e < kEmin || e > kEmax));
-  const double unit = nan ? __longlong_as_double(0x7ff8000000000000ll) : __hiloint2double((E - 56) << 20, 0);
+  const double unit = nan ? fx_nan() : fx_unit(E);
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
     const int c = k % 3;
@@ -525,14 +562,13 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
   if (sp == 0) out.e[cb] = wide ? kBad : e;
 }
 
-// a slow site's sums as a kBad site of that field
-__device__ __forceinline__ void fx_store_fp64(const FxField& out, int cb, int sp, bool minus_lo, const Cx<double> (&v)[6]) {
+// sums of fx_careful in FP64 as a kBad site of that field
+__device__ __forceinline__ void fx_store_fp64(const FxField& out, int cb, int sp, bool minus_lo, const int64_t (&v)[12]) {
   int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    const Cx<double> x = k >= 3 && minus_lo ? -v[k] : v[k];
-    o[(k < 3 ? k : 3 + k) * kSB] =
-        make_int4(__double2loint(x.re), __double2hiint(x.re), __double2loint(x.im), __double2hiint(x.im));
+    const int64_t sign = k >= 3 && minus_lo ? (int64_t)1 << 63 : 0, x = v[2 * k] ^ sign, y = v[2 * k + 1] ^ sign;
+    o[(k < 3 ? k : 3 + k) * kSB] = make_int4((int)x, (int)(x >> 32), (int)y, (int)(y >> 32));
   }
   if (sp == 0) out.e[cb] = kBad;
 }
@@ -564,21 +600,22 @@ __device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField&
   const int cb = L.valid ? L.cb : 0;
   const int E = fx_neighbours(A, W, f, cb);
   FxSum S;
-  bool slow;
-  const double unit = fx_sum(A, W, f, E, L.sp, S, slow);
-  if (__any_sync(0xffffffffu, slow)) {  // the warp's sites together: nothing of theirs has to be kept meanwhile
-    Cx<double> w[6];  // in memory, for the call: v stays in registers
-    fp64_sum(A, f, L.q, &W.sm->nb[0][W.warp * kSB + W.lane % kSB], cb, L.sp, w);
-    a[0] = A.a;
-#pragma unroll
-    for (int k = 0; k < 6; ++k) v[k] = w[k];
-  } else {
-    a[0] = A.a * unit;
+  a[0] = A.a * fx_unit(E);
+  if (!fx_sum(A, W, f, E, L.sp, S)) {
+    if (W.failed) a[0] = fx_nan();  // a copy that never arrived
 #pragma unroll
     for (int c = 0; c < 3; ++c) {
       v[c] = {(double)S.up[2 * c], (double)S.up[2 * c + 1]};
       v[3 + c] = {(double)S.lo[2 * c], (double)S.lo[2 * c + 1]};
     }
+  } else {
+    int64_t w[12];
+    const bool fp64 = fx_careful(A, f, W.links + W.lane % kSB, &W.sm->nb[0][W.warp * kSB + W.lane % kSB], L.q, E, cb, L.sp, w);
+    if (fp64) a[0] = A.a;
+#pragma unroll
+    for (int k = 0; k < 6; ++k)
+      v[k] = {fp64 ? __longlong_as_double(w[2 * k]) : (double)w[2 * k],
+              fp64 ? __longlong_as_double(w[2 * k + 1]) : (double)w[2 * k + 1]};
   }
   a[1] = A.dagger ? -a[0] : a[0];
 }
@@ -604,14 +641,20 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_const
     const int cb = L.valid ? L.cb : 0;
     const int E = fx_neighbours(A, W, f, cb);
     FxSum S;
-    bool slow;
-    fx_sum(A, W, f, E, L.sp, S, slow);
     const FxField o = fx_slice(O, L.q);
-    fx_store(o, L.cb, L.sp, L.valid, E, A.dagger != 0, W.failed, slow, S.up, S.lo);
-    if (__any_sync(0xffffffffu, slow)) {
-      Cx<double> v[6];
-      fp64_sum(A, f, L.q, &sm.nb[0][W.warp * kSB + W.lane % kSB], cb, L.sp, v);
-      if (slow && L.valid) fx_store_fp64(o, L.cb, L.sp, A.dagger != 0, v);
+    if (!fx_sum(A, W, f, E, L.sp, S)) {
+      fx_store(o, L.cb, L.sp, L.valid, E, A.dagger != 0, W.failed, S.up, S.lo);
+    } else {
+      int64_t w[12];
+      const bool fp64 = fx_careful(A, f, W.links + W.lane % kSB, &sm.nb[0][W.warp * kSB + W.lane % kSB], L.q, E, cb, L.sp, w);
+      int64_t up[6], lo[6];
+#pragma unroll
+      for (int k = 0; k < 6; ++k) {
+        up[k] = w[k];
+        lo[k] = w[6 + k];
+      }
+      fx_store(o, L.cb, L.sp, L.valid && !fp64, E, A.dagger != 0, false, up, lo);
+      if (fp64 && L.valid) fx_store_fp64(o, L.cb, L.sp, A.dagger != 0, w);
     }
     return;
   }
@@ -689,7 +732,7 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx_red(const __grid_c
 // 4.6, and 14 launches and 3 synchronisations became 6 and 1.  Measured: 24^3 x 48 with FP16 inner vectors (6
 // steps) 16.2 -> 14.6 ms, 8^3 x 16 2.77 -> 2.25 ms, 12 right-hand sides 156 -> 150 ms, 32^3 x 64 51.3 -> 49.5 ms.
 
-// two sums of the block (all its warps one slice) into partial[(q * nsb + block) * 4 + k0 ..]
+// a sum over the block (all its warps one slice) into partial[row * 4 + k]
 __device__ __forceinline__ void block_partial(double v0, double* partial, long row, int k) {
   double v[1] = {v0};
   block_sum<1>(v);
@@ -997,9 +1040,9 @@ void launch_fx(FxLaunch* L) {
     launch_k(k_hop_fx<MINB, 0>, sblocks * (unsigned)A.ntiles, block, smem, L->st, A, L->links, L->F, L->O);
 }
 
-// cfg.tile: blocks per SM that the registers are bounded for (5: 96 registers, 20 warps; 4: 128, 16 warps;
-// within 2% of each other where HBM bounds them, 4 is 10% faster on a few hundred sites.  6 and 7 spill: 0.345
-// and 0.376 ms against 0.315 at 32^3 x 64)
+// cfg.tile: blocks per SM that the registers are bounded for (5: 96 registers, 20 warps, 28 to 68 bytes of spill
+// stores; 4: 128, 16 warps, 20 to 76 bytes; within 2% of each other where HBM bounds them, 4 is 10% faster on a few
+// hundred sites.  6 and 7 took 0.345 and 0.376 ms against 0.315 at 32^3 x 64, before the sums of magnitudes)
 void run_fx(void* ctx, const LaunchCfg& cfg) {
   auto* L = (FxLaunch*)ctx;
   if (cfg.tile == 4)
