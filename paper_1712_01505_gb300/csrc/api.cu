@@ -157,9 +157,9 @@ void* Workspace::get(const std::string& name, size_t bytes) {
   return p;
 }
 
-bool Workspace::has(const std::string& name, size_t bytes) const {
+void* Workspace::find(const std::string& name, size_t bytes) const {
   auto it = bufs.find(name);
-  return it != bufs.end() && it->second.bytes >= bytes;
+  return it != bufs.end() && it->second.bytes >= bytes ? it->second.p : nullptr;
 }
 
 bool Workspace::drop_optional() {

@@ -111,7 +111,7 @@ struct Workspace {
   Workspace(const Workspace&) = delete;
   Workspace& operator=(const Workspace&) = delete;
   void* get(const std::string& name, size_t bytes);
-  bool has(const std::string& name, size_t bytes) const;  // get() would return it as it is
+  void* find(const std::string& name, size_t bytes) const;  // what get() would return as it is, or null
   bool drop_optional();
   void release();
 };

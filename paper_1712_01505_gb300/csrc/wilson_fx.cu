@@ -1070,8 +1070,11 @@ bool capturing(cudaStream_t st) {
 FxField fx_scratch(qcd_gauge* g, const char* name, const Field& like, cudaStream_t st) {
   const long nsb = (like.Vh + kSB - 1) / kSB, nq = (long)like.ls * like.nrhs;
   const size_t data = (size_t)nq * nsb * kSiteUnits * sizeof(int4), exps = (size_t)nq * nsb * kSB * sizeof(int);
-  if (!g->ws.has(name, data + exps) && capturing(st)) raise(QCD_ERR_OOM, "no scratch for the fixed-point stencil");
-  char* p = (char*)g->ws.get(name, data + exps);
+  char* p = (char*)g->ws.find(name, data + exps);
+  if (!p) {
+    if (capturing(st)) raise(QCD_ERR_OOM, "no scratch for the fixed-point stencil");
+    p = (char*)g->ws.get(name, data + exps);
+  }
   return {(int4*)p, (int*)(p + data), nsb};
 }
 
