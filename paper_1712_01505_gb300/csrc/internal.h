@@ -151,7 +151,7 @@ struct qcd_gauge {
   struct FxSet {
     bool owned = false, used = false;
     bool on_work = false;           // the last use was on `work`, the event not recorded
-    cudaStream_t owner = nullptr;   // a name only: the stream may be gone, or another by now
+    unsigned long long owner = 0;   // the stream's id: never given to another one, unlike its address
     cudaEvent_t done = nullptr;
   };
   static constexpr int kFxSets = 4;

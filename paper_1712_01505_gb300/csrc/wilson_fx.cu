@@ -214,52 +214,11 @@ struct FxSum {
   unsigned su[3], sl[3];
 };
 
-// The products of a hop, added to S; link(k): element k of its matrix.  Packed FP32 lanes: (re, im).
-template <int HOP, typename LINK>
-__device__ __forceinline__ void fx_products(LINK link, int d3, const int (&hr)[3], const int (&hi)[3], const float2 (&y)[3],
-                                            FxSum& S) {
-  constexpr int MU = HOP >> 1;
-  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
-  const float sc = __int_as_float((127 - d3) << 23);
-#pragma unroll
-  for (int a = 0; a < 3; ++a) {
-    int64_t Hr = hop_half(d3, HOP & 1), Hi = Hr;
-    float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
-#pragma unroll
-    for (int b = 0; b < 3; ++b) {
-      const int4 u = link(a * 3 + b);
-      const float2 g = make_float2((float)hr[b], (float)hi[b]);  // the integer parts as FP32
-      Hr += (int64_t)u.x * hr[b];
-      Hr += (int64_t)u.z * -hi[b];
-      Hi += (int64_t)u.x * hi[b];
-      Hi += (int64_t)u.z * hr[b];
-      C = fma2(bc2((float)u.x), y[b], C);
-      C = fma2(bc2(__int_as_float(u.y)), g, C);
-      D = fma2(bc2((float)u.z), swp(y[b]), D);
-      D = fma2(bc2(__int_as_float(u.w)), swp(g), D);
-    }
-    const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
-    const unsigned size = __byte_perm(abs((int)(wr >> 32)), abs((int)(wi >> 32)), 0x7632);
-    S.up[2 * a] += wr;
-    S.up[2 * a + 1] += wi;
-    S.su[a] += size;
-    if (MU == 0 || MU == 2) {  // SG i w
-      S.lo[2 * a] -= SG * wi;
-      S.lo[2 * a + 1] += SG * wr;
-      S.sl[a] += __byte_perm(size, size, 0x1032);
-    } else {
-      S.lo[2 * a] += SG * wr;
-      S.lo[2 * a + 1] += SG * wi;
-      S.sl[a] += size;
-    }
-  }
-}
-
-// Hop number I (of fx_order) added to S.  m: the sign of the lower input spin.
+// Hop number I (of fx_order) added to S.  m: the sign of the lower input spin.  Packed FP32 lanes: (re, im).
 template <int I>
 __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int sp, int m, FxSum& S) {
   constexpr int HOP = fx_order(I), MU = HOP >> 1;
-  constexpr int SG = (HOP & 1) ? 1 : -1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
   const int nbw = W.sm->nb[HOP][W.warp * kSB + W.lane % kSB];
   const int d3 = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100) + 3;
   int hr[3], hi[3];
@@ -267,8 +226,40 @@ __device__ __forceinline__ void fx_hop(FxWarp& W, const FxField& f, int E, int s
   fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
   if (!mbar_wait(&W.sm->bar[W.warp][I % kBuf], (unsigned)(I / kBuf) & 1u)) W.failed = true;
   if (d3 < kFar) {
+    const float sc = __int_as_float((127 - d3) << 23);
     const int4* w = &W.sm->w[W.warp][I % kBuf][W.lane % kSB];
-    fx_products<HOP>([&](int k) { return w[k * kSB]; }, d3, hr, hi, y, S);
+#pragma unroll
+    for (int a = 0; a < 3; ++a) {
+      int64_t Hr = hop_half(d3, HOP & 1), Hi = Hr;
+      float2 C = make_float2(0.f, 0.f), D = C;  // (re, im) = (C.x - D.x, C.y + D.y)
+#pragma unroll
+      for (int b = 0; b < 3; ++b) {
+        const int4 u = w[(a * 3 + b) * kSB];
+        const float2 g = make_float2((float)hr[b], (float)hi[b]);  // the integer parts as FP32
+        Hr += (int64_t)u.x * hr[b];
+        Hr += (int64_t)u.z * -hi[b];
+        Hi += (int64_t)u.x * hi[b];
+        Hi += (int64_t)u.z * hr[b];
+        C = fma2(bc2((float)u.x), y[b], C);
+        C = fma2(bc2(__int_as_float(u.y)), g, C);
+        D = fma2(bc2((float)u.z), swp(y[b]), D);
+        D = fma2(bc2(__int_as_float(u.w)), swp(g), D);
+      }
+      const int64_t wr = hop_round(Hr, C.x - D.x, sc, d3), wi = hop_round(Hi, C.y + D.y, sc, d3);
+      const unsigned size = __byte_perm(abs((int)(wr >> 32)), abs((int)(wi >> 32)), 0x7632);
+      S.up[2 * a] += wr;
+      S.up[2 * a + 1] += wi;
+      S.su[a] += size;
+      if (MU == 0 || MU == 2) {  // SG i w
+        S.lo[2 * a] -= SG * wi;
+        S.lo[2 * a + 1] += SG * wr;
+        S.sl[a] += __byte_perm(size, size, 0x1032);
+      } else {
+        S.lo[2 * a] += SG * wr;
+        S.lo[2 * a + 1] += SG * wi;
+        S.sl[a] += size;
+      }
+    }
   }
   __syncwarp();  // every lane has read the buffer
   if (I + kBuf < 8) W.issue(fx_order(I + kBuf < 8 ? I + kBuf : 0), I % kBuf);
@@ -281,21 +272,17 @@ struct FxMagnitudes {
   unsigned nz, nt;
 };
 
-// Hop number I and its magnitudes.  links: of the lane's site.
+// Those of hop number I.  links: of the lane's site.
 template <int I>
-__device__ __forceinline__ void fx_careful_hop(const int* nb, const FxField& f, const int4* links, int E, int sp, int m,
-                                               FxSum& S, FxMagnitudes& M) {
+__device__ __forceinline__ void fx_magnitudes(const int* nb, const FxField& f, const int4* links, int E, int sp, int m,
+                                              FxMagnitudes& M) {
   constexpr int HOP = fx_order(I), MU = HOP >> 1;
-  constexpr int SG = (HOP & 1) ? 1 : -1;
+  constexpr int SG = (HOP & 1) ? 1 : -1;  // (1 - gamma) forward, (1 + gamma) backward
   const int nbw = nb[HOP * (kWarps * kSB)];
   const int d = min(E - __ldg(f.e + (nbw & 0x7fffffff)), 100);
   int hr[3], hi[3];
   float2 y[3];
   fx_half<MU>(f, nbw, sp, m * SG, hr, hi, y);
-  int4 u[9];
-#pragma unroll
-  for (int k = 0; k < 9; ++k) u[k] = __ldg(links + HOP * kHopUnits + k * kSB);
-  if (d + 3 < kFar) fx_products<HOP>([&](int k) { return u[k]; }, d + 3, hr, hi, y, S);
   const float sc = __int_as_float((127 - d) << 23);
   M.size += sc;
 #pragma unroll
@@ -304,8 +291,8 @@ __device__ __forceinline__ void fx_careful_hop(const int* nb, const FxField& f, 
     unsigned br = 0, bi = 0;
 #pragma unroll
     for (int b = 0; b < 3; ++b) {
-      const int4 v = u[a * 3 + b];
-      const float ur = fabsf((float)v.x + __int_as_float(v.y)), ui = fabsf((float)v.z + __int_as_float(v.w));
+      const int4 u = __ldg(links + HOP * kHopUnits + (a * 3 + b) * kSB);
+      const float ur = fabsf((float)u.x + __int_as_float(u.y)), ui = fabsf((float)u.z + __int_as_float(u.w));
       const float xr = fabsf((float)hr[b] + y[b].x), xi = fabsf((float)hi[b] + y[b].y);
       mr = fmaf(ur, xr, fmaf(ui, xi, mr));
       mi = fmaf(ur, xi, fmaf(ui, xr, mi));
@@ -376,11 +363,11 @@ __device__ __forceinline__ void fp64_hop(const HA& A, const FxField& f, const do
 }
 
 // The hop sums of the lane (upper spin sp, lower spin 2 + sp, the latter times -1 for H^dag) in FP64; the whole warp calls
-// it, since a site's two lanes share the work; as bits of FP64 numbers.  Bound by the FP64 pipe.  The full matrix on
+// it, since a site's two lanes share the work; with keep into the lane's slots, as bits.  Bound by the FP64 pipe.  The full matrix on
 // 24^3 x 32 where every site comes here (a point source's solution, links within 1e-4 of 1): 1.34 ms with the two walks
 // before; the FP64 kernel, 0.82.
-__device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, const int* nb, int cb, int sp,
-                                      int64_t (&out)[12]) {
+__device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, const int* nb, int cb, int sp, bool keep,
+                                      int64_t* slots) {
   const double2* src = A.in.p;
   if (src) {
     const int r = fdiv(q, A.d_ls);
@@ -408,10 +395,11 @@ __device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, cons
   turn(sp != 0);
   fp64_hop<6>(A, f, src, nb, cb, sp, g5, v);
   fp64_hop<7>(A, f, src, nb, cb, sp, g5, v);
+  if (!keep) return;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    out[2 * k] = __double_as_longlong(v[k].re);
-    out[2 * k + 1] = __double_as_longlong(v[k].im);
+    slots[2 * k * 32] = __double_as_longlong(v[k].re);
+    slots[(2 * k + 1) * 32] = __double_as_longlong(v[k].im);
   }
 }
 
@@ -438,93 +426,94 @@ __device__ __forceinline__ void flip(int64_t (&v)[6], bool minus) {
   for (int k = 0; k < 6; ++k) v[k] = (v[k] ^ n) - n;
 }
 
-// the hops of both walks, in order: H(number, sign of the lower input spin); the lower spins' signs and lanes between them
-template <typename H>
-__device__ __forceinline__ void fx_walk(int sp, int g5, FxSum& S, H hop) {
-  const int gs = sp ? -g5 : g5;
-  hop(std::integral_constant<int, 0>{}, -gs);  // y: B = (-l1, l0)
-  hop(std::integral_constant<int, 1>{}, -gs);
-  flip(S.lo, sp == 0);                         // B^dag = (g1, -g0)
-  hop(std::integral_constant<int, 2>{}, g5);   // x: B = -i (l1, l0)
-  hop(std::integral_constant<int, 3>{}, g5);
+__device__ __forceinline__ double fx_unit(int E) { return __hiloint2double((E - 56) << 20, 0); }  // 2^(E - 1079)
+__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
+
+// S.up, S.lo = the sum of the eight hops for spins sp and 2 + sp, in units of 2^(E - 1079) (lo: times -1 for
+// H^dag = g5 H g5); the whole warp calls it.  true (for the whole warp): the sums do not show that they are exact
+// enough, or a neighbour is kept in FP64, and fx_careful decides.
+//
+// The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
+// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Without it a half-dslash on 32^3 x 64 took 352 us instead of 365,
+// the full matrix on 24^3 x 48 309 instead of 316, and a solve on 12x10x14x18 3.53 ms instead of 3.8.
+__device__ __forceinline__ bool fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S) {
+  const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) S.up[k] = S.lo[k] = 0;
+#pragma unroll
+  for (int k = 0; k < 3; ++k) S.su[k] = S.sl[k] = 0;
+  fx_hop<0>(W, f, E, sp, -gs, S);  // y: B = (-l1, l0)
+  fx_hop<1>(W, f, E, sp, -gs, S);
+  flip(S.lo, sp == 0);             // B^dag = (g1, -g0)
+  fx_hop<2>(W, f, E, sp, g5, S);   // x: B = -i (l1, l0)
+  fx_hop<3>(W, f, E, sp, g5, S);
 #pragma unroll
   for (int k = 0; k < 6; ++k) S.lo[k] = __shfl_xor_sync(0xffffffffu, S.lo[k], kSB);
 #pragma unroll
   for (int k = 0; k < 3; ++k) S.sl[k] = __shfl_xor_sync(0xffffffffu, S.sl[k], kSB);
   flip(S.lo, sp != 0);
-  hop(std::integral_constant<int, 4>{}, gs);   // z: B = (-i l0, i l1)
-  hop(std::integral_constant<int, 5>{}, gs);
+  fx_hop<4>(W, f, E, sp, gs, S);   // z: B = (-i l0, i l1)
+  fx_hop<5>(W, f, E, sp, gs, S);
   flip(S.lo, sp != 0);
-  hop(std::integral_constant<int, 6>{}, g5);   // t: B = 1
-  hop(std::integral_constant<int, 7>{}, g5);
-}
-__device__ __forceinline__ void fx_clear(FxSum& S) {
-#pragma unroll
-  for (int k = 0; k < 6; ++k) S.up[k] = S.lo[k] = 0;
-#pragma unroll
-  for (int k = 0; k < 3; ++k) S.su[k] = S.sl[k] = 0;
-}
-
-// S.up, S.lo = the sum of the eight hops for spins sp and 2 + sp, in units of 2^(E - 1079) (lo: times -1 for
-// H^dag = g5 H g5); the whole warp calls it.  true (for the whole warp): the sums do not show that they are exact
-// enough, or a neighbour is kept in FP64; fx_careful then computes the sites.
-//
-// The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
-// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Without it a half-dslash on 32^3 x 64 took 352 us instead of 365,
-// the full matrix on 24^3 x 48 309 instead of 316, a solve on 12x10x14x18 3.53 ms instead of 3.79, and twelve point sources on
-// 24^3 x 48, around which spins and colours differ most, 138 ms instead of 145.
-__device__ __forceinline__ bool fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S) {
-  fx_clear(S);
-  fx_walk(sp, A.dagger ? -1 : 1, S,
-          [&](auto i, int m) { fx_hop<decltype(i)::value>(W, f, E, sp, m, S); });
+  fx_hop<6>(W, f, E, sp, g5, S);   // t: B = 1
+  fx_hop<7>(W, f, E, sp, g5, S);
   unsigned least = 0xffffffffu;
 #pragma unroll
   for (int k = 0; k < 3; ++k) least = __vminu2(least, __vminu2(S.su[k], S.sl[k]));
   const bool weak = (min(least & 0xffffu, least >> 16) < 64u && E > kZero) || E == kBad;  // kZero: all neighbours are zero
   return __any_sync(0xffffffffu, weak);
 }
-__device__ __forceinline__ double fx_unit(int E) { return __hiloint2double((E - 56) << 20, 0); }  // 2^(E - 1079)
-__device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff8000000000000ll); }
 
-// The same sums once more with the magnitudes of their products, in out (up, then lo); of a site with a neighbour that
-// is kept in FP64, or with a component that is neither as exact as FP64 would have it (fixed.cuh) nor without a
-// product that is not zero, as FP64 numbers: true, for both lanes of the site.  A walk of its own, so that the
-// kernels' registers hold nothing meanwhile (with the first walk's sums kept, their spills added 110 MB to the
-// DRAM traffic of a half-dslash on 32^3 x 64, and 9 us).  It settles all but fields with components far smaller than others that the
-// links hardly mix with them.
-__device__ __noinline__ bool fx_careful(const HA& A, const FxField& f, const int4* links, const int* nb, int q, int E, int cb,
-                                        int sp, int64_t (&out)[12]) {
-  FxSum S;
+// What fx_sum left open: the magnitudes of the products are formed, and a site with a neighbour that is kept in
+// FP64, or with a component that is neither as exact as FP64 would have it (fixed.cuh) nor without a product that is not
+// zero, is computed in FP64: true, for both lanes of the site, and the sums in the lane's slots are FP64
+// numbers.  It settles all but fields with components far smaller than others that the links hardly mix with them.
+__device__ __noinline__ bool fx_decide(const HA& A, const FxField& f, const int4* links, const int* nb, int q, int E, int cb,
+                                       int sp, int64_t* slots) {
+  const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
   FxMagnitudes M = {};
-  fx_clear(S);
-  fx_walk(sp, A.dagger ? -1 : 1, S, [&](auto i, int m) {
-    constexpr int I = decltype(i)::value;
-    if constexpr (I == 4) {  // the lower spins have changed lanes
+  fx_magnitudes<0>(nb, f, links, E, sp, -gs, M);  // signs and lanes as in fx_sum
+  fx_magnitudes<1>(nb, f, links, E, sp, -gs, M);
+  fx_magnitudes<2>(nb, f, links, E, sp, g5, M);
+  fx_magnitudes<3>(nb, f, links, E, sp, g5, M);
 #pragma unroll
-      for (int k = 0; k < 6; ++k) M.t[k] = __shfl_xor_sync(0xffffffffu, M.t[k], kSB);
-      M.nt = __shfl_xor_sync(0xffffffffu, M.nt, kSB);
-    }
-    fx_careful_hop<I>(nb, f, links, E, sp, m, S, M);
-  });
+  for (int k = 0; k < 6; ++k) M.t[k] = __shfl_xor_sync(0xffffffffu, M.t[k], kSB);
+  M.nt = __shfl_xor_sync(0xffffffffu, M.nt, kSB);
+  fx_magnitudes<4>(nb, f, links, E, sp, gs, M);
+  fx_magnitudes<5>(nb, f, links, E, sp, gs, M);
+  fx_magnitudes<6>(nb, f, links, E, sp, g5, M);
+  fx_magnitudes<7>(nb, f, links, E, sp, g5, M);
   const float least = sum_min(M.size);
   bool bad = E == kBad;
 #pragma unroll
   for (int k = 0; k < 6; ++k)
     bad = bad || (M.s[k] < least && (M.nz >> k & 1)) || (M.t[k] < least && (M.nt >> k & 1));
   const unsigned all = __ballot_sync(0xffffffffu, bad), site = (all | all >> kSB) & 0xffffu;
-#pragma unroll
-  for (int k = 0; k < 6; ++k) {
-    out[k] = S.up[k];
-    out[6 + k] = S.lo[k];
-  }
   if (!site) return false;
   bad = site >> (threadIdx.x % kSB) & 1;
-  int64_t w[12];
-  fp64_sum(A, f, q, nb, cb, sp, w);
-  if (bad)
-#pragma unroll
-    for (int k = 0; k < 12; ++k) out[k] = w[k];
+  fp64_sum(A, f, q, nb, cb, sp, bad, slots);
   return bad;
+}
+
+// The sums of fx_sum go through the warp's link buffers, which are free now, so that the kernels' registers hold nothing
+// across the calls (with the sums kept in them their spills added 110 MB to the DRAM traffic of a half-dslash on
+// 32^3 x 64, and 9 us; with the sums formed again it took twice as long where it is called for every site).
+__device__ __forceinline__ bool fx_careful(const HA& A, FxWarp& W, const FxField& f, int q, int E, int cb, int sp, FxSum& S) {
+  static_assert(sizeof(W.sm->w[0]) >= 32 * 12 * sizeof(int64_t), "a warp's sums fit its link buffers");
+  int64_t* slots = reinterpret_cast<int64_t*>(&W.sm->w[W.warp][0][0]) + W.lane;
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    slots[k * 32] = S.up[k];
+    slots[(6 + k) * 32] = S.lo[k];
+  }
+  const bool fp64 = fx_decide(A, f, W.links + W.lane % kSB, &W.sm->nb[0][W.warp * kSB + W.lane % kSB], q, E, cb, sp, slots);
+#pragma unroll
+  for (int k = 0; k < 6; ++k) {
+    S.up[k] = slots[k * 32];
+    S.lo[k] = slots[(6 + k) * 32];
+  }
+  __syncwarp();
+  return fp64;
 }
 
 // The sums as a fixed-point field of their own (a = 1, no x term: the first half-dslash of Mhat, whose
@@ -562,12 +551,13 @@ __device__ __forceinline__ void fx_store(const FxField& out, int cb, int sp, boo
   if (sp == 0) out.e[cb] = wide ? kBad : e;
 }
 
-// sums of fx_careful in FP64 as a kBad site of that field
-__device__ __forceinline__ void fx_store_fp64(const FxField& out, int cb, int sp, bool minus_lo, const int64_t (&v)[12]) {
+// FP64 sums of fx_careful as a kBad site of that field
+__device__ __forceinline__ void fx_store_fp64(const FxField& out, int cb, int sp, bool minus_lo, const FxSum& S) {
   int4* o = out.p + (long)(cb / kSB) * kSiteUnits + sp * (3 * kSB) + cb % kSB;
 #pragma unroll
   for (int k = 0; k < 6; ++k) {
-    const int64_t sign = k >= 3 && minus_lo ? (int64_t)1 << 63 : 0, x = v[2 * k] ^ sign, y = v[2 * k + 1] ^ sign;
+    const int64_t sign = k >= 3 && minus_lo ? INT64_MIN : 0;
+    const int64_t x = k < 3 ? S.up[2 * k] : S.lo[2 * k - 6] ^ sign, y = k < 3 ? S.up[2 * k + 1] : S.lo[2 * k - 5] ^ sign;
     o[(k < 3 ? k : 3 + k) * kSB] = make_int4((int)x, (int)(x >> 32), (int)y, (int)(y >> 32));
   }
   if (sp == 0) out.e[cb] = kBad;
@@ -601,21 +591,16 @@ __device__ __forceinline__ void fx_values(const HA& A, FxWarp& W, const FxField&
   const int E = fx_neighbours(A, W, f, cb);
   FxSum S;
   a[0] = A.a * fx_unit(E);
-  if (!fx_sum(A, W, f, E, L.sp, S)) {
-    if (W.failed) a[0] = fx_nan();  // a copy that never arrived
-#pragma unroll
-    for (int c = 0; c < 3; ++c) {
-      v[c] = {(double)S.up[2 * c], (double)S.up[2 * c + 1]};
-      v[3 + c] = {(double)S.lo[2 * c], (double)S.lo[2 * c + 1]};
-    }
-  } else {
-    int64_t w[12];
-    const bool fp64 = fx_careful(A, f, W.links + W.lane % kSB, &W.sm->nb[0][W.warp * kSB + W.lane % kSB], L.q, E, cb, L.sp, w);
+  bool fp64 = false;
+  if (fx_sum(A, W, f, E, L.sp, S)) {
+    fp64 = fx_careful(A, W, f, L.q, E, cb, L.sp, S);
     if (fp64) a[0] = A.a;
+  }
+  if (W.failed) a[0] = fx_nan();  // a copy that never arrived
 #pragma unroll
-    for (int k = 0; k < 6; ++k)
-      v[k] = {fp64 ? __longlong_as_double(w[2 * k]) : (double)w[2 * k],
-              fp64 ? __longlong_as_double(w[2 * k + 1]) : (double)w[2 * k + 1]};
+  for (int k = 0; k < 6; ++k) {
+    const int64_t re = k < 3 ? S.up[2 * k] : S.lo[2 * k - 6], im = k < 3 ? S.up[2 * k + 1] : S.lo[2 * k - 5];
+    v[k] = {fp64 ? __longlong_as_double(re) : (double)re, fp64 ? __longlong_as_double(im) : (double)im};
   }
   a[1] = A.dagger ? -a[0] : a[0];
 }
@@ -642,20 +627,12 @@ __global__ void __launch_bounds__(32 * kWarps, MINB) k_hop_fx(const __grid_const
     const int E = fx_neighbours(A, W, f, cb);
     FxSum S;
     const FxField o = fx_slice(O, L.q);
-    if (!fx_sum(A, W, f, E, L.sp, S)) {
-      fx_store(o, L.cb, L.sp, L.valid, E, A.dagger != 0, W.failed, S.up, S.lo);
-    } else {
-      int64_t w[12];
-      const bool fp64 = fx_careful(A, f, W.links + W.lane % kSB, &sm.nb[0][W.warp * kSB + W.lane % kSB], L.q, E, cb, L.sp, w);
-      int64_t up[6], lo[6];
-#pragma unroll
-      for (int k = 0; k < 6; ++k) {
-        up[k] = w[k];
-        lo[k] = w[6 + k];
-      }
-      fx_store(o, L.cb, L.sp, L.valid && !fp64, E, A.dagger != 0, false, up, lo);
-      if (fp64 && L.valid) fx_store_fp64(o, L.cb, L.sp, A.dagger != 0, w);
+    bool fp64 = false;
+    if (fx_sum(A, W, f, E, L.sp, S)) {
+      fp64 = fx_careful(A, W, f, L.q, E, cb, L.sp, S);
+      if (fp64 && L.valid) fx_store_fp64(o, L.cb, L.sp, A.dagger != 0, S);
     }
+    fx_store(o, L.cb, L.sp, L.valid && !fp64, E, A.dagger != 0, W.failed, S.up, S.lo);
     return;
   }
   Cx<double> v[6];
@@ -1145,15 +1122,15 @@ void fx_launch(const qcd_gauge* gh, const FxField& in, const SpinorView<P64>* sr
 }
 
 // The scratch fields belong to the handle, and calls on device buffers are asynchronous on the caller's
-// stream.  A stream has a set of its own while there are sets (kFxSets), and always waits for the event of the set's last
-// use: a stream's address says nothing about which stream that was (it may have been destroyed with the work
-// pending and another one created there, and cudaStreamPerThread is one address for every thread's).  Only the solver's
-// own stream is known; its use is recorded when another stream follows.
+// stream.  A stream has a set of its own while there are sets (kFxSets); another stream that takes it over waits for the
+// event of its last use.  Streams are told apart by their ids: the address may be that of a stream that was destroyed
+// with its work pending, or cudaStreamPerThread, one address for every thread's (which always waits).  The solver's
+// own use is recorded when another stream follows.
 class FxOrder {
  public:
-  FxOrder(qcd_gauge* g, cudaStream_t st) : g_(g), st_(st), set_(g->fx_set[pick(g, st)]) {
+  FxOrder(qcd_gauge* g, cudaStream_t st) : g_(g), st_(st), set_(g->fx_set[pick(g, st, &same_)]) {
     if (!set_.done) QCD_CK(cudaEventCreateWithFlags(&set_.done, cudaEventDisableTiming));
-    if (!set_.used || (set_.on_work && st == g->work)) return;
+    if (!set_.used || (set_.on_work ? st == g->work : same_)) return;
     if (set_.on_work) QCD_CK(cudaEventRecord(set_.done, g->work));
     QCD_CK(cudaStreamWaitEvent(st, set_.done, 0));
   }
@@ -1171,20 +1148,26 @@ class FxOrder {
   }
 
  private:
-  static int pick(qcd_gauge* g, cudaStream_t st) {
+  // *same: the set's last use, if not by the solver, was on this very stream
+  static int pick(qcd_gauge* g, cudaStream_t st, bool* same) {
+    *same = false;
     if (st == g->work) return 0;
+    unsigned long long id = 0;
+    QCD_CK(cudaStreamGetId(st, &id));
     for (int k = 0; k < qcd_gauge::kFxSets; ++k)
-      if (!g->fx_set[k].owned || g->fx_set[k].owner == st) {
+      if (!g->fx_set[k].owned || g->fx_set[k].owner == id) {
+        *same = g->fx_set[k].owned && st != cudaStreamPerThread;
         g->fx_set[k].owned = true;
-        g->fx_set[k].owner = st;
+        g->fx_set[k].owner = id;
         return k;
       }
     const int k = g->fx_next++ % qcd_gauge::kFxSets;
-    g->fx_set[k].owner = st;
+    g->fx_set[k].owner = id;
     return k;
   }
   qcd_gauge* g_;
   cudaStream_t st_;
+  bool same_ = false;
   qcd_gauge::FxSet& set_;
 };
 
