@@ -1227,7 +1227,7 @@ void hop(const qcd_gauge* g, const Field& in, Field& out, int out_parity, int da
       hop_df(g, in, out, out_parity, dagger, a, x, nullptr, 0.0, st, stop, allow_tuning);
       break;
     case QCD_F64:
-      // in fixed point (32^3 x 64: 0.37 ms with its input conversion against 1.56; 6 x 4 x 6 x 10: 10 us against
+      // in fixed point (32^3 x 64: 0.37 ms with its input conversion against 1.56; 6 x 4 x 6 x 10: 11 us against
       // 31) unless the call may not use the handle's scratch or the links are not of unit size
       if (!allow_tuning || !hop_fx(g, in, out, out_parity, dagger, a, x, st, stop, red))
         hop_impl<P64, 18>(g, g->U64, in, out, out_parity, dagger, a, x, st, stop, allow_tuning, red);

@@ -8,8 +8,8 @@
 // are kept that way from the loading of the gauge field, and only the final sum goes through the
 // FP64 pipe: 24 conversions and 24 multiply-adds per site instead of 864.  Sites whose components the parts do not
 // hold as well as FP64 would are computed in FP64 (fx_sum, fx_careful).  Measured at 32^3 x 64:
-// FP64 kernel 1.56 ms (FP64 pipe), here 0.31 ms, 5.3 TB/s = 79% of the copy rate (links 1152 B, input 196 B, x and output
-// 192 B each per site; HBM and issue slots), and 0.056 ms for k_to_fx (HBM); 16^3 x 32 x 16 slices 1.56 -> 0.35 ms with
+// FP64 kernel 1.56 ms (FP64 pipe), here 0.318 ms, 5.3 TB/s = 78% of the copy rate (links 1152 B, input 196 B, x and output
+// 192 B each per site; HBM and issue slots), and 0.056 ms for k_to_fx (HBM); 16^3 x 32 x 16 slices 1.56 -> 0.36 ms with
 // the conversion (issue slots).  Forms that were slower than 0.315 ms, all without the sums of magnitudes: the conversion
 // inside the stencil (8 times per site: 0.555 ms), three integer products per real one instead of one and two FP32
 // ones (0.355 ms, the integer multiply pipe), one thread per site (0.333 ms at 168 registers, 12 warps per SM).
@@ -364,7 +364,7 @@ __device__ __forceinline__ void fp64_hop(const HA& A, const FxField& f, const do
 
 // The hop sums of the lane (upper spin sp, lower spin 2 + sp, the latter times -1 for H^dag) in FP64; the whole warp calls
 // it, since a site's two lanes share the work; with keep into the lane's slots, as bits.  Bound by the FP64 pipe.  The full matrix on
-// 24^3 x 32 where every site comes here (a point source's solution, links within 1e-4 of 1): 1.34 ms with the two walks
+// 24^3 x 32 where every site comes here (a point source's solution, links within 1e-4 of 1): 1.15 ms with the two walks
 // before; the FP64 kernel, 0.82.
 __device__ __noinline__ void fp64_sum(const HA& A, const FxField& f, int q, const int* nb, int cb, int sp, bool keep,
                                       int64_t* slots) {
@@ -434,8 +434,8 @@ __device__ __forceinline__ double fx_nan() { return __longlong_as_double(0x7ff80
 // enough, or a neighbour is kept in FP64, and fx_careful decides.
 //
 // The sum of |hop| is a lower bound of the sum of magnitudes that fixed.cuh asks for, and costs 17 instructions per hop: below
-// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Without it a half-dslash on 32^3 x 64 took 352 us instead of 365,
-// the full matrix on 24^3 x 48 309 instead of 316, and a solve on 12x10x14x18 3.53 ms instead of 3.8.
+// 2^(E - 1022) / 8 in one site of 10^5 of a Gaussian field.  Without it a half-dslash on 32^3 x 64 took 351 us instead of 371,
+// a solve on 12x10x14x18 3.53 ms instead of 3.71, and twelve point sources on 24^3 x 48 139 ms instead of 144 to 147 (fx_decide).
 __device__ __forceinline__ bool fx_sum(const HA& A, FxWarp& W, const FxField& f, int E, int sp, FxSum& S) {
   const int g5 = A.dagger ? -1 : 1, gs = sp ? -g5 : g5;
 #pragma unroll
@@ -497,7 +497,8 @@ __device__ __noinline__ bool fx_decide(const HA& A, const FxField& f, const int4
 
 // The sums of fx_sum go through the warp's link buffers, which are free now, so that the kernels' registers hold nothing
 // across the calls (with the sums kept in them their spills added 110 MB to the DRAM traffic of a half-dslash on
-// 32^3 x 64, and 9 us; with the sums formed again it took twice as long where it is called for every site).
+// 32^3 x 64, and 9 us; with the sums formed again by the second walk the full matrix took 1.34 ms instead of 1.15 where
+// every site needs it).
 __device__ __forceinline__ bool fx_careful(const HA& A, FxWarp& W, const FxField& f, int q, int E, int cb, int sp, FxSum& S) {
   static_assert(sizeof(W.sm->w[0]) >= 32 * 12 * sizeof(int64_t), "a warp's sums fit its link buffers");
   int64_t* slots = reinterpret_cast<int64_t*>(&W.sm->w[W.warp][0][0]) + W.lane;
@@ -912,7 +913,7 @@ __global__ void __launch_bounds__(256) k_outer_sums(const double* __restrict__ p
 // FP64 fields without FP64 copies of their halves.  Each warp's 16 sites leave through its link buffers, so that
 // whole sites are written in runs; zero: the other site of each pair (the other parity) is zeroed with them.
 // Bound by HBM (1732 B per site and half-dslash).  The full matrix at 24^3 x 48: two packings, two conversions, two
-// stencils and two unpackings 415 us, one conversion (66 us, at the copy rate) and two of these 309 us
+// stencils and two unpackings 415 us, one conversion (66 us, at the copy rate) and two of these 307 us
 // (96 registers; 327 at 128).  Reading x through shared memory in runs after the hops was slower (368 us): the
 // lanes' own loads of 48 bytes are in flight earlier.
 __global__ void __launch_bounds__(32 * kWarps, 5) k_hop_fx_canon(const __grid_constant__ HA A,
@@ -1017,8 +1018,8 @@ void launch_fx(FxLaunch* L) {
     launch_k(k_hop_fx<MINB, 0>, sblocks * (unsigned)A.ntiles, block, smem, L->st, A, L->links, L->F, L->O);
 }
 
-// cfg.tile: blocks per SM that the registers are bounded for (5: 96 registers, 20 warps, 28 to 68 bytes of spill
-// stores; 4: 128, 16 warps, 20 to 76 bytes; within 2% of each other where HBM bounds them, 4 is 10% faster on a few
+// cfg.tile: blocks per SM that the registers are bounded for (5: 96 registers, 20 warps, 52 to 144 bytes of spill
+// stores; 4: 128, 16 warps, 40 to 68 bytes; within 2% of each other where HBM bounds them, 4 is 10% faster on a few
 // hundred sites.  6 and 7 took 0.345 and 0.376 ms against 0.315 at 32^3 x 64, before the sums of magnitudes)
 void run_fx(void* ctx, const LaunchCfg& cfg) {
   auto* L = (FxLaunch*)ctx;
